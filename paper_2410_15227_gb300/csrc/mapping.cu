@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "exact.cuh"
+#include "fp64.cuh"
 #include "quad32.cuh"
 #include "split.cuh"
 
@@ -388,23 +389,37 @@ __device__ __forceinline__ T pair_weight(T rx, T ry, T rz, T h, T radius, int64_
 // FP64 closed form, one warp per pair (both the FP64 mode and the recompute
 // of the pairs the mixed pass flagged).
 //
-// An edge's term Phi(T1) - Phi(T0) (edge_full / edge_tilde) is linear in a
-// few evaluations: the basis b(tau) at an endpoint in region 1 or 2 (a
-// combination of region coefficient vectors and b0), the region-3 part at an
-// endpoint beyond 2h (the two angles b0, b1 alone), and the region
-// differences d1 = (c1 - c2).b(t1), d2 = (c2 - c3).b(t2), whose integer
-// coefficient sums the endpoints past t1 or t2 with their signs.  So each
-// lane takes an edge, lists these evaluations with their signed weights
-// (face orientation, edge orientation and endpoint sign folded in; a d1 or
-// d2 whose coefficient vanishes, as for both endpoints beyond t2 on one
-// side, is not listed), and appends them to one of two per-warp queues, one
-// of basis evaluations and one of angle evaluations.  Whenever a queue holds
-// 32 entries the warp evaluates them together, one per lane, so that the
-// transcendental code runs with the warp converged whatever the edges'
-// regions.  Each lane adds what it evaluated; a fixed-order warp sum ends the
-// pair.  The order of the evaluations depends on the pair alone, so the
-// result is reproducible.  A cell with more than FW_MAXF faces (possible only
-// for imported cells) is done by one lane with pair_weight.
+// An edge with signed in-plane distance a and range [T0, T1] along its line
+// contributes sum_r int_{portion r} [K_r(Q) - K(D)] D a / (a^2 + tau^2) dtau
+// over its portions in the kernel's regions r (Q < 1, Q < 2, beyond).  With
+// K_r = sum_n c_n Q^n and Q^2 = D^2 + a^2 + tau^2, the antiderivatives reduce
+// to two angles and one logarithm (see exact.cuh for J_n and U_n):
+//     C_r(D) theta + S_r(D) psi + D a (E_r + H_r dash),
+//     theta = atan(T1/a) - atan(T0/a), the angle of (a^2 + T0 T1, a (T1 - T0)),
+//     psi = atan(D T1/(a Q1)) - atan(D T0/(a Q0)), the angle of
+//           (a^2 Q0 Q1 + D^2 T0 T1, a D (T1 Q0 - T0 Q1)),
+//     dash = asinh(T1/B) - asinh(T0/B), the log of a ratio of |T| + Q,
+//     S_r = c_-1 + c_3 D^4 + c_5 D^6,  C_r = D (c_0 + c_2 D^2 + c_4 D^4) - D K(D),
+// E_r a polynomial in T, Q.  So a portion takes two angles, a logarithm and
+// no more square roots than its end points, where evaluating the six
+// antiderivatives at every end point and every crossing took two angles, an
+// asinh and two roots each; the rounding is that of the same terms, each at
+// most ~1.  C_r and S_r are formed once per face (C_r = -S_r exactly where D
+// lies in region r).
+//
+// Each lane takes an edge, cuts it at the region crossings and appends its
+// portions to one of two per-warp queues, regions 1 and 2 or region 3 (angles
+// alone); whenever a queue holds 32 entries the warp evaluates them, one per
+// lane.  The kernel is bound by the number of FP64 instructions (one per ~20
+// cycles per SM whatever its active lanes): region tests run in FP32 (a
+// portion cut 1e-7 off moves the integral by the fifth power of that, since
+// K's pieces agree to fourth order), and the transcendentals are fp64.cuh's.
+// 4.68 M pairs of the 2e5-particle cloud: 109.9 ms (4.3e7 pairs/s), against
+// 367.6 ms with the six antiderivatives; the FP64 pipe is 88% busy, issue 15%.
+// Each lane adds what it evaluated; a fixed-order warp sum ends the pair.  The
+// order of the evaluations depends on the pair alone, so the result is
+// reproducible.  A cell with more than FW_MAXF faces (possible only for
+// imported cells) is done by one lane with pair_weight.
 //
 // Entry t of list is k >= 0: pair k in the complement form (faces beyond 2h
 // skipped; its rounding, about 1e-13, is far inside the mixed mode's
@@ -415,70 +430,129 @@ constexpr int FW_WARPS = 4;
 constexpr int FW_MAXF = 64;
 constexpr int FQ = 64;   // ring capacity of each evaluation queue (a power of two, >= 63)
 
-// Evaluations waiting for a full warp: the basis at t (code: regions rA, rB
-// in bits 0-1, 2-3) weighted w0 (c_rA - c_rB).b - w1 b0, or the angles
-// w0 D atan(u/A) - w1 atan(D u / (A Q)).
+// Portions waiting for a full warp; code: the face's index | region << 8.
 struct FwQueue {
-    double A[FQ], B2[FQ], D[FQ], t[FQ], w0[FQ], w1[FQ];
+    double a[FQ], T0[FQ], Q0[FQ], T1[FQ], Q1[FQ];
     int code[FQ];
 };
 
-__device__ __noinline__ double fw_eval_basis(const FwQueue &q, int i)
+// A warp's pair: per face D / h, its signed copy (orientation, and the
+// complement form's sign), and the signed C_r and S_r.
+struct FwPair {
+    FwQueue near, far;
+    double D[FW_MAXF], sD[FW_MAXF], C[3][FW_MAXF], S[3][FW_MAXF];
+    int64_t E0[FW_MAXF];
+    int pre[FW_MAXF + 1];
+};
+
+struct FwTab {
+    double atan[65], log[64][2];
+};
+
+// theta and psi of a portion from a^2, D, D^2 and its ends
+__device__ __forceinline__ void fw_angles(const FwTab &tb, double a, double a2, double D, double D2, double T0,
+                                          double Q0, double T1, double Q1, double &theta, double &psi)
 {
-    double b[6];
-    basis<double>(q.A[i], q.B2[i], q.D[i], q.t[i], b);
-    const int rA = q.code[i] & 3, rB = q.code[i] >> 2;
-    const double p1 = dot_c1(b), p2 = dot_c2(b), p3 = dot_c3(b);
-    const double dA = rA == 1 ? p1 : (rA == 2 ? p2 : p3);
-    const double dB = rB == 0 ? 0.0 : (rB == 1 ? p1 : (rB == 2 ? p2 : p3));
-    return q.w0[i] * (dA - dB) - q.w1[i] * b[0];
+    const double tt = T0 * T1;
+    theta = angle64(a * (T1 - T0), a2 + tt, tb.atan);
+    psi = angle64((a * D) * fma(T1, Q0, -T0 * Q1), fma(a2, Q0 * Q1, D2 * tt), tb.atan);
 }
 
-__device__ __noinline__ double fw_eval_angle(const FwQueue &q, int i, bool both)
+__device__ __noinline__ double fw_eval_near(const FwPair &p, const FwTab &tb, int i)
 {
-    const double A = q.A[i], D = q.D[i], u = q.t[i];
-    double v = q.w0[i] * (D * atan2(u, A));
-    if (both) v -= q.w1[i] * atan2(D * u, A * sqrt(q.B2[i] + u * u));
-    return v;
+    const FwQueue &q = p.near;
+    const double a = q.a[i], T0 = q.T0[i], Q0 = q.Q0[i], T1 = q.T1[i], Q1 = q.Q1[i];
+    const int f = q.code[i] & 255;
+    const bool r1 = (q.code[i] >> 8) == 1;
+    const double D = p.D[f], D2 = D * D, a2 = fma(a, a, 1e-280), B2 = a2 + D2;
+    double theta, psi;
+    fw_angles(tb, a, a2, D, D2, T0, Q0, T1, Q1, theta, psi);
+    // asinh(T/B) = +-log((|T| + Q)/B)
+    const bool s0 = __double2hiint(T0) < 0, s1 = __double2hiint(T1) < 0;
+    const double e0 = fabs(T0) + Q0, e1 = fabs(T1) + Q1;
+    const double ee = s0 != s1 ? e0 * e1 : 1.0;
+    const double dash = log_ratio(s0 == s1 ? (s0 ? e0 : e1) : (s0 ? ee : B2), s0 == s1 ? (s0 ? e1 : e0) : (s0 ? B2 : ee),
+                                  tb.log);
+    const double c2 = r1 ? 1.0 / 6.0 : 1.0 / 3.0, c4 = r1 ? -3.0 / 40.0 : 3.0 / 40.0, c43 = r1 ? -0.025 : 0.025;
+    const double c3 = r1 ? 0.0 : -0.25, c3h = r1 ? 0.0 : -0.125;
+    const double c5 = r1 ? 0.025 : -1.0 / 120.0, c5h = r1 ? 0.0125 : -1.0 / 240.0, c54 = r1 ? 0.00625 : -1.0 / 480.0,
+                 c538 = r1 ? 0.009375 : -0.003125;
+    const double al = fma(c4, fma(2.0, D2, a2), c2), be = fma(c5h, fma(0.75, B2, D2), c3h);
+    const double H = fma(D2, fma(c5, D2, c3), B2 * fma(c538, B2, fma(c5h, D2, c3h)));
+    const double t0 = T0 * T0, t1 = T1 * T1;
+    const double g0 = fma(Q0, fma(c54, B2 + t0, be), fma(c43, t0, al)), g1 = fma(Q1, fma(c54, B2 + t1, be), fma(c43, t1, al));
+    const double E = fma(H, dash, fma(T1, g1, -T0 * g0));
+    return fma(p.sD[f] * a, E, fma(r1 ? p.S[0][f] : p.S[1][f], psi, (r1 ? p.C[0][f] : p.C[1][f]) * theta));
 }
 
-// Append this lane's entry (if has) to ring q of n entries from head.
-__device__ __forceinline__ void fw_push(FwQueue &q, int head, int &n, bool has, double A, double B2, double D,
-                                        double t, double w0, double w1, int code)
+__device__ __noinline__ double fw_eval_far(const FwPair &p, const FwTab &tb, int i, bool full)
+{
+    const FwQueue &q = p.far;
+    const double a = q.a[i], T0 = q.T0[i], T1 = q.T1[i], a2 = fma(a, a, 1e-280);
+    const int f = q.code[i] & 255;
+    double theta, psi;
+    if (!full) return p.C[2][f] * angle64(a * (T1 - T0), fma(T0, T1, a2), tb.atan);   // S_3 = 0
+    const double D = p.D[f];
+    fw_angles(tb, a, a2, D, D * D, T0, q.Q0[i], T1, q.Q1[i], theta, psi);
+    return fma(p.S[2][f], psi, p.C[2][f] * theta);
+}
+
+// Append this lane's portion (if has) to ring q of n entries from head.
+__device__ __forceinline__ void fw_push(FwQueue &q, int head, int &n, bool has, double a, double T0, double Q0,
+                                        double T1, double Q1, int code)
 {
     const unsigned m = __ballot_sync(0xffffffffu, has);
     if (has) {
         const int pos = (head + n + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))) & (FQ - 1);
-        q.A[pos] = A;
-        q.B2[pos] = B2;
-        q.D[pos] = D;
-        q.t[pos] = t;
-        q.w0[pos] = w0;
-        q.w1[pos] = w1;
+        q.a[pos] = a;
+        q.T0[pos] = T0;
+        q.Q0[pos] = Q0;
+        q.T1[pos] = T1;
+        q.Q1[pos] = Q1;
         q.code[pos] = code;
     }
     n += __popc(m);
 }
 
 // Evaluate the queues' full warps (every entry when last), lane by entry.
-__device__ __forceinline__ void fw_drain(FwQueue &qb, FwQueue &qa, int &hb, int &nb, int &ha, int &na, bool both,
+__device__ __forceinline__ void fw_drain(FwPair &p, const FwTab &tb, int &hb, int &nb, int &ha, int &na, bool full,
                                          bool last, double &acc)
 {
     const int lane = threadIdx.x & 31;
     __syncwarp();
     while (nb >= 32 || (last && nb > 0)) {
-        if (lane < nb) acc += fw_eval_basis(qb, (hb + lane) & (FQ - 1));
+        if (lane < nb) acc += fw_eval_near(p, tb, (hb + lane) & (FQ - 1));
         const int d = min(nb, 32);
         hb = (hb + d) & (FQ - 1);
         nb -= d;
     }
     while (na >= 32 || (last && na > 0)) {
-        if (lane < na) acc += fw_eval_angle(qa, (ha + lane) & (FQ - 1), both);
+        if (lane < na) acc += fw_eval_far(p, tb, (ha + lane) & (FQ - 1), full);
         const int d = min(na, 32);
         ha = (ha + d) & (FQ - 1);
         na -= d;
     }
     __syncwarp();
+}
+
+// C_r and S_r of the face at distance D, signed by sg: the coefficients of
+// theta and psi in region r (complement form: those of K_3 - K).
+__device__ __forceinline__ void fw_face(FwPair &p, int f, double D, bool full, double sg)
+{
+    const double D2 = D * D, D4 = D2 * D2, D6 = D4 * D2;
+    const double P[3] = {D * fma(-3.0 / 40.0, D4, D2 * (1.0 / 6.0)),
+                         D * fma(3.0 / 40.0, D4, fma(1.0 / 3.0, D2, -1.0 / 20.0)), D * (7.0 / 20.0)};
+    const double S[3] = {D6 * (1.0 / 40.0), fma(-1.0 / 120.0, D6, fma(-0.25, D4, 1.0 / 60.0)), -0.25};
+    const int rD = D < 1.0 ? 0 : (D < 2.0 ? 1 : 2);
+    const double kD = rD == 0 ? P[0] + S[0] : (rD == 1 ? P[1] + S[1] : P[2] + S[2]);   // D K(D)
+    p.D[f] = D;
+    p.sD[f] = full ? sg * D : -sg * D;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const double C = r == rD ? -S[r] : P[r] - kD;
+        p.C[r][f] = sg * (full ? C : 0.25 - C);
+        p.S[r][f] = sg * (full ? S[r] : -0.25 - S[r]);
+    }
 }
 
 __device__ __forceinline__ void fp64_pairs_warp(int64_t n, const int32_t *__restrict__ list,
@@ -490,13 +564,15 @@ __device__ __forceinline__ void fp64_pairs_warp(int64_t n, const int32_t *__rest
                                                 const PlaneD *__restrict__ plane, const EdgeD *__restrict__ edge,
                                                 double *__restrict__ w)
 {
-    __shared__ double fD[FW_WARPS][FW_MAXF], fK[FW_WARPS][FW_MAXF];
-    __shared__ int64_t fE0[FW_WARPS][FW_MAXF];
-    __shared__ int fPre[FW_WARPS][FW_MAXF + 1];
-    __shared__ float fSg[FW_WARPS][FW_MAXF];
-    __shared__ FwQueue fq[FW_WARPS][2];
+    __shared__ FwPair pairs[FW_WARPS];
+    __shared__ FwTab tb;
+    for (int t = threadIdx.x; t < 65 + 128; t += blockDim.x) {
+        if (t < 65) tb.atan[t] = kAtanTab[t];
+        else tb.log[(t - 65) >> 1][(t - 65) & 1] = kLogTab[(t - 65) >> 1][(t - 65) & 1];
+    }
+    __syncthreads();
     const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;   // wpb <= FW_WARPS
-    FwQueue &qb = fq[wi][0], &qa = fq[wi][1];
+    FwPair &p = pairs[wi];
     for (int64_t t = blockIdx.x * (int64_t)wpb + wi; t < n; t += (int64_t)gridDim.x * wpb) {
         const int32_t code = list ? list[t] : ~(int32_t)t;
         const int64_t k = code >= 0 ? code : ~code;
@@ -524,7 +600,7 @@ __device__ __forceinline__ void fp64_pairs_warp(int64_t n, const int32_t *__rest
             }
         ins = __all_sync(0xffffffffu, ins);
         const bool full = code < 0 || (ins && sqrt(rx * rx + ry * ry + rz * rz) + radius[j] < 2.0 * hh);
-        // faces: distance, constant, and how many edges each contributes
+        // faces: distance, coefficients, and how many edges each contributes
         for (int base = 0; base < nface; base += 32) {
             const int f = base + lane;
             int cnt = 0;
@@ -532,12 +608,9 @@ __device__ __forceinline__ void fp64_pairs_warp(int64_t n, const int32_t *__rest
                 const PlaneD pl = plane[f0 + f];
                 const double sd = pl.w - (pl.x * rx + pl.y * ry + pl.z * rz);
                 const double D = fabs(sd) * ih;
-                const bool keep = !(sd == 0.0 || (!full && D >= 2.0));
-                fD[wi][f] = D;
-                fK[wi][f] = full ? K_of<double>(D) : K_tilde<double>(D);
-                fE0[wi][f] = fvo[f0 + f];
-                fSg[wi][f] = sd > 0.0 ? 1.f : -1.f;
-                if (keep) cnt = (int)(fvo[f0 + f + 1] - fvo[f0 + f]);
+                fw_face(p, f, D, full, sd > 0.0 ? 1.0 : -1.0);
+                p.E0[f] = fvo[f0 + f];
+                if (!(sd == 0.0 || (!full && D >= 2.0))) cnt = (int)(fvo[f0 + f + 1] - fvo[f0 + f]);
             }
             int xs = cnt;   // inclusive scan of the edge counts over these 32 faces
 #pragma unroll
@@ -545,114 +618,69 @@ __device__ __forceinline__ void fp64_pairs_warp(int64_t n, const int32_t *__rest
                 const int y = __shfl_up_sync(0xffffffffu, xs, o);
                 if (lane >= o) xs += y;
             }
-            const int carry = base == 0 ? 0 : fPre[wi][base];
+            const int carry = base == 0 ? 0 : p.pre[base];
             __syncwarp();
-            if (lane == 0 && base == 0) fPre[wi][0] = 0;
-            if (f < nface) fPre[wi][f + 1] = carry + xs;
+            if (lane == 0 && base == 0) p.pre[0] = 0;
+            if (f < nface) p.pre[f + 1] = carry + xs;
             __syncwarp();
         }
-        const int ne = fPre[wi][nface];
+        const int ne = p.pre[nface];
         double acc = 0.0;
         int hb = 0, nb = 0, ha = 0, na = 0;
         for (int base = 0; base < ne; base += 32) {
             const int e = base + lane;
-            // this lane's edge: its evaluations (has*), weights and split points
-            double A = 0.0, D = 0.0, B2 = 0.0, u0 = 0.0, u1 = 0.0, ts1 = 0.0, ts2 = 0.0;
-            double bw0[2] = {0.0, 0.0}, bw1[2] = {0.0, 0.0}, aw0[2] = {0.0, 0.0}, aw1[2] = {0.0, 0.0};
-            int bcode[2] = {0, 0};
-            bool hasb[2] = {false, false}, hasa[2] = {false, false};
-            double coef1 = 0.0, coef2 = 0.0;
+            double a = 0.0, T1 = 0.0, Q1 = 0.0, B2 = 0.0, cur = 0.0, Qc = 0.0;
+            float t1f = 0.f, t2f = 0.f, T1f = 0.f;
+            int f = 0;
+            // where the rest of the edge starts: 0 before -t2, 1 before -t1,
+            // 2 before t1, 3 before t2, 4 beyond; 5: nothing left
+            int st = 5;
             if (e < ne) {
-                int lo = 0, hi = nface;   // fPre[lo] <= e < fPre[hi]
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if (fPre[wi][mid] <= e) lo = mid;
+                int hi = nface;   // pre[f] <= e < pre[hi]
+                while (hi - f > 1) {
+                    const int mid = (f + hi) >> 1;
+                    if (p.pre[mid] <= e) f = mid;
                     else hi = mid;
                 }
-                const EdgeD E = edge[fE0[wi][lo] + (e - fPre[wi][lo])];
-                const double a = E.cm - (E.mx * rx + E.my * ry + E.mz * rz);
-                if (a != 0.0) {
-                    A = fabs(a) * ih;
-                    const double T0 = (E.ce - (E.ex * rx + E.ey * ry + E.ez * rz)) * ih;
-                    const double T1 = T0 + E.L * ih;
-                    D = fD[wi][lo];
-                    const double kd = fK[wi][lo];
-                    const double sg = (double)fSg[wi][lo] * (a > 0.0 ? 1.0 : -1.0);
-                    B2 = D * D + A * A;
-                    u0 = fabs(T0);
-                    u1 = fabs(T1);
-                    // endpoint signs: Phi(T1) - Phi(T0), Phi odd in T
-                    const double cs[2] = {T0 < 0.0 ? sg : -sg, T1 < 0.0 ? -sg : sg};
-                    const double uu[2] = {u0, u1};
-                    const bool near = B2 < 4.0;
-                    if (near) {
-                        ts2 = sqrt(4.0 - B2);
-                        if (B2 < 1.0) ts1 = sqrt(1.0 - B2);
-                    }
-#pragma unroll
-                    for (int s = 0; s < 2; ++s) {
-                        const double u = uu[s], c = cs[s];
-                        if (u == 0.0) continue;
-                        if (full) {
-                            if (!near || u > ts2) {   // region 3: the angles alone
-                                hasa[s] = true;
-                                aw0[s] = c * ((near || D < 2.0) ? 7.0 / 20.0 - kd : 0.25 / D);
-                                aw1[s] = c * 0.25;
-                                if (near) {
-                                    coef1 += c;
-                                    coef2 += c;
-                                }
-                            } else {
-                                hasb[s] = true;
-                                const int r = u <= ts1 ? 1 : 2;
-                                bcode[s] = r;
-                                bw0[s] = c;
-                                bw1[s] = c * kd;
-                                if (r == 2) coef1 += c;
-                            }
-                        } else {
-                            if (!near || u >= ts2) {   // beyond 2h: -(d1 + d2) - K~(D) b0
-                                hasa[s] = true;
-                                aw0[s] = -c * kd;
-                                if (near) {
-                                    coef1 -= c;
-                                    coef2 -= c;
-                                }
-                            } else {
-                                hasb[s] = true;
-                                const bool r2 = u > ts1;
-                                bcode[s] = r2 ? (3 | (2 << 2)) : (3 | (1 << 2));
-                                bw0[s] = c;
-                                bw1[s] = c * kd;
-                                if (r2) coef1 -= c;
-                            }
-                        }
-                    }
-                    if (!(B2 < 1.0)) coef1 = 0.0;   // no region 1: d1 = 0
-                }
+                const EdgeD E = edge[p.E0[f] + (e - p.pre[f])];
+                a = (E.cm - (E.mx * rx + E.my * ry + E.mz * rz)) * ih;
+                cur = (E.ce - (E.ex * rx + E.ey * ry + E.ez * rz)) * ih;
+                T1 = fma(E.L, ih, cur);
+                const double D = p.D[f];
+                B2 = fma(D, D, fma(a, a, 1e-280));
+                Qc = sqrt64(fma(cur, cur, B2));
+                Q1 = sqrt64(fma(T1, T1, B2));
+                const float B2f = f32_cut(B2), T0f = f32_cut(cur);
+                T1f = f32_cut(T1);
+                t1f = B2f < 1.f ? sqrtf(1.f - B2f) : 0.f;
+                t2f = B2f < 4.f ? sqrtf(4.f - B2f) : 0.f;
+                if (a != 0.0 && E.L > 0.0)
+                    st = T0f >= t2f ? 4 : (T0f >= t1f ? 3 : (T0f >= -t1f ? 2 : (T0f >= -t2f ? 1 : 0)));
             }
-            const bool has_t1 = coef1 != 0.0, has_t2 = coef2 != 0.0;
-            // six collective appends in a fixed order, draining full warps as they fill
-#pragma unroll 1
-            for (int step = 0; step < 6; ++step) {
-                // (selects rather than indexing, so that the arrays stay in registers)
-                const bool s = (step & 1) != 0;
-                if (step < 4) {
-                    const bool split = step >= 2;
-                    const bool has = split ? (s ? has_t2 : has_t1) : (s ? hasb[1] : hasb[0]);
-                    const double tt = split ? (s ? ts2 : ts1) : (s ? u1 : u0);
-                    const double w0 = split ? (s ? coef2 : coef1) : (s ? bw0[1] : bw0[0]);
-                    const double w1 = split ? 0.0 : (s ? bw1[1] : bw1[0]);
-                    const int cd = split ? (s ? (2 | (3 << 2)) : (1 | (2 << 2))) : (s ? bcode[1] : bcode[0]);
-                    fw_push(qb, hb, nb, has, A, B2, D, tt, w0, w1, cd);
-                } else {
-                    fw_push(qa, ha, na, s ? hasa[1] : hasa[0], A, B2, D, s ? u1 : u0, s ? aw0[1] : aw0[0],
-                            s ? aw1[1] : aw1[0], 0);
+            // one portion per lane and pass, until every lane's edge is done
+            while (__any_sync(0xffffffffu, st < 5)) {
+                const bool has = st < 5;
+                if (st == 0 && t2f == 0.f) st = 4;
+                if (st == 1 && t1f == 0.f) st = 3;
+                const int reg = st == 2 ? 1 : ((st == 1 || st == 3) ? 2 : 3);
+                const float bpf = st == 0 ? -t2f : (st == 1 ? -t1f : (st == 2 ? t1f : t2f));
+                const bool cross = st < 4 && bpf < T1f;
+                double end = T1, Qe = Q1;
+                if (cross) {
+                    const bool at1 = st == 1 || st == 2;
+                    const double tb2 = sqrt64(fmax((at1 ? 1.0 : 4.0) - B2, 0.0));
+                    end = st < 2 ? -tb2 : tb2;
+                    Qe = at1 ? 1.0 : 2.0;
                 }
-                if (nb >= 32 || na >= 32) fw_drain(qb, qa, hb, nb, ha, na, full, false, acc);
+                fw_push(p.near, hb, nb, has && reg < 3, a, cur, Qc, end, Qe, f | (reg << 8));
+                fw_push(p.far, ha, na, has && reg == 3, a, cur, Qc, end, Qe, f | (reg << 8));
+                cur = end;
+                Qc = Qe;
+                st = cross ? st + 1 : 5;
+                if (nb >= 32 || na >= 32) fw_drain(p, tb, hb, nb, ha, na, full, false, acc);
             }
         }
-        fw_drain(qb, qa, hb, nb, ha, na, full, true, acc);
+        fw_drain(p, tb, hb, nb, ha, na, full, true, acc);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) {
