@@ -721,23 +721,30 @@ __global__ void __launch_bounds__(32 * FW_WARPS) k_map_fp64(
 // distance D in float-float and an FP32 pass for the reference R = distance
 // from p to the face polygon (any value used consistently for the face is
 // exact when P is outside the polygon; inside, R = D), then R, 2 - R, K(R)
-// and K(1) - K(R) in FP32; per edge A, T0, T1, B^2 - 1, 4 - B^2 and
-// A^2 - rho^2 in float-float, each rounded once to FP32.  The FP64 pipe runs
-// at 1/64 of the FP32 rate, so nothing per face, edge or quadrature segment
-// touches it: the pieces are summed in float-float.
+// and K(1) - K(R) in FP32; per edge A, T0, T1 and B^2 in float-float, and from
+// them the segments' Q^2 - R^2 and 4 - Q^2, each rounded once to FP32.  The
+// FP64 pipe runs at 1/64 of the FP32 rate, so nothing per face, edge or
+// quadrature segment touches it: the pieces are summed in float-float.
 //
-// Each edge yields up to four quadrature segments, which the lane appends to
-// its column of a per-warp queue in shared memory; whenever a lane's column
-// may overflow, the warp evaluates all queued segments together, one 4-node
-// slot (a 4-point segment, or half of an 8-point sub-piece) per lane, so that
-// the node loop runs with the warp converged whatever the pairs' geometry.
-// Each lane then adds its own segments' results in a fixed order, which keeps
-// the result bit-reproducible.  The queue is small (9.1 KB per warp) so that
-// 12 two-warp blocks fit an SM: the pass is bound by instruction issue, and
-// the warps hide its latencies.  The estimated error 8 eps times the sum of
-// the magnitudes of the non-negative pieces flags the pair for the FP64 pass
-// when it exceeds max(tol |w|, 1e-14) (relative accuracy tol for every weight
-// above 1e-14 / tol, absolute 1e-14 below); so does a face plane through P.
+// Each edge yields up to four quadrature segments (one for most), which the
+// lane appends to its column of a per-warp queue in shared memory; whenever a
+// lane's column may overflow, the warp evaluates all queued segments together,
+// one 6-node slot (a 6-point segment, or half of a 12-point sub-piece) per
+// lane, so that the node loop runs with the warp converged whatever the pairs'
+// geometry.  Each lane then adds its own segments' results in a fixed order,
+// which keeps the result bit-reproducible.  The queue is small (9 KB per
+// warp) so that 12 two-warp blocks fit an SM: the pass is bound by instruction
+// issue, and the warps hide its latencies.  The estimated error 8 eps times
+// the sum of the magnitudes of the non-negative pieces flags the pair for the
+// FP64 pass when it exceeds max(tol |w|, 1e-14) (relative accuracy tol for
+// every weight above 1e-14 / tol, absolute 1e-14 below); so does a face plane
+// through P.
+//
+// 24.06 M pairs of the 1e6-particle cloud: 71.2 ms (3.4e8 pairs/s), against
+// 111 ms with 4- and 8-point rules in s = asinh(tau / A), an asinh per
+// segment and an exponential per node, the two sides of every edge queued in
+// turn, and correctly rounded or subnormal-safe reciprocals; the error against
+// FP64 fell from 2.5e-7 to 2.4e-7 RMS.
 namespace {
 
 // factor of the FP32 pass's error estimate: fp32_err_ulps units of 2^-24
@@ -754,18 +761,6 @@ double em_est_k(const em_params *p)
 #ifndef EM_MQ_WARPS
 #define EM_MQ_WARPS 2
 #endif
-#ifndef EM_G8_MAXLEN_FAR
-// longest 8-point sub-piece (in s) of the second kernel piece on a face
-// whose plane lies beyond h (R >= 1); elsewhere 2.  On that branch the
-// 8-point rule's truncation reaches ~5 ulp of the segment at length 2 and
-// ~0.3 ulp at 1.5 (an FP64 model of the integrand against adaptive
-// quadrature); the error estimate counts rounding only
-#define EM_G8_MAXLEN_FAR 2.0
-#endif
-static_assert(EM_G8_MAXLEN_FAR >= 0.5 && EM_G8_MAXLEN_FAR <= 2.0, "sub-pieces per segment must stay below 256");
-#ifndef EM_GL4_MAXLEN
-#define EM_GL4_MAXLEN 0.125   // longest segment (in s) integrated with 4 points
-#endif
 #ifndef EM_MQ_MINB
 // minimum resident blocks per SM asked of the compiler (0: none): 12 two-warp
 // blocks, 24 warps, is what the shared memory of 12 queues allows (18.2 KB a
@@ -777,17 +772,17 @@ constexpr int MQ_WARPS = EM_MQ_WARPS;   // warps per block
 constexpr int MQ_CHUNK = 64;            // sub-piece results a warp holds between accumulations
 static_assert(MQ_SLOTS >= 5, "an edge queues up to four segments");
 static_assert(MQ_CHUNK % 32 == 0, "whole rounds of the warp");
-// a lane holds at most MQ_SLOTS segments of at most 2 x 141 slots each (m <= 141)
+// a lane holds at most MQ_SLOTS segments of at most 2 x 28 slots each (m <= 28)
 constexpr int MQ_NOSLOT = 4095;
-static_assert(MQ_SLOTS * 282 < MQ_NOSLOT, "slot indices fit in 12 bits");
+static_assert(MQ_SLOTS * 56 < MQ_NOSLOT, "slot indices fit in 12 bits");
 constexpr unsigned FULL_MASK = 0xffffffffu;
 
 struct SegQueue {
-    float ts[MQ_SLOTS][32], hl[MQ_SLOTS][32], A[MQ_SLOTS][32];
+    float ts[MQ_SLOTS][32], len[MQ_SLOTS][32], A[MQ_SLOTS][32];
     float B2[MQ_SLOTS][32], c4s[MQ_SLOTS][32], es[MQ_SLOTS][32], Rr[MQ_SLOTS][32], vv[MQ_SLOTS][32];
     float add[MQ_SLOTS][32], scale[MQ_SLOTS][32];
-    // m | piece1 | tilde | gl4 (quad32.cuh) in the low 16 bits; during a
-    // flush, the index of the segment's first 4-node slot among its lane's
+    // m | piece1 | tilde | six (quad32.cuh) in the low 16 bits; during a
+    // flush, the index of the segment's first slot among its lane's
     // in bits 16-27 (MQ_NOSLOT for an empty row)
     int meta[MQ_SLOTS][32];
     float vhi[MQ_CHUNK], vlo[MQ_CHUNK];   // scale * integral of each evaluated slot (float-float)
@@ -796,13 +791,13 @@ struct SegQueue {
 
 // Evaluate every queued segment of the warp and add each lane's results to
 // its pair.  Called with the warp converged.  The work is spread by
-// slot (4 quadrature nodes: a 4-point segment, or half of an 8-point
+// slot (6 quadrature nodes: a 6-point segment, or half of a 12-point
 // sub-piece): lane L's segments hold M_L slots in queue order, the warp
 // numbers all of them L by L and evaluates them 32 at a time, whoever owns
 // them, so that a segment cut into many sub-pieces does not hold up the
 // lanes.  Each result, times its segment's signed factor, is
 // kept exactly as a float-float product; the owner then adds its own results
-// in order into its float-float sum (to about 2^-44 of the magnitudes), which
+// in order into its float-float sum, which
 // keeps the sum bit-reproducible, and their magnitudes in FP32: they only
 // scale the error bound.
 __device__ __forceinline__ void mq_flush(SegQueue &q, int lane, int cnt, emq::ff &acc, float &mag)
@@ -812,7 +807,7 @@ __device__ __forceinline__ void mq_flush(SegQueue &q, int lane, int cnt, emq::ff
     for (int sl = 0; sl < MQ_SLOTS; ++sl) {
         const int mt = q.meta[sl][lane] & 0xffff;
         q.meta[sl][lane] = mt | ((sl < cnt ? M : MQ_NOSLOT) << 16);
-        if (sl < cnt) M += (mt & emq::SEG_GL4) ? (mt & 255) : 2 * (mt & 255);   // 4-point: 1 slot, 8-point: 2 per sub-piece
+        if (sl < cnt) M += (mt & emq::SEG_SIX) ? 1 : 2 * (mt & 255);   // 6-point: 1 slot, 12-point: 2 per sub-piece
     }
     int x = M;
 #pragma unroll
@@ -842,19 +837,10 @@ __device__ __forceinline__ void mq_flush(SegQueue &q, int lane, int cnt, emq::ff
             const int mw = q.meta[sl][lo];
             const int rr = r - (mw >> 16);
             const int mt = mw & 0xffff;
-            const bool gl4 = (mt & emq::SEG_GL4) != 0;
-            const int p = gl4 ? rr : rr >> 1;           // the sub-piece
-            const int half = gl4 ? 2 : (rr & 1);        // which 4 nodes of its rule
-            const float hl = q.hl[sl][lo];
-            // sinh and cosh of s at the segment's start, ts / A and
-            // sqrt(1 + (ts / A)^2) (not stored, which keeps the queue small
-            // enough for more warps per SM)
-            const float ts = q.ts[sl][lo], A = q.A[sl][lo];
-            const float Sa = ts * __frcp_rn(A);
-            const float Ca = emq::sqrt_nr(fmaf(Sa, Sa, 1.f));
-            const float val = emq::slot_eval((2.f * (float)p + 1.f) * hl, hl, half, ts, Sa, Ca, A, q.B2[sl][lo],
-                                             q.c4s[sl][lo], q.es[sl][lo],
-                                             q.Rr[sl][lo], q.vv[sl][lo], q.add[sl][lo], mt);
+            const bool six = (mt & emq::SEG_SIX) != 0;
+            const float val = emq::slot_eval(six ? 0 : rr >> 1, six ? 0 : 1 + (rr & 1), q.ts[sl][lo], q.len[sl][lo],
+                                             q.A[sl][lo], q.B2[sl][lo], q.c4s[sl][lo], q.es[sl][lo], q.Rr[sl][lo],
+                                             q.vv[sl][lo], q.add[sl][lo], mt);
             const emq::ff v = emq::ff_two_prod(q.scale[sl][lo], val);
             q.vhi[t - c0] = v.hi;
             q.vlo[t - c0] = v.lo;
@@ -862,9 +848,11 @@ __device__ __forceinline__ void mq_flush(SegQueue &q, int lane, int cnt, emq::ff
         __syncwarp();
         const int e1 = min(x, c1);
         for (int t = max(mine0, c0); t < e1; ++t) {
-            const emq::ff v{q.vhi[t - c0], q.vlo[t - c0]};
-            acc = emq::ff_add(acc, v);
-            mag += fabsf(v.hi);
+            // (the low parts' sum needs no renormalisation: its rounding is 2^-48 of the magnitudes)
+            const emq::ff s2 = emq::ff_two_sum(acc.hi, q.vhi[t - c0]);
+            acc.hi = s2.hi;
+            acc.lo += s2.lo + q.vlo[t - c0];
+            mag += fabsf(q.vhi[t - c0]);
         }
         __syncwarp();
     }
@@ -872,8 +860,7 @@ __device__ __forceinline__ void mq_flush(SegQueue &q, int lane, int cnt, emq::ff
 
 // Face constants of the lane's current face.
 struct FaceState {
-    emq::ff dm1, d4;            // D^2 - 1, 4 - D^2 (float-float, units of h)
-    float rr2;                  // rho^2 (units of h; FP32 by construction)
+    emq::ff D2, R2;             // D^2 and R^2 (float-float, units of h)
     float Df, R, v, KR, C1;     // v = 2 - R
     float sign;   // orientation of the face as seen from P (sign of the signed distance)
 };
@@ -928,81 +915,94 @@ __device__ __forceinline__ void face_consts(emq::ff R2x, bool tilde, FaceState &
     fs.KR = tilde ? kt2 : k3 - kt2;
 }
 
-// Queue the kernel pieces of (D/pi) int over |tau| in [ua, ua + du] (one
-// g-integral of an edge) with the signed factor sc; the part beyond 2h is
-// added directly.  du is the range's length from an accurate difference (the
-// edge length L/h, or |T| for a range starting at the foot), and every
-// segment's length in s is formed from such a difference: with a = ua and
-// b = ua + o,
-//     asinh(b/A) - asinh(a/A) = asinh(o (a + b) / (b sqrt(A^2 + a^2) + a sqrt(A^2 + b^2))),
-// an identity whose right side keeps the relative precision of o.  The
-// difference of two asinh values, each rounded to FP32, would carry an
-// absolute error of about 2^-24 |s|, which on a short segment (a small face
-// seen from afar: |T| ~ 1, L/h ~ 0.05) is tens of ulps of the segment, and
-// the error estimate, which counts rounding relative to the segments' sizes,
-// would not see it.  Where a segment starts (sa) needs no such care: shifting
-// a short segment moves its integral only by the integrand's change across it.
-__device__ __forceinline__ void mq_push_g(SegQueue &q, int lane, int &cnt, float ua, float du, float A, float B2,
-                                          emq::ff c1x, emq::ff c4x, emq::ff ccx, float sc, const FaceState &fs,
-                                          bool tilde, emq::ff &acc, float &mag)
+// Queue one segment of an edge: tau from t (float-float) over length len (from
+// accurate offsets, see mq_edge) on kernel piece `piece`, with signed factor sc.
+// The nodes lie at offsets from t rounded to FP32, but Q^2 - Rr^2 and 4 - Q^2
+// are taken at t itself: t's rounding, 6e-8, would shift a segment of length
+// 0.05 against its neighbours by a millionth of itself.
+__device__ __forceinline__ void mq_push(SegQueue &q, int lane, int sl, int piece, emq::ff t, float len, float A,
+                                        float A2, float B2f, emq::ff B2, float sc, const FaceState &fs, bool tilde)
 {
-    const float c1 = c1x.hi + c1x.lo, c4 = c4x.hi + c4x.lo;
-    const float t1 = c1 < 0.f ? emq::sqrt_nr(-c1) : 0.f;
-    const float t2 = c4 > 0.f ? emq::sqrt_nr(c4) : 0.f;
-    const int tflag = tilde ? emq::SEG_TILDE : 0;
-    // a segment of kernel piece `piece` from tau = ts (s-length len)
-    auto push = [&](int piece, float ts, float len) {
-        // 4 points for a short segment, else 8 on sub-pieces of length <= 2
-        const bool gl4 = len <= (float)EM_GL4_MAXLEN;
-        const float g8 = (piece == 2 && fs.R >= 1.f) ? (float)EM_G8_MAXLEN_FAR : 2.f;
-        // m <= ceil(70.5 / g8) <= 141: A >= 1e-30, |tau| <= 2
-        const int m = len > g8 ? (int)ceilf(len * (1.f / g8)) : 1;
-        const int sl = cnt++;
-        const bool ref1 = piece == 2 && fs.R < 1.f;   // difference split at Q = 1
-        // Q^2 - Rr^2 and 4 - Q^2 at ts, from the edge's float-float
-        // differences and ts^2 as an exact product
-        const emq::ff ts2 = emq::ff_two_prod(ts, ts);
-        const emq::ff es = emq::ff_add(ref1 ? c1x : ccx, ts2);
-        const emq::ff c4s = emq::ff_add(c4x, emq::ff_neg(ts2));
-        q.ts[sl][lane] = ts;
-        q.hl[sl][lane] = 0.5f * len / (float)m;
-        q.A[sl][lane] = A;
-        q.B2[sl][lane] = B2;
-        q.c4s[sl][lane] = c4s.hi + c4s.lo;
-        q.es[sl][lane] = es.hi + es.lo;
-        q.Rr[sl][lane] = ref1 ? 1.f : fs.R;
-        q.vv[sl][lane] = ref1 ? 1.f : fs.v;
-        q.add[sl][lane] = ref1 ? fs.C1 : 0.f;
-        q.scale[sl][lane] = sc;
-        q.meta[sl][lane] = m | (piece == 1 ? emq::SEG_PIECE1 : 0) | tflag | (gl4 ? emq::SEG_GL4 : 0);
-    };
-    // piece 1 is |tau| in [ua, b1], piece 2 in [a2, b2]; when both are present
-    // they meet at t1
-    const float ub = ua + du;
-    const float b1 = fminf(ub, t1), a2 = fmaxf(ua, t1), b2 = fminf(ub, t2);
-    const bool has1 = b1 > ua, has2 = b2 > a2;
-    if (has1 || has2) {
-        const float ra = emq::sqrt_nr(fmaf(ua, ua, A * A));
-        // s at ua + o minus s at ua, from the offset o
-        auto ds = [&](float o) {
-            const float b = ua + o;
-            const float rb = emq::sqrt_nr(fmaf(b, b, A * A));
-            return asinhf(__fdividef(o * (ua + b), fmaf(b, ra, ua * rb)));
-        };
-        // offset in s of the end of the quadrature (ub, or Q = 2), and of Q = 1
-        const float d_end = ds(has2 && ub > t2 ? t2 - ua : du);
-        const float d_mid = (has1 && has2) ? ds(t1 - ua) : 0.f;
-        if (has1) push(1, ua, has2 ? d_mid : d_end);
-        if (has2) push(2, a2, d_end - d_mid);
+    const bool ref1 = piece == 2 && fs.R < 1.f;   // difference split at Q = 1
+    // eta^2 = len^2 / r2 chooses the rule (quad32.cuh)
+    const float ts = t.hi, r2 = fmaf(ts, ts, A2), l2 = len * len;
+    const bool six = l2 <= emq::SIX_ETA * emq::SIX_ETA * r2;
+    int m = 1;
+    if (l2 > emq::TWELVE_ETA * emq::TWELVE_ETA * r2) {
+        // m <= 28: A >= 1e-18, tau <= 2
+        const float te = ts + len;
+        const float e = __logf((te + emq::sqrt_nr(fmaf(te, te, A2))) * emq::rcp_a(ts + emq::sqrt_nr(r2)));
+        m = max(1, min(28, (int)ceilf(e * (1.f / emq::SUB_LOG))));
+    }
+    // Q^2 at t, then Q^2 - Rr^2 and 4 - Q^2 there, each a float-float
+    // difference rounded once
+    emq::ff t2 = emq::ff_two_prod(ts, ts);
+    t2.lo = fmaf(2.f * ts, t.lo, t2.lo);
+    const emq::ff Q2 = emq::ff_add(B2, t2);
+    q.ts[sl][lane] = ts;
+    q.len[sl][lane] = len;
+    q.A[sl][lane] = A;
+    q.B2[sl][lane] = B2f;
+    q.c4s[sl][lane] = emq::ff_diff(emq::ff{4.f, 0.f}, Q2);
+    q.es[sl][lane] = emq::ff_diff(Q2, ref1 ? emq::ff{1.f, 0.f} : fs.R2);
+    q.Rr[sl][lane] = ref1 ? 1.f : fs.R;
+    q.vv[sl][lane] = ref1 ? 1.f : fs.v;
+    q.add[sl][lane] = ref1 ? fs.C1 : 0.f;
+    q.scale[sl][lane] = sc;
+    q.meta[sl][lane] = m | (piece == 1 ? emq::SEG_PIECE1 : 0) | (tilde ? emq::SEG_TILDE : 0) | (six ? emq::SEG_SIX : 0);
+}
+
+// Queue the kernel pieces of (D/pi) int over tau in [T0, T1] of one edge, with
+// the signed factor sc; the part beyond 2h is added directly.  The integrand
+// is even in tau, so a range on one side of the foot is taken as [ua, ua + du],
+// ua >= 0.  du is from an accurate difference (the edge length L/h, or |T| for
+// a range that starts at the foot), and so is every segment's length: offsets
+// of the breakpoints from ua, then differences of offsets.  Forming a length
+// as a difference of two tau of size ~1 instead would carry an absolute error
+// of 2^-24, tens of ulps of a short segment (a small face seen from afar).
+// A breakpoint itself may be off by a few ulp: K's pieces agree to fourth
+// order there, and both sides use the same offset.
+// A range across the foot is taken as its two sides.  Most edges yield one
+// segment: the loop runs once for each that the warp's busiest lane has, with
+// the lanes converged.
+__device__ __forceinline__ void mq_edge(SegQueue &q, int lane, int &cnt, emq::ff T0x, emq::ff T1x, float dT, float A,
+                                        emq::ff B2, float sc, const FaceState &fs, bool tilde, emq::ff &acc,
+                                        float &mag)
+{
+    const float A2 = A * A, B2f = fmaxf(B2.hi, A2);
+    const float c1 = emq::ff_diff(emq::ff{1.f, 0.f}, B2), c4 = emq::ff_diff(emq::ff{4.f, 0.f}, B2);
+    const float t1 = c1 > 1e-30f ? c1 * emq::rsqrt_a(c1) : 0.f;
+    const float t2 = c4 > 1e-30f ? c4 * emq::rsqrt_a(c4) : 0.f;
+    const float T0 = T0x.hi, T1 = T1x.hi;
+    const bool foot = T0 < 0.f && T1 > 0.f;
+    const float ua = foot ? 0.f : (T0 >= 0.f ? T0 : -T1), ualo = foot ? 0.f : (T0 >= 0.f ? T0x.lo : -T1x.lo);
+    const float du = foot ? T1 : dT;      // this side, from ua
+    const float xo = foot ? -T0 : 0.f;    // the other side of the foot, from 0
+    const float o1 = t1 - ua, o2 = t2 - ua;
+    // pieces: piece 1 on offsets [0, e1], piece 2 on [s2, e2]
+    const float e1 = fminf(du, o1), s2 = fmaxf(0.f, o1), e2 = fminf(du, o2);
+    // the other side's: piece 1 up to x1, piece 2 from t1 to x2
+    const float x1 = fminf(xo, t1), x2 = fminf(xo, t2);
+    unsigned todo = (e1 > 0.f ? 1u : 0u) | (e2 > s2 ? 2u : 0u) | (x1 > 0.f ? 4u : 0u) | (x2 > t1 ? 8u : 0u);
+    while (todo) {
+        const int k = __ffs(todo) - 1;
+        todo &= todo - 1;
+        // start: ua, ua + s2, 0 or t1
+        emq::ff t = emq::ff_two_sum(k < 2 ? ua : 0.f, k == 1 ? s2 : (k == 3 ? t1 : 0.f));
+        if (k < 2) t.lo += ualo;
+        const float len = k == 0 ? e1 : (k == 1 ? e2 - s2 : (k == 2 ? x1 : x2 - t1));
+        mq_push(q, lane, cnt++, (k & 1) ? 2 : 1, t, len, A, A2, B2f, B2, sc, fs, tilde);
     }
     if (tilde) {   // beyond 2h: K~(Q) = 0, the integrand is -K~(R) >= 0
-        const float a = fmaxf(ua, t2), b = ub;
-        if (b > a) {
-            const float ba = ua >= t2 ? du : du - (t2 - ua);   // b - a from the offsets
-            const emq::ff v = emq::ff_two_prod(sc, -fs.KR * atan2f(ba * A, A * A + a * b));
-            acc = emq::ff_add(acc, v);
+        auto far = [&](float u, float l) {   // tau from u over length l
+            const emq::ff v = emq::ff_two_prod(sc, -fs.KR * emq::angle_q1(l * A, fmaf(u, u + l, A2)));
+            const emq::ff s = emq::ff_two_sum(acc.hi, v.hi);
+            acc.hi = s.hi;
+            acc.lo += s.lo + v.lo;
             mag += fabsf(v.hi);
-        }
+        };
+        if (du > o2) far(fmaxf(ua, t2), o2 > 0.f ? du - o2 : du);
+        if (xo > t2) far(t2, xo - t2);
     }
 }
 
@@ -1098,9 +1098,9 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_map_fp32(int64_t npairs, c
             const emq::ff sd = plane_dist(g);
             inside = inside && !(sd.hi < 0.f);
             const emq::ff D = emq::ff_mul(sd.hi < 0.f ? emq::ff_neg(sd) : sd, ihh);
-            // P in (or within underflow of) the face plane: in the complement
-            // form such a face would carry half of the kernel
-            if (tilde && D.hi < 1e-30f) force = true;
+            // P in (or next to) the face plane: in the complement form such a
+            // face would carry half of the kernel
+            if (tilde && D.hi < 1e-15f) force = true;
             const bool beyond = D.hi > 2.f || (D.hi == 2.f && D.lo >= 0.f);
             if (!(sd.hi == 0.f || (tilde && beyond))) {
                 // reference distance to the polygon (FP32)
@@ -1117,15 +1117,12 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_map_fp32(int64_t npairs, c
                     rho2 = fminf(rho2, a * a + tc * tc);
                 }
                 const float rr2 = inpoly ? 0.f : rho2;
-                const emq::ff D2 = emq::ff_mul(D, D);
-                const emq::ff R2 = emq::ff_add(D2, emq::ff{rr2, 0.f});
-                const bool far = R2.hi > 4.f || (R2.hi == 4.f && R2.lo >= 0.f);
+                fs.D2 = emq::ff_mul(D, D);
+                fs.R2 = emq::ff_add(fs.D2, emq::ff{rr2, 0.f});
+                const bool far = fs.R2.hi > 4.f || (fs.R2.hi == 4.f && fs.R2.lo >= 0.f);
                 if (!(tilde && far)) {   // else the polygon lies entirely beyond 2h
-                    fs.rr2 = rr2;
-                    fs.dm1 = emq::ff_add(D2, emq::ff{-1.f, 0.f});
-                    fs.d4 = emq::ff_add(emq::ff{4.f, 0.f}, emq::ff_neg(D2));
-                    fs.Df = D.hi + D.lo;
-                    face_consts(R2, tilde, fs);
+                    fs.Df = D.hi;
+                    face_consts(fs.R2, tilde, fs);
                     fs.sign = sd.hi > 0.f ? 1.f : -1.f;
                     e0 = g0;
                     ne = (int)(g1 - g0);
@@ -1135,7 +1132,7 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_map_fp32(int64_t npairs, c
         for (int ei = 0; last ? ei == 0 : __any_sync(FULL_MASK, ei < ne); ++ei) {
             if (ei < ne) {
                 // edge geometry in float-float (see quad32.cuh): A, T0, T1 and
-                // B^2 - 1, 4 - B^2, A^2 - rho^2 each rounded once to FP32
+                // B^2, each rounded once to FP32 where it is used so
                 const EdgeF H = edge_f[e0 + ei], Lo = edge_fl[e0 + ei];
                 const emq::ff ah = emq::ff_offset_dot(H.cm, Lo.cm, H.mx, Lo.mx, H.my, Lo.my, H.mz, Lo.mz, rxx, ryy, rzz);
                 const emq::ff a = emq::ff_mul(ah, ihh);
@@ -1144,29 +1141,14 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_map_fp32(int64_t npairs, c
                     const emq::ff t0 = emq::ff_mul(th, ihh);
                     const emq::ff lh = emq::ff_mul(emq::ff{H.L, Lo.L}, ihh);   // L/h
                     const emq::ff t1 = emq::ff_add(t0, lh);
-                    const emq::ff a2 = emq::ff_mul(a, a);
-                    // A below 1e-30 h changes the integral by ~1e-30 relative and would
-                    // make the s-range of the sinh substitution unbounded
-                    const float A = fmaxf(fabsf(a.hi + a.lo), 1e-30f), T0 = t0.hi + t0.lo, T1 = t1.hi + t1.lo;
-                    const float dT = lh.hi + lh.lo;   // T1 - T0 = L/h, from the edge length itself
-                    const float B2f = fs.Df * fs.Df + A * A;
-                    const emq::ff c1x = emq::ff_add(fs.dm1, a2), c4x = emq::ff_add(fs.d4, emq::ff_neg(a2));
-                    const emq::ff ccx = emq::ff_add(a2, emq::ff{-fs.rr2, 0.f});
-
-                    // signed factor: D/pi, face orientation, side of the edge line, direction along it
-                    const float base = fs.sign * (a.hi > 0.f ? 1.f : -1.f) * fs.Df * 0.31830988618379067154f;
-                    // the edge's |tau| ranges: one if T0 and T1 lie on one side of
-                    // the foot F, else [0, |T0|] and [0, |T1|]
-                    const float u0 = fabsf(T0), u1 = fabsf(T1);
-                    const bool one_side = (T0 >= 0.f && T1 >= 0.f) || (T0 <= 0.f && T1 <= 0.f);
-                    const float sc = (one_side ? T1 >= T0 : T1 > T0) ? base : -base;
-#pragma unroll 1
-                    for (int part = 0; part < (one_side ? 1 : 2); ++part) {
-                        // one side: [min |T|, min |T| + L/h]; else [0, |T0|] and [0, |T1|]
-                        const float ua = one_side ? fminf(u0, u1) : 0.f;
-                        const float du = one_side ? dT : (part ? u1 : u0);
-                        mq_push_g(q, lane, cnt, ua, du, A, B2f, c1x, c4x, ccx, sc, fs, tilde, acc_far, mag_far);
-                    }
+                    // A below 1e-18 h changes the integral by ~1e-18 relative and would
+                    // leave A^2 below FP32's normal range
+                    const float A = fmaxf(fabsf(a.hi), 1e-18f);
+                    // signed factor: D/pi, face orientation, side of the edge line
+                    // (T1 >= T0: the edge runs along its direction)
+                    const float sc = fs.sign * (a.hi > 0.f ? 1.f : -1.f) * fs.Df * 0.31830988618379067154f;
+                    mq_edge(q, lane, cnt, t0, t1, lh.hi, A, emq::ff_add(fs.D2, emq::ff_mul(a, a)), sc, fs, tilde,
+                            acc_far, mag_far);
                 }
             }
             // an edge queues at most four segments

@@ -1,10 +1,11 @@
-// The FP64 primitives of the closed form (csrc/fp64.cuh) against a host
-// reference in long double: per function its name, its largest error in units
-// of its bound, and the sample count.  The bounds sum the roundings:
+// The FP64 primitives of the closed form (csrc/fp64.cuh) and the FP32 pass's
+// angle (csrc/quad32.cuh) against a host reference in long double: per function
+// its name, its largest error in units of its bound, and the sample count.  The bounds sum the roundings:
 //   sqrt64     2^-52 relative;
 //   log_ratio  4e-16 + 2.3e-16 |log| (num s, the table's log, the FP32 tail of
 //              the series, and the sum's own rounding);
-//   angle64    6e-16 (the table's angle, the rounded pi, two sums of size <= pi).
+//   angle64    6e-16 (the table's angle, the rounded pi, two sums of size <= pi);
+//   angle_q1   4 x 2^-24 relative (the difference, the reciprocal, the product, the sum).
 // Built and run by tests/test_gpu_fp64_primitives.py.
 #include <cmath>
 #include <cstdio>
@@ -14,8 +15,9 @@
 #include <cuda_runtime.h>
 
 #include "fp64.cuh"
+#include "quad32.cuh"
 
-__global__ void eval(int n, const double *a, const double *b, double *s, double *l, double *t)
+__global__ void eval(int n, const double *a, const double *b, double *s, double *l, double *t, double *g)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -23,6 +25,8 @@ __global__ void eval(int n, const double *a, const double *b, double *s, double 
     s[i] = em::sqrt64(p);
     l[i] = p > 0.0 && q > 0.0 ? em::log_ratio(p, q, em::kLogTab) : 0.0;
     t[i] = em::angle64(a[i], b[i], em::kAtanTab);
+    const float x = (float)q, y = (float)p;
+    g[i] = x > 1e-30f && x < 1e30f && y < 1e30f ? (double)emq::angle_q1(y, x) : 0.0;
 }
 
 int main()
@@ -47,17 +51,17 @@ int main()
     for (double u : edge)
         for (double v : edge) add(u, v);
     const int n = (int)a.size();
-    double *d[5];
-    std::vector<double> r[3];
+    double *d[6];
+    std::vector<double> r[4];
     for (auto &p : d) cudaMalloc(&p, n * sizeof(double));
     cudaMemcpy(d[0], a.data(), n * sizeof(double), cudaMemcpyHostToDevice);
     cudaMemcpy(d[1], b.data(), n * sizeof(double), cudaMemcpyHostToDevice);
-    eval<<<(n + 255) / 256, 256>>>(n, d[0], d[1], d[2], d[3], d[4]);
-    for (int k = 0; k < 3; ++k) {
+    eval<<<(n + 255) / 256, 256>>>(n, d[0], d[1], d[2], d[3], d[4], d[5]);
+    for (int k = 0; k < 4; ++k) {
         r[k].resize(n);
         if (cudaMemcpy(r[k].data(), d[2 + k], n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess) return 1;
     }
-    double worst[3] = {0, 0, 0};
+    double worst[4] = {0, 0, 0, 0};
     for (int i = 0; i < n; ++i) {
         const double p = std::fabs(a[i]), q = std::fabs(b[i]);
         const long double s = sqrtl((long double)p);
@@ -69,9 +73,14 @@ int main()
         // the zero vector's angle is 0 whatever its signs
         const long double t = p == 0.0 && q == 0.0 ? 0.0L : atan2l((long double)a[i], (long double)b[i]);
         worst[2] = std::fmax(worst[2], (double)fabsl(r[2][i] - t) / 6e-16);
+        const float x = (float)q, y = (float)p;
+        if (x > 1e-30f && x < 1e30f && y > 1e-30f && y < 1e30f && y / x > 1e-30f) {
+            const long double g = atan2l((long double)y, (long double)x);
+            worst[3] = std::fmax(worst[3], (double)(fabsl(r[3][i] - g) / g) / 0x1p-22);
+        }
         for (auto &v : r)
             if (!std::isfinite(v[i])) worst[2] = 1e9;
     }
-    std::printf("sqrt64 %g %d\nlog_ratio %g %d\nangle64 %g %d\n", worst[0], n, worst[1], n, worst[2], n);
+    std::printf("sqrt64 %g %d\nlog_ratio %g %d\nangle64 %g %d\nangle_q1 %g %d\n", worst[0], n, worst[1], n, worst[2], n, worst[3], n);
     return 0;
 }

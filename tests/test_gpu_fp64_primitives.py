@@ -1,5 +1,5 @@
 """The FP64 closed form's own square root, logarithm and angle (csrc/fp64.cuh)
-against a long double host reference, within the bounds derived beside their
+and the FP32 pass's angle (csrc/quad32.cuh) against a long double host reference, within the bounds derived beside their
 check (gpu_fp64_check.cu): random arguments of every sign, 120 binades of
 range, ratios near 1, both sides of the tables' breakpoints, zeros."""
 import os
@@ -26,7 +26,7 @@ def worst():
     return {p[0]: (float(p[1]), int(p[2])) for p in (line.split() for line in out.strip().splitlines())}
 
 
-@pytest.mark.parametrize("name", ["sqrt64", "log_ratio", "angle64"])
+@pytest.mark.parametrize("name", ["sqrt64", "log_ratio", "angle64", "angle_q1"])
 def test_within_bound(worst, name):
     w, n = worst[name]
     assert n > 500_000 and w <= 1.0, w
