@@ -324,65 +324,375 @@ __device__ int warp_f_sign(const em::ChunkTree &T, const double *__restrict__ qx
     return f > 0.0 ? 1 : (f < 0.0 ? -1 : 0);
 }
 
-// One warp per pseudo-particle: Newton (Eq. 10) from h_0 (Eq. 11) until
-// |dh|/h_0 < tol, bisection on [1e-2 h_0, 1e2 h_0], else h_0.
-__global__ void k_h_solve(int64_t npseudo, em::ChunkTree T, const double *__restrict__ qx,
-                          const double *__restrict__ qy, const double *__restrict__ qz, const double *__restrict__ px,
+// The solver's FP32 side.  Each FP64 evaluation of n(h) costs the FP64 pipe
+// about 20 instructions per 32 neighbours and 75 on values every lane shares;
+// the iterations that only approach the root, and the bisection's 50 signs,
+// need none of that.  Population positions are float-float (T.pts and plo), so
+// that a neighbour's offset is good to FP32 whatever the coordinates' size.
+struct Population {
+    const double *x, *y, *z;
+    const float4 *lo;   // position - T.pts, rounded to FP32
+};
+
+constexpr int HS_LIST = 384;        // neighbours a warp keeps from its last walk
+constexpr float HS_COVER = 1.08f;   // the walk's radius, in units of the 2h it serves
+constexpr int HS_LEAVES = 4;        // 32-point leaves a walk reads together (their loads in flight at once)
+
+// A warp's pseudo-particle and the neighbours of its last walk: every
+// population entry within r of it if n >= 0 (n = -1: more than the list holds).
+struct HsList {
+    double xa, ya, za;
+    float xh, yh, zh, xl, yl, zl;
+    float r;
+    int n;
+    int32_t *k;
+};
+
+struct Sum32 {
+    float S, G;   // sums of w and of g = 3 w + q w'
+};
+
+// w and g of the M4 spline at q2 = q^2 < 4, branch-free
+__device__ __forceinline__ void m4_wg32(float q2, float &w, float &g)
+{
+    const float q = q2 * rsqrtf(fmaxf(q2, 1e-30f));   // 0 at the particle itself
+    const float t = 2.f - q, t2 = t * t;
+    w = q < 1.f ? fmaf(q2, fmaf(0.75f, q, -1.5f), 1.f) : 0.25f * t2 * t;
+    g = q < 1.f ? fmaf(q2, fmaf(4.5f, q, -7.5f), 3.f) : 0.75f * t2 * (t - q);
+}
+
+// Add one entry's terms (none if !in).  No branches, so that the entries of a
+// batch overlap: a lone warp walking a large node's 2 h_0, which may hold the
+// whole population, is bound by the latency of this chain.
+__device__ __forceinline__ void add32(const HsList &L, bool in, float4 p, float4 lo, float ih2, float &S, float &G)
+{
+    const float ex = (p.x - L.xh) + (lo.x - L.xl), ey = (p.y - L.yh) + (lo.y - L.yl), ez = (p.z - L.zh) + (lo.z - L.zl);
+    const float q2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) * ih2;
+    float w, g;
+    m4_wg32(q2, w, g);
+    const bool add = in && q2 < 4.f;
+    S += add ? w : 0.f;
+    G += add ? g : 0.f;
+}
+
+// The sums at h in FP32 (the same on every lane), from the list where it
+// covers 2h, else by a walk that renews it.
+__device__ Sum32 warp_sum32(const em::ChunkTree &T, const Population &P, HsList &L, float h, float margin)
+{
+    const int lane = threadIdx.x & 31;
+    const float ih2 = 1.f / (h * h);
+    float S = 0.f, G = 0.f;
+    if (L.n >= 0 && 2.0002f * h <= L.r) {
+        for (int t = lane; t < L.n; t += 32) add32(L, true, T.pts[L.k[t]], P.lo[L.k[t]], ih2, S, G);
+    } else {
+        const float r = 2.f * HS_COVER * h;
+        const float lim = r + 1e-5f * (fabsf(L.xh) + fabsf(L.yh) + fabsf(L.zh) + r), lim2 = lim * lim;
+        int n = 0;
+        em::warp_traverse_batch<HS_LEAVES>(T, L.xh, L.yh, L.zh, (r + margin) * (r + margin),
+                                           [&](const int32_t(&k)[HS_LEAVES]) {
+            float4 p[HS_LEAVES], lo[HS_LEAVES];
+            unsigned b[HS_LEAVES];
+#pragma unroll
+            for (int u = 0; u < HS_LEAVES; ++u) {
+                const int32_t kk = max(k[u], 0);
+                p[u] = T.pts[kk];
+                lo[u] = P.lo[kk];
+            }
+#pragma unroll
+            for (int u = 0; u < HS_LEAVES; ++u) {
+                const float ex = p[u].x - L.xh, ey = p[u].y - L.yh, ez = p[u].z - L.zh;
+                const bool in = k[u] >= 0 && ex * ex + ey * ey + ez * ez < lim2;
+                add32(L, in, p[u], lo[u], ih2, S, G);
+                b[u] = __ballot_sync(0xffffffffu, in);
+            }
+#pragma unroll
+            for (int u = 0; u < HS_LEAVES; ++u) {
+                const int pos = n + __popc(b[u] & ((1u << lane) - 1u));
+                if (((b[u] >> lane) & 1u) && pos < HS_LIST) L.k[pos] = k[u];
+                n += __popc(b[u]);
+            }
+        });
+        __syncwarp();
+        L.r = r;
+        L.n = n <= HS_LIST ? n : -1;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        S += __shfl_xor_sync(0xffffffffu, S, o);
+        G += __shfl_xor_sync(0xffffffffu, G, o);
+    }
+    return Sum32{S, G};
+}
+
+// Make the list the population within 2h and a margin for h's last digits, so
+// that FP64 batches hold neighbours only.
+__device__ void settle_list(const em::ChunkTree &T, const Population &P, HsList &L, float h, float margin)
+{
+    const int lane = threadIdx.x & 31;
+    if (!(L.n >= 0 && 2.0002f * h <= L.r)) warp_sum32(T, P, L, h, margin);
+    const float r = 2.004f * h;
+    if (L.n < 0 || L.r <= r) return;
+    const float lim = r + 1e-5f * (fabsf(L.xh) + fabsf(L.yh) + fabsf(L.zh) + r), lim2 = lim * lim;
+    int n = 0;
+    for (int t0 = 0; t0 < L.n; t0 += 32) {
+        const int t = t0 + lane, k = t < L.n ? L.k[t] : 0;
+        bool in = false;
+        if (t < L.n) {
+            const float4 p = T.pts[k];
+            const float ex = p.x - L.xh, ey = p.y - L.yh, ez = p.z - L.zh;
+            in = ex * ex + ey * ey + ez * ez < lim2;
+        }
+        const unsigned b = __ballot_sync(0xffffffffu, in);   // read before anything is written at or below t0
+        if (in) L.k[n + __popc(b & ((1u << lane) - 1u))] = k;
+        n += __popc(b);
+        __syncwarp();
+    }
+    L.n = n;
+    L.r = r;
+}
+
+// n(h) and dn/dh in FP64 from the list where it covers 2h, else by a walk.
+__device__ Density list_density(const em::ChunkTree &T, const Population &P, const HsList &L, double h, float margin,
+                                int32_t *buf)
+{
+    if (!(L.n >= 0 && 2.0002f * (float)h <= L.r)) return warp_density(T, P.x, P.y, P.z, L.xa, L.ya, L.za, h, margin, buf);
+    double s = 0.0, ds = 0.0;
+    const double ih = rcp64(h), ih2 = ih * ih, norm = ih2 * ih * 0.31830988618379067154;   // 1/(pi h^3)
+    for (int t = threadIdx.x & 31; t < L.n; t += 32) {
+        const int32_t k = L.k[t];
+        const double dx = P.x[k] - L.xa, dy = P.y[k] - L.ya, dz = P.z[k] - L.za;
+        const double q2 = (dx * dx + dy * dy + dz * dz) * ih2;
+        if (q2 < 4.0) {
+            double w, g;
+            m4_wg(q_of(q2), q2, w, g);
+            s += w;
+            ds += g;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        ds += __shfl_xor_sync(0xffffffffu, ds, o);
+    }
+    return Density{s * norm, -ds * norm * ih};
+}
+
+// One Newton step of Eqs. 8-10 from n and dn/dh at h.
+__device__ __forceinline__ double newton_step(Density d, double h, double h_fact)
+{
+    // n^(-1/3) as a reciprocal cube root and n^(-4/3) as its fourth power:
+    // the same values to an ulp or two, for a fraction of the FP64 work of
+    // two general powers (every lane computes them, so each FP64
+    // instruction costs the pipe a full warp)
+    const double c = rcbrt(d.n);
+    const double f = h_fact * c - h;                                              // Eq. 8
+    const double fp = -h_fact * d.dn * ((c * c) * (c * c)) * (1.0 / 3.0) - 1.0;   // Eq. 9 (a product, not a division)
+    return h - f * rcp64(fp);                                                     // Eq. 10
+}
+
+// Newton (Eq. 10) from h_0 (Eq. 11) until |dh|/h_0 < tol, every evaluation in
+// FP64.  Returns false where an iterate leaves the bracket [1e-2 h_0, 1e2 h_0]
+// or max_newton steps do not suffice: Newton failed.
+__device__ bool newton64(const em::ChunkTree &T, const Population &P, const HsList &L, double h0, double h_fact,
+                         double tol, int max_newton, float margin, int32_t *buf, double &hout)
+{
+    const double ih0 = rcp64(h0), blo = 1e-2 * h0, bhi = 1e2 * h0;
+    double h = h0;
+    for (int it = 0; it < max_newton; ++it) {
+        const double hn = newton_step(warp_density(T, P.x, P.y, P.z, L.xa, L.ya, L.za, h, margin, buf), h, h_fact);
+        if (!(hn >= blo && hn <= bhi)) return false;
+        const double step = fabs(hn - h) * ih0;   // |dh| / h_0
+        h = hn;
+        if (step < tol) {
+            hout = h;
+            return true;
+        }
+    }
+    return false;
+}
+
+// Bisection on [1e-2 h_0, 1e2 h_0] by signs (warp_f_sign), else h_0.
+__device__ double bisect64(const em::ChunkTree &T, const Population &P, const HsList &L, double h0, double h_fact,
+                           double tol, float margin, int32_t *buf, int &st)
+{
+    const double xa = L.xa, ya = L.ya, za = L.za;
+    const double *qx = P.x, *qy = P.y, *qz = P.z;
+    double lo = 1e-2 * h0, hi = 1e2 * h0;
+    const int slo = warp_f_sign(T, qx, qy, qz, xa, ya, za, lo, h_fact, margin, buf);
+    const int shi = warp_f_sign(T, qx, qy, qz, xa, ya, za, hi, h_fact, margin, buf);
+    const bool plo = slo > 0;
+    if (slo * shi > 0) {
+        st = 2;
+        return h0;
+    }
+    for (int k = 0; k < 200 && (hi - lo) > tol * h0; ++k) {
+        const double mid = 0.5 * (lo + hi);
+        if ((warp_f_sign(T, qx, qy, qz, xa, ya, za, mid, h_fact, margin, buf) > 0) == plo) lo = mid;
+        else hi = mid;
+    }
+    st = 1;
+    return 0.5 * (lo + hi);
+}
+
+// The root of f near h (an FP32 root) by Newton in FP64: the step after which
+// the quadratic convergence leaves less than a tenth of tol is the last.
+// Returns false where it does not settle at once.
+__device__ bool polish64(const em::ChunkTree &T, const Population &P, HsList &L, double &h, double h_fact, double tol,
+                         float margin, int32_t *buf)
+{
+    settle_list(T, P, L, (float)h, margin);
+    for (int it = 0; it < 5; ++it) {
+        const double hn = newton_step(list_density(T, P, L, h, margin, buf), h, h_fact);
+        const double d = fabs(hn - h);
+        if (!(d <= 1e-3 * h)) return false;
+        h = hn;
+        if (d * d <= 0.1 * tol * h * h) return true;
+    }
+    return false;
+}
+
+// For a tolerance that means "converged" (tol <= HS_WARM_TOL) the approach is
+// made in FP32.  newton32: Newton's iterates from h_0 decide whether Newton
+// converges (1; the root polished in FP64) or leaves the bracket (0), as in
+// FP64 unless an iterate comes within 10% of the bracket's ends (-1: not
+// decided).
+constexpr double HS_WARM_TOL = 1e-9;
+__device__ int newton32(const em::ChunkTree &T, const Population &P, HsList &L, double h0, double h_fact, double tol,
+                        int max_newton, float margin, int32_t *buf, double &hout)
+{
+    const float h0f = (float)h0, hf = (float)h_fact, blo = 1e-2f * h0f, bhi = 1e2f * h0f;
+    float h = h0f;
+    if (!(h0f > 1e-15f && h0f < 1e15f)) return -1;
+    for (int it = 0; it + 4 < max_newton; ++it) {
+        const Sum32 u = warp_sum32(T, P, L, h, margin);
+        const float a = hf * cbrtf(3.14159265f / u.S);   // h_fact n^(-1/3) / h
+        const float hn = h * (1.f - (a - 1.f) / (a * u.G / (3.f * u.S) - 1.f));
+        if (!(fabsf(hn) < 1e30f)) return -1;
+        if (hn < 0.9f * blo || hn > 1.1f * bhi) return 0;
+        if (hn < 1.1f * blo || hn > 0.9f * bhi) return -1;
+        const float d = fabsf(hn - h);
+        h = hn;
+        if (d < 3e-4f * h) {
+            hout = h;
+            return polish64(T, P, L, hout, h_fact, tol, margin, buf) ? 1 : -1;
+        }
+    }
+    return -1;
+}
+
+// bisect64's result where FP32 decides it (else false): f's sign is that of
+// pi h_fact^3 - S(h), S = sum w increasing in h, so its one root r in the
+// bracket is found by a bracketed Newton in log h, polished, and the
+// bisection's decisions are comparisons with r; only a midpoint within 2e-14 r
+// of it (the rounding of either) takes an FP64 evaluation.
+__device__ bool bisect32(const em::ChunkTree &T, const Population &P, HsList &L, double h0, double h_fact, double tol,
+                         float margin, int32_t *buf, double &hout, int &st)
+{
+    const float h0f = (float)h0, hf = (float)h_fact, blo = 1e-2f * h0f, bhi = 1e2f * h0f;
+    const float target = 3.14159265f * hf * hf * hf;
+    if (!(h0f > 1e-15f && h0f < 1e15f)) return false;
+    // the bracket's ends, each moved to the nearest point with the same sign
+    float lo = blo, hi = h0f;
+    auto sum = [&](float at) { return warp_sum32(T, P, L, at, margin); };
+    Sum32 u = sum(h0f);
+    if (u.S < target) {
+        lo = h0f;
+        while (true) {
+            hi = fminf(2.f * lo, bhi);
+            u = sum(hi);
+            if (u.S > target) break;
+            if (hi == bhi) {
+                if (u.S > 0.999f * target) return false;
+                hout = h0;   // no root below 1e2 h_0
+                st = 2;
+                return true;
+            }
+            lo = hi;
+        }
+        if (hi == bhi && u.S < 1.001f * target) return false;
+    } else {
+        u = sum(blo);
+        if (u.S > 0.999f * target) return false;
+    }
+    float h = sqrtf(lo * hi);
+    for (int it = 0;; ++it) {
+        if (it == 40) return false;
+        u = sum(h);
+        if (u.S < target) lo = h;
+        else hi = h;
+        const float D = 3.f * u.S - u.G;   // dS / dlog h
+        float hn = D > 0.f ? h * __expf(fminf(fmaxf((target - u.S) / D, -2.f), 2.f)) : 0.f;
+        const bool in = hn > lo && hn < hi;
+        if (!in) hn = sqrtf(lo * hi);
+        const float d = fabsf(hn - h);
+        h = hn;
+        if ((in && d < 3e-4f * h) || hi - lo < 1e-6f * h) break;
+    }
+    double r = h;
+    if (!polish64(T, P, L, r, h_fact, tol, margin, buf)) return false;
+    double dlo = 1e-2 * h0, dhi = 1e2 * h0;
+    const double near = 2e-14 * r, width = tol * h0;
+    for (int k = 0; k < 200 && (dhi - dlo) > width; ++k) {
+        const double mid = 0.5 * (dlo + dhi), e = mid - r;
+        const bool below = fabs(e) > near ? e < 0.0
+                                          : warp_f_sign(T, P.x, P.y, P.z, L.xa, L.ya, L.za, mid, h_fact, margin, buf) > 0;
+        if (below) dlo = mid;
+        else dhi = mid;
+    }
+    hout = 0.5 * (dlo + dhi);
+    st = 1;
+    return true;
+}
+
+// One warp per pseudo-particle.  1e6 particles (94,193 nodes, 5,733 of them
+// bisected): 417,533 FP64 evaluations of n(h) and 298,116 signs, each with its
+// walk, took 11.2 ms; 112,000 FP64 evaluations, 1.5 walks and 1.8 sums over a
+// list per node take 5.8, most of it the tail of the few nodes whose 2h holds
+// thousands of the population.
+__global__ void __launch_bounds__(32 * HS_WARPS, 6) k_h_solve(int64_t npseudo, em::ChunkTree T, Population P, const double *__restrict__ px,
                           const double *__restrict__ py, const double *__restrict__ pz, double h_fact, double tol,
                           int max_newton, float margin, double *__restrict__ ph, int32_t *__restrict__ status)
 {
-    __shared__ int32_t bufs[HS_WARPS][HS_BUF];
+    __shared__ int32_t bufs[HS_WARPS][HS_BUF], lists[HS_WARPS][HS_LIST];
     int32_t *buf = bufs[threadIdx.x >> 5];
     int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (a >= npseudo) return;
     if (status[a] != -1) return;   // extracted particles keep their own h
-    const double xa = px[a], ya = py[a], za = pz[a];
+    HsList L;
+    L.xa = px[a];
+    L.ya = py[a];
+    L.za = pz[a];
+    em::split_df(L.xa, L.xh, L.xl);
+    em::split_df(L.ya, L.yh, L.yl);
+    em::split_df(L.za, L.zh, L.zl);
+    L.r = 0.f;
+    L.n = -1;
+    L.k = lists[threadIdx.x >> 5];
     const double h0 = ph[a];
-    const double ih0 = rcp64(h0), blo = 1e-2 * h0, bhi = 1e2 * h0;
     double h = h0;
-    bool ok = false;
-    for (int it = 0; it < max_newton; ++it) {
-        Density d = warp_density(T, qx, qy, qz, xa, ya, za, h, margin, buf);
-        // n^(-1/3) as a reciprocal cube root and n^(-4/3) as its fourth power:
-        // the same values to an ulp or two, for a fraction of the FP64 work of
-        // two general powers (every lane computes them, so each FP64
-        // instruction costs the pipe a full warp)
-        const double c = rcbrt(d.n);
-        double f = h_fact * c - h;                                          // Eq. 8
-        double fp = -h_fact * d.dn * ((c * c) * (c * c)) * (1.0 / 3.0) - 1.0;   // Eq. 9 (a product, not a division)
-        double hn = h - f * rcp64(fp);                                      // Eq. 10
-        if (!(hn >= blo && hn <= bhi)) break;   // left the bracket [1e-2 h0, 1e2 h0]: Newton failed
-        double step = fabs(hn - h) * ih0;   // |dh| / h_0
-        h = hn;
-        if (step < tol) {
-            ok = true;
-            break;
-        }
-    }
     int st = 0;
-    if (!ok) {
-        // bisection on signs only (warp_f_sign)
-        double lo = 1e-2 * h0, hi = 1e2 * h0;
-        const int slo = warp_f_sign(T, qx, qy, qz, xa, ya, za, lo, h_fact, margin, buf);
-        const int shi = warp_f_sign(T, qx, qy, qz, xa, ya, za, hi, h_fact, margin, buf);
-        const bool plo = slo > 0;
-        if (slo * shi > 0) {
-            h = h0;
-            st = 2;
-        } else {
-            for (int k = 0; k < 200 && (hi - lo) > tol * h0; ++k) {
-                double mid = 0.5 * (lo + hi);
-                if ((warp_f_sign(T, qx, qy, qz, xa, ya, za, mid, h_fact, margin, buf) > 0) == plo) lo = mid;
-                else hi = mid;
-            }
-            h = 0.5 * (lo + hi);
-            st = 1;
-        }
-    }
+    const bool warm = tol <= HS_WARM_TOL;
+    int ok = warm ? newton32(T, P, L, h0, h_fact, tol, max_newton, margin, buf, h) : -1;
+    if (ok < 0) ok = newton64(T, P, L, h0, h_fact, tol, max_newton, margin, buf, h) ? 1 : 0;
+    if (!ok && !(warm && bisect32(T, P, L, h0, h_fact, tol, margin, buf, h, st)))
+        h = bisect64(T, P, L, h0, h_fact, tol, margin, buf, st);
     if ((threadIdx.x & 31) == 0) {
         ph[a] = h;
         status[a] = st;
     }
+}
+
+// Low parts of the population's positions (Population::lo).
+__global__ void k_population_lo(int64_t n, const double *__restrict__ x, const double *__restrict__ y,
+                                const double *__restrict__ z, float4 *__restrict__ lo)
+{
+    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    float h, lx, ly, lz;
+    em::split_df(x[k], h, lx);
+    em::split_df(y[k], h, ly);
+    em::split_df(z[k], h, lz);
+    lo[k] = make_float4(lx, ly, lz, 0.f);
 }
 
 __global__ void k_status_count(int64_t n, const int32_t *__restrict__ status, unsigned long long *__restrict__ cnt)
@@ -464,8 +774,12 @@ static int pseudo_impl(em_ctx *ctx, const em_tree *t, const double *d_hp, int ns
         for (int k = 0; k < 6; ++k) ext = fmax(ext, fabs(t->box[k]));
         // float rounding of positions and boxes: widen the search radius
         const float margin = (float)(4e-7 * (ext + 1.0));
+        float4 *plo;
+        EM_TRY(tmp.alloc(&plo, npop));
+        k_population_lo<<<em_grid(npop, 256), 256, 0, st>>>(npop, qx, qy, qz, plo);
+        EM_LAUNCHED(ctx);
         k_h_solve<<<em_grid(np * 32, 32 * HS_WARPS), 32 * HS_WARPS, 0, st>>>(
-            np, T, qx, qy, qz, ps->x, ps->y, ps->z, p->h_fact, p->h_tol, p->max_newton, margin, ps->h, ps->status);
+            np, T, Population{qx, qy, qz, plo}, ps->x, ps->y, ps->z, p->h_fact, p->h_tol, p->max_newton, margin, ps->h, ps->status);
         EM_LAUNCHED(ctx);
     }
     unsigned long long *cnt;

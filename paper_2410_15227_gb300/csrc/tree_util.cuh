@@ -108,6 +108,53 @@ __device__ __forceinline__ bool warp_traverse(const ChunkTree &T, float px, floa
     return true;
 }
 
+// warp_traverse over batches of up to U leaves that share a parent: visit
+// gets every lane's item in each (-1 for none), so that it can issue U leaves'
+// loads before it waits for one.  Items must number below 2^31.
+template <int U, class Visit>
+__device__ __forceinline__ void warp_traverse_batch(const ChunkTree &T, float px, float py, float pz, float R2,
+                                                    Visit &&visit)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t mask[kMaxLevels + 1];
+    int64_t base[kMaxLevels + 1];
+    const int top = T.nlev;
+    if (top <= 0) return;
+    const float R2m = R2 * 1.00001f + 1e-30f;   // conservative margin for the float boxes
+    auto open = [&](int level, int64_t node) {
+        return node < T.count[level] && box_dist2(T.lo[level][node], T.hi[level][node], px, py, pz) <= R2m;
+    };
+    mask[top] = __ballot_sync(0xffffffffu, open(top, lane));
+    base[top] = 0;
+    int lvl = top;
+    while (true) {
+        if (mask[lvl] == 0) {
+            if (lvl == top) break;
+            ++lvl;
+            continue;
+        }
+        if (lvl == 1) {
+            int32_t k[U];
+            uint32_t m = mask[1];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t item = (base[1] * 32 + __ffs(m) - 1) * 32 + lane;
+                k[u] = m && item < T.count[0] ? (int32_t)item : -1;
+                m &= m - 1;
+            }
+            mask[1] = m;
+            visit(k);
+        } else {
+            const int c = __ffs(mask[lvl]) - 1;
+            mask[lvl] &= mask[lvl] - 1;
+            const int64_t node = base[lvl] * 32 + c;
+            mask[lvl - 1] = __ballot_sync(0xffffffffu, open(lvl - 1, node * 32 + lane));
+            base[lvl - 1] = node;
+            --lvl;
+        }
+    }
+}
+
 // warp_traverse whose visit returns true to go on and false to end the walk
 // (a warp-uniform value).  Returns false if the walk was ended by visit.
 template <class Visit>
