@@ -13,6 +13,7 @@
 // 32-ary box hierarchy over the solver population (selected nodes plus the
 // leaves of extracted particles, Morton order) with radius 2h, so the sum
 // n(h) = sum_b W(r_ab, h) always covers every neighbour of the current h.
+#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
@@ -227,103 +228,6 @@ __device__ __forceinline__ void m4_wg(double q, double q2, double &w, double &g)
     }
 }
 
-// n(h) and dn/dh for the pseudo-particle at (xa, ya, za), summed over the
-// population inside 2h; the result is identical on all lanes.
-__device__ Density warp_density(const em::ChunkTree &T, const double *__restrict__ qx,
-                                const double *__restrict__ qy, const double *__restrict__ qz, double xa, double ya,
-                                double za, double h, float margin, int32_t *buf)
-{
-    const int lane = threadIdx.x & 31;
-    double s = 0.0, ds = 0.0;
-    const double ih = rcp64(h);
-    const double norm = ih * ih * ih * 0.31830988618379067154;   // 1/(pi h^3)
-    float R = (float)(2.0 * h) + margin;
-    const float xaf = (float)xa, yaf = (float)ya, zaf = (float)za, h2f = (float)(2.0 * h);
-    const float lim = h2f + 1e-5f * (fabsf(xaf) + fabsf(yaf) + fabsf(zaf) + h2f);
-    const float lim2 = lim * lim;
-    // sums of w and of g = 3w + q w' over the neighbours; n = norm sum w,
-    // dn/dh = -norm sum g / h
-    const double ih2 = ih * ih;
-    auto sum_one = [&](int64_t k) {
-        const double dx = qx[k] - xa, dy = qy[k] - ya, dz = qz[k] - za;
-        const double q2 = (dx * dx + dy * dy + dz * dz) * ih2;
-        if (q2 < 4.0) {
-            double w, g;
-            m4_wg(q_of(q2), q2, w, g);
-            s += w;
-            ds += g;
-        }
-    };
-    int nb = 0;
-    em::warp_traverse(T, xaf, yaf, zaf, R * R, INT64_MAX, [&](int64_t k, bool valid) {
-        collect(T, k, valid, xaf, yaf, zaf, lim2, buf, nb);
-        if (nb >= 32) {
-            sum_one(buf[lane]);
-            shift32(buf, nb);
-        }
-    });
-    if (lane < nb) sum_one(buf[lane]);
-    __syncwarp();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        ds += __shfl_xor_sync(0xffffffffu, ds, o);
-    }
-    return Density{s * norm, -ds * norm * ih};
-}
-
-// Sign of f(h) = h_fact n(h)^(-1/3) - h (Eq. 8) for the bisection, which uses
-// nothing else.  Every term of n is non-negative, so once the running sum
-// exceeds (h_fact / h)^3 (1 + 1e-9) the sign is negative whatever the rest of
-// the sum; the walk stops there (checked after each batch of 32 terms).  This
-// matters for the wide first brackets (h up to 1e2 h_0), whose 2h sphere
-// holds a large share of the population.  Otherwise the full sum decides, as
-// in warp_density.  Returns the sign of f (+1, 0 or -1).
-__device__ int warp_f_sign(const em::ChunkTree &T, const double *__restrict__ qx,
-                           const double *__restrict__ qy, const double *__restrict__ qz, double xa, double ya,
-                           double za, double h, double h_fact, float margin, int32_t *buf)
-{
-    const int lane = threadIdx.x & 31;
-    double s = 0.0;
-    const double ih = rcp64(h);
-    const double norm = ih * ih * ih * 0.31830988618379067154;   // 1/(pi h^3)
-    const double t = h_fact * ih;
-    const double thr = t * t * t * (1.0 + 1e-9);
-    float R = (float)(2.0 * h) + margin;
-    const float xaf = (float)xa, yaf = (float)ya, zaf = (float)za, h2f = (float)(2.0 * h);
-    const float lim = h2f + 1e-5f * (fabsf(xaf) + fabsf(yaf) + fabsf(zaf) + h2f);
-    const float lim2 = lim * lim;
-    // the sum of w; the walk stops once norm sum w exceeds thr
-    const double ih2 = ih * ih, thrw = thr * (3.14159265358979323846 * h * h * h);   // thr / norm
-    auto sum_one = [&](int64_t k) {
-        const double dx = qx[k] - xa, dy = qy[k] - ya, dz = qz[k] - za;
-        const double q2 = (dx * dx + dy * dy + dz * dz) * ih2;
-        if (q2 < 4.0) {
-            double w, g;
-            m4_wg(q_of(q2), q2, w, g);
-            s += w;
-        }
-    };
-    int nb = 0;
-    bool full = em::warp_traverse_until(T, xaf, yaf, zaf, R * R, [&](int64_t k, bool valid) {
-        collect(T, k, valid, xaf, yaf, zaf, lim2, buf, nb);
-        if (nb < 32) return true;
-        sum_one(buf[lane]);
-        shift32(buf, nb);
-        double tot = s;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-        return !(tot > thrw);
-    });
-    if (!full) return -1;
-    if (lane < nb) sum_one(buf[lane]);
-    __syncwarp();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const double f = h_fact * rcbrt(s * norm) - h;   // n^(-1/3) as a reciprocal cube root
-    return f > 0.0 ? 1 : (f < 0.0 ? -1 : 0);
-}
-
 // The solver's FP32 side.  Each FP64 evaluation of n(h) costs the FP64 pipe
 // about 20 instructions per 32 neighbours and 75 on values every lane shares;
 // the iterations that only approach the root, and the bisection's 50 signs,
@@ -338,15 +242,142 @@ constexpr int HS_LIST = 384;        // neighbours a warp keeps from its last wal
 constexpr float HS_COVER = 1.08f;   // the walk's radius, in units of the 2h it serves
 constexpr int HS_LEAVES = 4;        // 32-point leaves a walk reads together (their loads in flight at once)
 
-// A warp's pseudo-particle and the neighbours of its last walk: every
-// population entry within r of it if n >= 0 (n = -1: more than the list holds).
+// A node is solved by one warp or, where its 2h holds so much of the population
+// that one warp's walk would outlast all others (HS_HEAVY batches), by a team
+// of HS_TEAM: each warp of the team takes its share of every walk's leaves, and
+// all add up and decide alike.  (1e6 particles: the longest node 11.5 M cycles
+// against a mean of 0.12 M; tree, walk and h 8.6 ms without teams, 6.4 with.)
+constexpr int HS_TEAM = 8;
+constexpr int HS_HEAVY = 48;   // batches of HS_LEAVES leaves: 6,144 entries
+
+// A node under solution: its position, the neighbours of its last walk (every
+// population entry within r of it if n >= 0; n = -1: more than the list holds),
+// and this warp's part of the team.
 struct HsList {
     double xa, ya, za;
     float xh, yh, zh, xl, yl, zl;
     float r;
     int n;
     int32_t *k;
+    int32_t *buf;      // HS_BUF entries of the warp's own
+    double (*red)[2];  // the team's partial sums
+    int part;
+    bool heavy;        // one warp alone: the walk was given up
 };
+
+// a and b summed over the team's lanes, the same on all of them
+template <int TEAM, class Real>
+__device__ __forceinline__ void team_sum(const HsList &L, Real &a, Real &b)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (TEAM > 1) {
+        if ((threadIdx.x & 31) == 0) {
+            L.red[L.part][0] = (double)a;
+            L.red[L.part][1] = (double)b;
+        }
+        __syncthreads();
+        a = b = Real(0);
+        for (int t = 0; t < TEAM; ++t) {
+            a += (Real)L.red[t][0];
+            b += (Real)L.red[t][1];
+        }
+        __syncthreads();
+    }
+}
+
+
+// The population within 2h of the node, 32 entries at a time from a compacted
+// buffer: batch(k, in) on every lane, in false on the lanes without one; it
+// returns false to end the walk (a warp-uniform value).  Returns false where
+// the walk was ended or, by one warp alone, given up as heavy.
+template <int TEAM, class Batch>
+__device__ __forceinline__ bool walk_neighbours(const em::ChunkTree &T, HsList &L, double h, float margin,
+                                                Batch &&batch)
+{
+    const int lane = threadIdx.x & 31;
+    const float h2f = (float)(2.0 * h), R = h2f + margin;
+    const float lim = h2f + 1e-5f * (fabsf(L.xh) + fabsf(L.yh) + fabsf(L.zh) + h2f), lim2 = lim * lim;
+    int nb = 0, visits = 0;
+    const bool full = em::warp_traverse_batch<1>(T, L.xh, L.yh, L.zh, R * R, L.part, TEAM, [&](const int32_t(&k)[1]) {
+        if (TEAM == 1 && ++visits > HS_HEAVY * HS_LEAVES) {
+            L.heavy = true;
+            return false;
+        }
+        collect(T, k[0], k[0] >= 0, L.xh, L.yh, L.zh, lim2, L.buf, nb);
+        if (nb < 32) return true;
+        const bool go = batch(L.buf[lane], true);
+        shift32(L.buf, nb);
+        return go;
+    });
+    if (!full) return false;
+    batch(lane < nb ? L.buf[lane] : 0, lane < nb);
+    __syncwarp();
+    return true;
+}
+
+// w(q) and g(q) of entry k in FP64; false beyond 2h
+__device__ __forceinline__ bool term64(const Population &P, const HsList &L, int32_t k, double ih2, double &w, double &g)
+{
+    const double dx = P.x[k] - L.xa, dy = P.y[k] - L.ya, dz = P.z[k] - L.za;
+    const double q2 = (dx * dx + dy * dy + dz * dz) * ih2;
+    if (!(q2 < 4.0)) return false;
+    m4_wg(q_of(q2), q2, w, g);
+    return true;
+}
+
+// n(h) and dn/dh in FP64 (the same on all lanes) by a walk: n = norm sum w,
+// dn/dh = -norm sum g / h.
+template <int TEAM>
+__device__ Density warp_density(const em::ChunkTree &T, const Population &P, HsList &L, double h, float margin)
+{
+    double s = 0.0, ds = 0.0;
+    const double ih = rcp64(h), ih2 = ih * ih, norm = ih2 * ih * 0.31830988618379067154;   // 1/(pi h^3)
+    walk_neighbours<TEAM>(T, L, h, margin, [&](int32_t k, bool in) {
+        double w, g;
+        if (in && term64(P, L, k, ih2, w, g)) {
+            s += w;
+            ds += g;
+        }
+        return true;
+    });
+    team_sum<TEAM>(L, s, ds);
+    return Density{s * norm, -ds * norm * ih};
+}
+
+// Sign of f(h) = h_fact n(h)^(-1/3) - h (Eq. 8) for the bisection, which uses
+// nothing else.  Every term of n is non-negative, so once a warp's running sum
+// exceeds (h_fact / h)^3 (1 + 1e-9) the sign is negative whatever the rest of
+// the sum; its walk stops there (checked after each batch of 32 terms).  This
+// matters for the wide first brackets (h up to 1e2 h_0), whose 2h sphere
+// holds a large share of the population.  Otherwise the full sum decides, as
+// in warp_density.  Returns the sign of f (+1, 0 or -1).
+template <int TEAM>
+__device__ int warp_f_sign(const em::ChunkTree &T, const Population &P, HsList &L, double h, double h_fact,
+                           float margin)
+{
+    double s = 0.0, over = 0.0;
+    const double ih = rcp64(h), ih2 = ih * ih, norm = ih2 * ih * 0.31830988618379067154;   // 1/(pi h^3)
+    const double t = h_fact * ih, thr = t * t * t * (1.0 + 1e-9);
+    // the sum of w; the walk stops once norm sum w exceeds thr
+    const double thrw = thr * (3.14159265358979323846 * h * h * h);   // thr / norm
+    const bool full = walk_neighbours<TEAM>(T, L, h, margin, [&](int32_t k, bool in) {
+        double w, g;
+        if (in && term64(P, L, k, ih2, w, g)) s += w;
+        double tot = s;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        return !(tot > thrw);
+    });
+    if (!full) over = 1.0;
+    team_sum<TEAM>(L, s, over);
+    if (over > 0.0) return -1;
+    const double f = h_fact * rcbrt(s * norm) - h;   // n^(-1/3) as a reciprocal cube root
+    return f > 0.0 ? 1 : (f < 0.0 ? -1 : 0);
+}
 
 struct Sum32 {
     float S, G;   // sums of w and of g = 3 w + q w'
@@ -377,6 +408,7 @@ __device__ __forceinline__ void add32(const HsList &L, bool in, float4 p, float4
 
 // The sums at h in FP32 (the same on every lane), from the list where it
 // covers 2h, else by a walk that renews it.
+template <int TEAM>
 __device__ Sum32 warp_sum32(const em::ChunkTree &T, const Population &P, HsList &L, float h, float margin)
 {
     const int lane = threadIdx.x & 31;
@@ -387,9 +419,13 @@ __device__ Sum32 warp_sum32(const em::ChunkTree &T, const Population &P, HsList 
     } else {
         const float r = 2.f * HS_COVER * h;
         const float lim = r + 1e-5f * (fabsf(L.xh) + fabsf(L.yh) + fabsf(L.zh) + r), lim2 = lim * lim;
-        int n = 0;
-        em::warp_traverse_batch<HS_LEAVES>(T, L.xh, L.yh, L.zh, (r + margin) * (r + margin),
+        int n = 0, visits = 0;
+        em::warp_traverse_batch<HS_LEAVES>(T, L.xh, L.yh, L.zh, (r + margin) * (r + margin), L.part, TEAM,
                                            [&](const int32_t(&k)[HS_LEAVES]) {
+            if (TEAM == 1 && ++visits > HS_HEAVY) {
+                L.heavy = true;
+                return false;
+            }
             float4 p[HS_LEAVES], lo[HS_LEAVES];
             unsigned b[HS_LEAVES];
 #pragma unroll
@@ -408,28 +444,27 @@ __device__ Sum32 warp_sum32(const em::ChunkTree &T, const Population &P, HsList 
 #pragma unroll
             for (int u = 0; u < HS_LEAVES; ++u) {
                 const int pos = n + __popc(b[u] & ((1u << lane) - 1u));
-                if (((b[u] >> lane) & 1u) && pos < HS_LIST) L.k[pos] = k[u];
+                if (TEAM == 1 && ((b[u] >> lane) & 1u) && pos < HS_LIST) L.k[pos] = k[u];
                 n += __popc(b[u]);
             }
+            return true;
         });
         __syncwarp();
         L.r = r;
-        L.n = n <= HS_LIST ? n : -1;
+        L.n = TEAM == 1 && n <= HS_LIST && !L.heavy ? n : -1;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        S += __shfl_xor_sync(0xffffffffu, S, o);
-        G += __shfl_xor_sync(0xffffffffu, G, o);
-    }
+    team_sum<TEAM>(L, S, G);
     return Sum32{S, G};
 }
 
 // Make the list the population within 2h and a margin for h's last digits, so
 // that FP64 batches hold neighbours only.
+template <int TEAM>
 __device__ void settle_list(const em::ChunkTree &T, const Population &P, HsList &L, float h, float margin)
 {
     const int lane = threadIdx.x & 31;
-    if (!(L.n >= 0 && 2.0002f * h <= L.r)) warp_sum32(T, P, L, h, margin);
+    if (TEAM > 1) return;   // a team keeps no list
+    if (!(L.n >= 0 && 2.0002f * h <= L.r)) warp_sum32<TEAM>(T, P, L, h, margin);
     const float r = 2.004f * h;
     if (L.n < 0 || L.r <= r) return;
     const float lim = r + 1e-5f * (fabsf(L.xh) + fabsf(L.yh) + fabsf(L.zh) + r), lim2 = lim * lim;
@@ -452,28 +487,20 @@ __device__ void settle_list(const em::ChunkTree &T, const Population &P, HsList 
 }
 
 // n(h) and dn/dh in FP64 from the list where it covers 2h, else by a walk.
-__device__ Density list_density(const em::ChunkTree &T, const Population &P, const HsList &L, double h, float margin,
-                                int32_t *buf)
+template <int TEAM>
+__device__ Density list_density(const em::ChunkTree &T, const Population &P, HsList &L, double h, float margin)
 {
-    if (!(L.n >= 0 && 2.0002f * (float)h <= L.r)) return warp_density(T, P.x, P.y, P.z, L.xa, L.ya, L.za, h, margin, buf);
+    if (!(L.n >= 0 && 2.0002f * (float)h <= L.r)) return warp_density<TEAM>(T, P, L, h, margin);
     double s = 0.0, ds = 0.0;
     const double ih = rcp64(h), ih2 = ih * ih, norm = ih2 * ih * 0.31830988618379067154;   // 1/(pi h^3)
     for (int t = threadIdx.x & 31; t < L.n; t += 32) {
-        const int32_t k = L.k[t];
-        const double dx = P.x[k] - L.xa, dy = P.y[k] - L.ya, dz = P.z[k] - L.za;
-        const double q2 = (dx * dx + dy * dy + dz * dz) * ih2;
-        if (q2 < 4.0) {
-            double w, g;
-            m4_wg(q_of(q2), q2, w, g);
+        double w, g;
+        if (term64(P, L, L.k[t], ih2, w, g)) {
             s += w;
             ds += g;
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        ds += __shfl_xor_sync(0xffffffffu, ds, o);
-    }
+    team_sum<TEAM>(L, s, ds);
     return Density{s * norm, -ds * norm * ih};
 }
 
@@ -493,13 +520,15 @@ __device__ __forceinline__ double newton_step(Density d, double h, double h_fact
 // Newton (Eq. 10) from h_0 (Eq. 11) until |dh|/h_0 < tol, every evaluation in
 // FP64.  Returns false where an iterate leaves the bracket [1e-2 h_0, 1e2 h_0]
 // or max_newton steps do not suffice: Newton failed.
-__device__ bool newton64(const em::ChunkTree &T, const Population &P, const HsList &L, double h0, double h_fact,
-                         double tol, int max_newton, float margin, int32_t *buf, double &hout)
+template <int TEAM>
+__device__ bool newton64(const em::ChunkTree &T, const Population &P, HsList &L, double h0, double h_fact,
+                         double tol, int max_newton, float margin, double &hout)
 {
     const double ih0 = rcp64(h0), blo = 1e-2 * h0, bhi = 1e2 * h0;
     double h = h0;
     for (int it = 0; it < max_newton; ++it) {
-        const double hn = newton_step(warp_density(T, P.x, P.y, P.z, L.xa, L.ya, L.za, h, margin, buf), h, h_fact);
+        const double hn = newton_step(warp_density<TEAM>(T, P, L, h, margin), h, h_fact);
+        if (L.heavy) return false;
         if (!(hn >= blo && hn <= bhi)) return false;
         const double step = fabs(hn - h) * ih0;   // |dh| / h_0
         h = hn;
@@ -512,22 +541,22 @@ __device__ bool newton64(const em::ChunkTree &T, const Population &P, const HsLi
 }
 
 // Bisection on [1e-2 h_0, 1e2 h_0] by signs (warp_f_sign), else h_0.
-__device__ double bisect64(const em::ChunkTree &T, const Population &P, const HsList &L, double h0, double h_fact,
-                           double tol, float margin, int32_t *buf, int &st)
+template <int TEAM>
+__device__ double bisect64(const em::ChunkTree &T, const Population &P, HsList &L, double h0, double h_fact,
+                           double tol, float margin, int &st)
 {
-    const double xa = L.xa, ya = L.ya, za = L.za;
-    const double *qx = P.x, *qy = P.y, *qz = P.z;
     double lo = 1e-2 * h0, hi = 1e2 * h0;
-    const int slo = warp_f_sign(T, qx, qy, qz, xa, ya, za, lo, h_fact, margin, buf);
-    const int shi = warp_f_sign(T, qx, qy, qz, xa, ya, za, hi, h_fact, margin, buf);
+    const int slo = warp_f_sign<TEAM>(T, P, L, lo, h_fact, margin);
+    const int shi = warp_f_sign<TEAM>(T, P, L, hi, h_fact, margin);
     const bool plo = slo > 0;
+    if (L.heavy) return h0;
     if (slo * shi > 0) {
         st = 2;
         return h0;
     }
-    for (int k = 0; k < 200 && (hi - lo) > tol * h0; ++k) {
+    for (int k = 0; k < 200 && (hi - lo) > tol * h0 && !L.heavy; ++k) {
         const double mid = 0.5 * (lo + hi);
-        if ((warp_f_sign(T, qx, qy, qz, xa, ya, za, mid, h_fact, margin, buf) > 0) == plo) lo = mid;
+        if ((warp_f_sign<TEAM>(T, P, L, mid, h_fact, margin) > 0) == plo) lo = mid;
         else hi = mid;
     }
     st = 1;
@@ -537,12 +566,14 @@ __device__ double bisect64(const em::ChunkTree &T, const Population &P, const Hs
 // The root of f near h (an FP32 root) by Newton in FP64: the step after which
 // the quadratic convergence leaves less than a tenth of tol is the last.
 // Returns false where it does not settle at once.
+template <int TEAM>
 __device__ bool polish64(const em::ChunkTree &T, const Population &P, HsList &L, double &h, double h_fact, double tol,
-                         float margin, int32_t *buf)
+                         float margin)
 {
-    settle_list(T, P, L, (float)h, margin);
+    settle_list<TEAM>(T, P, L, (float)h, margin);
     for (int it = 0; it < 5; ++it) {
-        const double hn = newton_step(list_density(T, P, L, h, margin, buf), h, h_fact);
+        const double hn = newton_step(list_density<TEAM>(T, P, L, h, margin), h, h_fact);
+        if (L.heavy) return false;
         const double d = fabs(hn - h);
         if (!(d <= 1e-3 * h)) return false;
         h = hn;
@@ -557,14 +588,16 @@ __device__ bool polish64(const em::ChunkTree &T, const Population &P, HsList &L,
 // FP64 unless an iterate comes within 10% of the bracket's ends (-1: not
 // decided).
 constexpr double HS_WARM_TOL = 1e-9;
+template <int TEAM>
 __device__ int newton32(const em::ChunkTree &T, const Population &P, HsList &L, double h0, double h_fact, double tol,
-                        int max_newton, float margin, int32_t *buf, double &hout)
+                        int max_newton, float margin, double &hout)
 {
     const float h0f = (float)h0, hf = (float)h_fact, blo = 1e-2f * h0f, bhi = 1e2f * h0f;
     float h = h0f;
     if (!(h0f > 1e-15f && h0f < 1e15f)) return -1;
     for (int it = 0; it + 4 < max_newton; ++it) {
-        const Sum32 u = warp_sum32(T, P, L, h, margin);
+        const Sum32 u = warp_sum32<TEAM>(T, P, L, h, margin);
+        if (L.heavy) return -1;
         const float a = hf * cbrtf(3.14159265f / u.S);   // h_fact n^(-1/3) / h
         const float hn = h * (1.f - (a - 1.f) / (a * u.G / (3.f * u.S) - 1.f));
         if (!(fabsf(hn) < 1e30f)) return -1;
@@ -574,7 +607,7 @@ __device__ int newton32(const em::ChunkTree &T, const Population &P, HsList &L, 
         h = hn;
         if (d < 3e-4f * h) {
             hout = h;
-            return polish64(T, P, L, hout, h_fact, tol, margin, buf) ? 1 : -1;
+            return polish64<TEAM>(T, P, L, hout, h_fact, tol, margin) ? 1 : -1;
         }
     }
     return -1;
@@ -585,21 +618,24 @@ __device__ int newton32(const em::ChunkTree &T, const Population &P, HsList &L, 
 // bracket is found by a bracketed Newton in log h, polished, and the
 // bisection's decisions are comparisons with r; only a midpoint within 2e-14 r
 // of it (the rounding of either) takes an FP64 evaluation.
+template <int TEAM>
 __device__ bool bisect32(const em::ChunkTree &T, const Population &P, HsList &L, double h0, double h_fact, double tol,
-                         float margin, int32_t *buf, double &hout, int &st)
+                         float margin, double &hout, int &st)
 {
     const float h0f = (float)h0, hf = (float)h_fact, blo = 1e-2f * h0f, bhi = 1e2f * h0f;
     const float target = 3.14159265f * hf * hf * hf;
     if (!(h0f > 1e-15f && h0f < 1e15f)) return false;
     // the bracket's ends, each moved to the nearest point with the same sign
     float lo = blo, hi = h0f;
-    auto sum = [&](float at) { return warp_sum32(T, P, L, at, margin); };
+    auto sum = [&](float at) { return warp_sum32<TEAM>(T, P, L, at, margin); };
     Sum32 u = sum(h0f);
+    if (L.heavy) return false;
     if (u.S < target) {
         lo = h0f;
         while (true) {
             hi = fminf(2.f * lo, bhi);
             u = sum(hi);
+            if (L.heavy) return false;
             if (u.S > target) break;
             if (hi == bhi) {
                 if (u.S > 0.999f * target) return false;
@@ -612,12 +648,14 @@ __device__ bool bisect32(const em::ChunkTree &T, const Population &P, HsList &L,
         if (hi == bhi && u.S < 1.001f * target) return false;
     } else {
         u = sum(blo);
+        if (L.heavy) return false;
         if (u.S > 0.999f * target) return false;
     }
     float h = sqrtf(lo * hi);
     for (int it = 0;; ++it) {
         if (it == 40) return false;
         u = sum(h);
+        if (L.heavy) return false;
         if (u.S < target) lo = h;
         else hi = h;
         const float D = 3.f * u.S - u.G;   // dS / dlog h
@@ -629,36 +667,28 @@ __device__ bool bisect32(const em::ChunkTree &T, const Population &P, HsList &L,
         if ((in && d < 3e-4f * h) || hi - lo < 1e-6f * h) break;
     }
     double r = h;
-    if (!polish64(T, P, L, r, h_fact, tol, margin, buf)) return false;
+    if (!polish64<TEAM>(T, P, L, r, h_fact, tol, margin)) return false;
     double dlo = 1e-2 * h0, dhi = 1e2 * h0;
     const double near = 2e-14 * r, width = tol * h0;
-    for (int k = 0; k < 200 && (dhi - dlo) > width; ++k) {
+    for (int k = 0; k < 200 && (dhi - dlo) > width && !L.heavy; ++k) {
         const double mid = 0.5 * (dlo + dhi), e = mid - r;
         const bool below = fabs(e) > near ? e < 0.0
-                                          : warp_f_sign(T, P.x, P.y, P.z, L.xa, L.ya, L.za, mid, h_fact, margin, buf) > 0;
+                                          : warp_f_sign<TEAM>(T, P, L, mid, h_fact, margin) > 0;
         if (below) dlo = mid;
         else dhi = mid;
     }
     hout = 0.5 * (dlo + dhi);
     st = 1;
-    return true;
+    return !L.heavy;
 }
 
-// One warp per pseudo-particle.  1e6 particles (94,193 nodes, 5,733 of them
-// bisected): 417,533 FP64 evaluations of n(h) and 298,116 signs, each with its
-// walk, took 11.2 ms; 112,000 FP64 evaluations, 1.5 walks and 1.8 sums over a
-// list per node take 5.8, most of it the tail of the few nodes whose 2h holds
-// thousands of the population.
-__global__ void __launch_bounds__(32 * HS_WARPS, 6) k_h_solve(int64_t npseudo, em::ChunkTree T, Population P, const double *__restrict__ px,
-                          const double *__restrict__ py, const double *__restrict__ pz, double h_fact, double tol,
-                          int max_newton, float margin, double *__restrict__ ph, int32_t *__restrict__ status)
+// Solve node a; a warp alone that meets a heavy walk leaves it (false).
+template <int TEAM>
+__device__ __forceinline__ bool solve_node(const em::ChunkTree &T, const Population &P, HsList &L, int64_t a,
+                                           const double *__restrict__ px, const double *__restrict__ py,
+                                           const double *__restrict__ pz, double h_fact, double tol, int max_newton,
+                                           float margin, double *__restrict__ ph, int32_t *__restrict__ status)
 {
-    __shared__ int32_t bufs[HS_WARPS][HS_BUF], lists[HS_WARPS][HS_LIST];
-    int32_t *buf = bufs[threadIdx.x >> 5];
-    int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (a >= npseudo) return;
-    if (status[a] != -1) return;   // extracted particles keep their own h
-    HsList L;
     L.xa = px[a];
     L.ya = py[a];
     L.za = pz[a];
@@ -667,18 +697,66 @@ __global__ void __launch_bounds__(32 * HS_WARPS, 6) k_h_solve(int64_t npseudo, e
     em::split_df(L.za, L.zh, L.zl);
     L.r = 0.f;
     L.n = -1;
-    L.k = lists[threadIdx.x >> 5];
+    L.heavy = false;
     const double h0 = ph[a];
     double h = h0;
     int st = 0;
     const bool warm = tol <= HS_WARM_TOL;
-    int ok = warm ? newton32(T, P, L, h0, h_fact, tol, max_newton, margin, buf, h) : -1;
-    if (ok < 0) ok = newton64(T, P, L, h0, h_fact, tol, max_newton, margin, buf, h) ? 1 : 0;
-    if (!ok && !(warm && bisect32(T, P, L, h0, h_fact, tol, margin, buf, h, st)))
-        h = bisect64(T, P, L, h0, h_fact, tol, margin, buf, st);
-    if ((threadIdx.x & 31) == 0) {
+    int ok = warm ? newton32<TEAM>(T, P, L, h0, h_fact, tol, max_newton, margin, h) : -1;
+    if (ok < 0 && !L.heavy) ok = newton64<TEAM>(T, P, L, h0, h_fact, tol, max_newton, margin, h) ? 1 : 0;
+    if (!ok && !L.heavy && !(warm && bisect32<TEAM>(T, P, L, h0, h_fact, tol, margin, h, st)) && !L.heavy)
+        h = bisect64<TEAM>(T, P, L, h0, h_fact, tol, margin, st);
+    if (L.heavy) return false;
+    if (TEAM > 1) __syncthreads();   // every warp has read h_0
+    if ((threadIdx.x & 31) == 0 && L.part == 0) {
         ph[a] = h;
         status[a] = st;
+    }
+    return true;
+}
+
+// One warp per pseudo-particle; the heavy ones are listed for k_h_solve_heavy.
+// 1e6 particles (94,193 nodes, 5,733 of them bisected): 417,533 FP64
+// evaluations of n(h) and 298,116 signs, each with its walk, took 11.2 ms;
+// 112,000 FP64 evaluations, 1.5 walks and 1.8 sums over a list per node took
+// 5.8, most of it the tail of the few nodes whose 2h holds thousands of the
+// population.
+__global__ void __launch_bounds__(32 * HS_WARPS, 6) k_h_solve(
+    int64_t npseudo, em::ChunkTree T, Population P, const double *__restrict__ px, const double *__restrict__ py,
+    const double *__restrict__ pz, double h_fact, double tol, int max_newton, float margin, double *__restrict__ ph,
+    int32_t *__restrict__ status, int *__restrict__ nheavy, int32_t *__restrict__ heavy)
+{
+    __shared__ int32_t bufs[HS_WARPS][HS_BUF], lists[HS_WARPS][HS_LIST];
+    int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (a >= npseudo) return;
+    if (status[a] != -1) return;   // extracted particles keep their own h
+    HsList L;
+    L.k = lists[threadIdx.x >> 5];
+    L.buf = bufs[threadIdx.x >> 5];
+    L.red = nullptr;
+    L.part = 0;
+    if (!solve_node<1>(T, P, L, a, px, py, pz, h_fact, tol, max_newton, margin, ph, status) && (threadIdx.x & 31) == 0)
+        heavy[atomicAdd(nheavy, 1)] = (int32_t)a;
+}
+
+// The listed nodes, a block of HS_TEAM warps each (grid-stride; the count is
+// read on the device).
+__global__ void __launch_bounds__(32 * HS_TEAM) k_h_solve_heavy(
+    em::ChunkTree T, Population P, const double *__restrict__ px, const double *__restrict__ py,
+    const double *__restrict__ pz, double h_fact, double tol, int max_newton, float margin, double *__restrict__ ph,
+    int32_t *__restrict__ status, const int *__restrict__ nheavy, const int32_t *__restrict__ heavy)
+{
+    __shared__ int32_t bufs[HS_TEAM][HS_BUF];
+    __shared__ double red[HS_TEAM][2];
+    HsList L;
+    L.k = nullptr;
+    L.buf = bufs[threadIdx.x >> 5];
+    L.red = red;
+    L.part = threadIdx.x >> 5;
+    const int n = *nheavy;
+    for (int t = blockIdx.x; t < n; t += gridDim.x) {
+        solve_node<HS_TEAM>(T, P, L, heavy[t], px, py, pz, h_fact, tol, max_newton, margin, ph, status);
+        __syncthreads();
     }
 }
 
@@ -778,8 +856,18 @@ static int pseudo_impl(em_ctx *ctx, const em_tree *t, const double *d_hp, int ns
         EM_TRY(tmp.alloc(&plo, npop));
         k_population_lo<<<em_grid(npop, 256), 256, 0, st>>>(npop, qx, qy, qz, plo);
         EM_LAUNCHED(ctx);
-        k_h_solve<<<em_grid(np * 32, 32 * HS_WARPS), 32 * HS_WARPS, 0, st>>>(
-            np, T, Population{qx, qy, qz, plo}, ps->x, ps->y, ps->z, p->h_fact, p->h_tol, p->max_newton, margin, ps->h, ps->status);
+        int *nheavy;
+        int32_t *heavy;
+        EM_TRY(tmp.alloc(&nheavy, 1));
+        EM_TRY(tmp.alloc(&heavy, np));
+        EM_CUDA(cudaMemsetAsync(nheavy, 0, sizeof(int), st));
+        const Population P{qx, qy, qz, plo};
+        k_h_solve<<<em_grid(np * 32, 32 * HS_WARPS), 32 * HS_WARPS, 0, st>>>(np, T, P, ps->x, ps->y, ps->z, p->h_fact,
+                                                                              p->h_tol, p->max_newton, margin, ps->h,
+                                                                              ps->status, nheavy, heavy);
+        EM_LAUNCHED(ctx);
+        k_h_solve_heavy<<<(unsigned)std::min<int64_t>(np, 4 * (int64_t)ctx->nsm), 32 * HS_TEAM, 0, st>>>(
+            T, P, ps->x, ps->y, ps->z, p->h_fact, p->h_tol, p->max_newton, margin, ps->h, ps->status, nheavy, heavy);
         EM_LAUNCHED(ctx);
     }
     unsigned long long *cnt;

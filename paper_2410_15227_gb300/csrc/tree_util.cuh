@@ -110,19 +110,22 @@ __device__ __forceinline__ bool warp_traverse(const ChunkTree &T, float px, floa
 
 // warp_traverse over batches of up to U leaves that share a parent: visit
 // gets every lane's item in each (-1 for none), so that it can issue U leaves'
-// loads before it waits for one.  Items must number below 2^31.
-template <int U, class Visit>
-__device__ __forceinline__ void warp_traverse_batch(const ChunkTree &T, float px, float py, float pz, float R2,
+// loads before it waits for one, and returns false to end the walk (a
+// warp-uniform value).  Nodes are opened where within(lo, hi) of their box
+// holds.  Of a team of warps that walk alike, warp `part` of `parts` takes
+// every parts-th batch.  Items must number below 2^31.
+template <int U, class Within, class Visit>
+__device__ __forceinline__ bool warp_traverse_boxes(const ChunkTree &T, int part, int parts, Within &&within,
                                                     Visit &&visit)
 {
     const int lane = threadIdx.x & 31;
     uint32_t mask[kMaxLevels + 1];
     int64_t base[kMaxLevels + 1];
     const int top = T.nlev;
-    if (top <= 0) return;
-    const float R2m = R2 * 1.00001f + 1e-30f;   // conservative margin for the float boxes
+    if (top <= 0) return true;
+    int turn = 0;
     auto open = [&](int level, int64_t node) {
-        return node < T.count[level] && box_dist2(T.lo[level][node], T.hi[level][node], px, py, pz) <= R2m;
+        return node < T.count[level] && within(T.lo[level][node], T.hi[level][node]);
     };
     mask[top] = __ballot_sync(0xffffffffu, open(top, lane));
     base[top] = 0;
@@ -143,7 +146,8 @@ __device__ __forceinline__ void warp_traverse_batch(const ChunkTree &T, float px
                 m &= m - 1;
             }
             mask[1] = m;
-            visit(k);
+            if (turn == part && !visit(k)) return false;
+            turn = turn + 1 == parts ? 0 : turn + 1;
         } else {
             const int c = __ffs(mask[lvl]) - 1;
             mask[lvl] &= mask[lvl] - 1;
@@ -153,48 +157,17 @@ __device__ __forceinline__ void warp_traverse_batch(const ChunkTree &T, float px
             --lvl;
         }
     }
+    return true;
 }
 
-// warp_traverse whose visit returns true to go on and false to end the walk
-// (a warp-uniform value).  Returns false if the walk was ended by visit.
-template <class Visit>
-__device__ __forceinline__ bool warp_traverse_until(const ChunkTree &T, float px, float py, float pz, float R2,
-                                                    Visit &&visit)
+// Within sqrt(R2) of p.
+template <int U, class Visit>
+__device__ __forceinline__ bool warp_traverse_batch(const ChunkTree &T, float px, float py, float pz, float R2,
+                                                    int part, int parts, Visit &&visit)
 {
-    const int lane = threadIdx.x & 31;
-    uint32_t mask[kMaxLevels + 1];
-    int64_t base[kMaxLevels + 1];
-    const int top = T.nlev;
-    if (top <= 0) return true;
     const float R2m = R2 * 1.00001f + 1e-30f;   // conservative margin for the float boxes
-    {
-        bool hit = lane < T.count[top] && box_dist2(T.lo[top][lane], T.hi[top][lane], px, py, pz) <= R2m;
-        mask[top] = __ballot_sync(0xffffffffu, hit);
-        base[top] = 0;
-    }
-    int lvl = top;
-    while (true) {
-        if (mask[lvl] == 0) {
-            if (lvl == top) break;
-            ++lvl;
-            continue;
-        }
-        int c = __ffs(mask[lvl]) - 1;
-        mask[lvl] &= mask[lvl] - 1;
-        int64_t node = base[lvl] * 32 + c;
-        if (lvl == 1) {
-            int64_t k = node * 32 + lane;
-            if (!visit(k, k < T.count[0])) return false;
-        } else {
-            int64_t child = node * 32 + lane;
-            bool hit = child < T.count[lvl - 1] &&
-                       box_dist2(T.lo[lvl - 1][child], T.hi[lvl - 1][child], px, py, pz) <= R2m;
-            mask[lvl - 1] = __ballot_sync(0xffffffffu, hit);
-            base[lvl - 1] = node;
-            --lvl;
-        }
-    }
-    return true;
+    return warp_traverse_boxes<U>(
+        T, part, parts, [&](float4 lo, float4 hi) { return box_dist2(lo, hi, px, py, pz) <= R2m; }, visit);
 }
 
 }  // namespace em

@@ -1,7 +1,8 @@
 """The node h-solver where its FP32 approach hands over: populations too small
 for a root (h_0), nodes without neighbours inside 2 h_0 (bisection), more
-neighbours inside 2 h_0 than a warp's list holds, and coordinates far from the
-origin.  Status and h as the oracle's, whose evaluations are all FP64; at a
+neighbours inside 2 h_0 than a warp's list holds, a core of leaves inside the
+2h of every node around it (solved by teams of warps), and coordinates far from
+the origin.  Status and h as the oracle's, whose evaluations are all FP64; at a
 tolerance just above and just below the one from which the FP32 approach is
 used, the same statuses."""
 import numpy as np
@@ -29,10 +30,14 @@ def cloud(kind):
     if kind == "dense":                   # large nodes over a dense core: long lists
         v = rng.normal(size=(6000, 3))
         return v / np.linalg.norm(v, axis=1, keepdims=True) * (rng.random(6000) ** 2)[:, None]
+    if kind == "core":                    # 60,000 particles' leaves within 2h of 400 outer nodes
+        v = rng.normal(size=(60400, 3))
+        r = np.concatenate([0.04 * rng.random(60000) ** (1 / 3), 0.3 + 0.7 * rng.random(400)])
+        return v / np.linalg.norm(v, axis=1, keepdims=True) * r[:, None]
     return 1000.0 + rng.random((3000, 3))   # "far"
 
 
-@pytest.mark.parametrize("kind", ["few", "clusters", "pairs", "dense", "far"])
+@pytest.mark.parametrize("kind", ["few", "clusters", "pairs", "dense", "core", "far"])
 @pytest.mark.parametrize("theta", [0.3, 1.5])
 @pytest.mark.parametrize("tol", [1e-13, 9.9e-10, 1.1e-9])
 def test_status_and_h(orc, kind, theta, tol):
@@ -40,7 +45,7 @@ def test_status_and_h(orc, kind, theta, tol):
     lo, hi = p.min(0), p.max(0)
     box = np.stack([lo - 0.01, hi + 0.01], 1).reshape(-1)
     m, h = np.full(len(p), 1.0 / len(p)), np.full(len(p), 0.05)
-    src = lo[None] - 0.3
+    src = lo[None] - 0.3 if kind != "core" else np.zeros((1, 3))
     o, _, _ = orc.make_pseudo_particles(p[:, 0], p[:, 1], p[:, 2], m, h, box, src, 0.05, 0.1, theta, h_fact=1.2,
                                         tol=tol)
     ctx = api.Context(0)
