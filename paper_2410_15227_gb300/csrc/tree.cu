@@ -399,8 +399,8 @@ __global__ void k_chunk_leaf(int64_t nbox, int64_t n, const double *__restrict__
     float lx = INFINITY, ly = INFINITY, lz = INFINITY, hx = -INFINITY, hy = -INFINITY, hz = -INFINITY;
     int64_t e = (b + 1) * 32 < n ? (b + 1) * 32 : n;
     for (int64_t k = b * 32; k < e; ++k) {
-        pts[k] = make_float4((float)xs[k], (float)ys[k], (float)zs[k], 0.f);
         double rr = r ? r[k] * rscale : 0.0;
+        pts[k] = make_float4((float)xs[k], (float)ys[k], (float)zs[k], __double2float_ru(rr));
         lx = fminf(lx, __double2float_rd(xs[k] - rr));
         ly = fminf(ly, __double2float_rd(ys[k] - rr));
         lz = fminf(lz, __double2float_rd(zs[k] - rr));

@@ -49,7 +49,7 @@ struct ChunkTree {
     int64_t count[kMaxLevels + 1];    // nodes per level (count[0] = items)
     float4 *lo[kMaxLevels + 1];       // per level l >= 1: box min (xyz)
     float4 *hi[kMaxLevels + 1];       // box max
-    float4 *pts = nullptr;            // level 0: item positions rounded to FP32 (w = 0)
+    float4 *pts = nullptr;            // level 0: item positions rounded to FP32, w the radius rounded up (0 without)
 };
 
 __host__ __device__ __forceinline__ float box_dist2(const float4 lo, const float4 hi, float px, float py, float pz)
