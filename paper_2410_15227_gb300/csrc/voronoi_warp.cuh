@@ -39,7 +39,7 @@ template <int NV>
 struct WCell {
     static constexpr int MAXV = NV;
     static_assert(NV <= 255, "vertex indices are bytes, 0xff marks a removed vertex");
-    float vf[NV][4];   // FP32 vertex in the site's frame, w = |x| + |y| + |z|
+    float4 vf[NV];     // FP32 vertex in the site's frame, w = |x| + |y| + |z|
     float ev[NV];      // bound on |vf - v| per coordinate, v the exact meet of its planes
     float4 pf[WMAXP];
     int sid[WMAXP];
@@ -50,16 +50,19 @@ struct WCell {
         } k;                    // while the cell is built
         double vx[NV][3];       // the FP64 vertices of the finished cell
     } u;
-    // clip in progress: 1 if the vertex lies beyond the plane, then its new
-    // index (0xff if removed)
-    uint8_t side[NV];
+    uint8_t side[NV];       // clip in progress: the vertex's new index (0xff if removed)
     uint8_t out_list[NV];   // clip in progress: the removed vertices
-    uint8_t tri[2][NV][4];
-    // adj[t][e]: the vertex across edge e of vertex t, i.e. the one whose
-    // triangle holds the reversed edge (tri[t][e + 1], tri[t][e])
-    uint8_t adj[2][NV][4];
+    // clip in progress: the new vertex whose edge leaves plane p (a = p), and the
+    // one whose edge ends at it (b = p)
+    uint8_t of_a[WMAXP], of_b[WMAXP];
+    uint32_t tri[2][NV];    // the vertex's three planes, one per byte (byte_of)
+    // byte e of adj[t]: the vertex across edge e of vertex t, i.e. the one whose
+    // triangle holds the reversed edge (tri e + 1, tri e)
+    uint32_t adj[2][NV];
     int np, nt, cur;
 };
+
+__device__ __forceinline__ int byte_of(uint32_t w, int e) { return (int)((w >> (8 * e)) & 0xffu); }
 
 // Bisector plane n.x <= d of the site g (at the origin of the cell's frame)
 // and generator k: n = g_k - g, d = |n|^2 / 2.
@@ -151,18 +154,15 @@ __device__ void meet64(const C &c, const Frame &F, int t, double &x, double &y, 
 {
     double P[3][4];
 #pragma unroll
-    for (int e = 0; e < 3; ++e) plane64(F, c.sid[c.tri[c.cur][t][e]], P[e][0], P[e][1], P[e][2], P[e][3]);
+    for (int e = 0; e < 3; ++e) plane64(F, c.sid[byte_of(c.tri[c.cur][t], e)], P[e][0], P[e][1], P[e][2], P[e][3]);
     meet64p(P[0], P[1], P[2], x, y, z);
 }
 
 // FP32 copy of a vertex from its FP64 meet, and the bound of its rounding.
-__device__ __forceinline__ void set_vf(float *vf, float &ev, double x, double y, double z)
+__device__ __forceinline__ void set_vf(float4 &vf, float &ev, double x, double y, double z)
 {
     const float xf = (float)x, yf = (float)y, zf = (float)z;
-    vf[0] = xf;
-    vf[1] = yf;
-    vf[2] = zf;
-    vf[3] = fabsf(xf) + fabsf(yf) + fabsf(zf);
+    vf = make_float4(xf, yf, zf, fabsf(xf) + fabsf(yf) + fabsf(zf));
     ev = U32 * fmaxf(fabsf(xf), fmaxf(fabsf(yf), fabsf(zf)));
 }
 
@@ -190,10 +190,13 @@ __device__ void wcell_box(C &c, const Frame &F)
         const uint8_t X = (uint8_t)sx, Y = (uint8_t)(2 + sy), Z = (uint8_t)(4 + sz);
         const bool pos = ((sx ? 1 : -1) * (sy ? 1 : -1) * (sz ? 1 : -1)) > 0;
         const uint8_t t[3] = {X, pos ? Y : Z, pos ? Z : Y};
+        uint32_t tw = 0, aw = 0;
         for (int e = 0; e < 3; ++e) {
-            c.tri[0][i][e] = t[e];
-            c.adj[0][i][e] = (uint8_t)(i ^ (1 << (t[(e + 2) % 3] >> 1)));
+            tw |= (uint32_t)t[e] << (8 * e);
+            aw |= (uint32_t)(i ^ (1 << (t[(e + 2) % 3] >> 1))) << (8 * e);
         }
+        c.tri[0][i] = tw;
+        c.adj[0][i] = aw;
         set_vf(c.vf[i], c.ev[i], sx ? F.box[1] - F.gx : F.box[0] - F.gx, sy ? F.box[3] - F.gy : F.box[2] - F.gy,
                sz ? F.box[5] - F.gz : F.box[4] - F.gz);
     }
@@ -215,7 +218,7 @@ __device__ int wcompact(C &c)
         for (int q = 0; q < c.np; ++q) map[q] = -1;
         const int cur = c.cur;
         for (int t = 0; t < c.nt; ++t)
-            for (int e = 0; e < 3; ++e) map[c.tri[cur][t][e]] = 0;
+            for (int e = 0; e < 3; ++e) map[byte_of(c.tri[cur][t], e)] = 0;
         int n = 0;
         for (int q = 0; q < c.np; ++q) {
             if (map[q] < 0) continue;
@@ -224,69 +227,79 @@ __device__ int wcompact(C &c)
             c.pf[n] = c.pf[q];
             ++n;
         }
-        for (int t = 0; t < c.nt; ++t)
-            for (int e = 0; e < 3; ++e) c.tri[cur][t][e] = (uint8_t)map[c.tri[cur][t][e]];
+        for (int t = 0; t < c.nt; ++t) {
+            const uint32_t w = c.tri[cur][t];
+            c.tri[cur][t] = (uint32_t)map[byte_of(w, 0)] | (uint32_t)map[byte_of(w, 1)] << 8 | (uint32_t)map[byte_of(w, 2)] << 16;
+        }
         c.np = n;
     }
     __syncwarp();
     return c.np;
 }
 
-// Clip by the plane n.x <= d of generator sid.  Returns 1 changed, 0
-// unchanged, < 0 error (all lanes).
-template <class C>
-__device__ int wclip(C &c, const Frame &F, double nx, double ny, double nz, double d, int sid)
+// The FP32 side of vertex (v, ev) of the plane P = (n, d): f = n.v - d from
+// the FP32 vertex and plane differs from the exact f by at most |n|_1 ev (the
+// vertex) + 5u (|n|_1 |v|_1 + |d|) (the plane's rounding and the FP32 sum);
+// beyond the band, twice that, its sign is exact.
+__device__ __forceinline__ void side32(float4 P, float nsum, float4 v, float ev, bool &out, bool &unsure)
 {
+    const float ff = fmaf(P.x, v.x, fmaf(P.y, v.y, fmaf(P.z, v.z, -P.w)));
+    const float band = 2.f * (nsum * ev + 5.f * U32 * (nsum * v.w + fabsf(P.w)));
+    out = ff > band;
+    unsure = !out && !(ff < -band);
+}
+
+// Clip by the bisector P (rounded to FP32) of generator sid.  Returns 1
+// changed, 0 unchanged, < 0 error (all lanes).
+template <class C>
+__device__ int wclip(C &c, const Frame &F, float4 P, int sid)
+{
+    constexpr int IT = (C::MAXV + 31) / 32;
     const int lane = threadIdx.x & 31;
     const int cur = c.cur, nxt = cur ^ 1, nt = c.nt;
-    // The side of each vertex: f = n.v - d in FP32 from the FP32 vertex and
-    // plane.  It differs from the exact f by at most |n|_1 ev (the vertex) +
-    // 5u (|n|_1 |v|_1 + |d|) (the plane's rounding and the FP32 sum); beyond
-    // the band, twice that, its sign is exact.  Inside the band the vertex's
+    // The side of each vertex (side32).  Inside the band the vertex's
     // FP64 meet decides, with the warp converged on the few that need it; a
     // vertex within 1e-13 of the plane's scale (above the rounding of the
     // FP64 meet and value) counts as on the plane and is kept, so that a plane
     // through existing vertices, as in degenerate (lattice) site sets, cuts
     // no sliver off.
-    const float4 P = make_float4(em::f32_rn(nx), em::f32_rn(ny), em::f32_rn(nz), em::f32_rn(d));
     const float nsum = fabsf(P.x) + fabsf(P.y) + fabsf(P.z);
-    bool any = false;
-    for (int base = 0; base < nt; base += 32) {
-        const int t = base + lane;
+    unsigned mo[IT];   // the removed vertices
+    unsigned any = 0;
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+        mo[it] = 0;
+        if (it * 32 >= nt) continue;
+        const int t = it * 32 + lane;
         bool out = false, unsure = false;
-        if (t < nt) {
-            const float *vf = c.vf[t];
-            const float ff = fmaf(P.x, vf[0], fmaf(P.y, vf[1], fmaf(P.z, vf[2], -P.w)));
-            const float band = 2.f * (nsum * c.ev[t] + 5.f * U32 * (nsum * vf[3] + fabsf(P.w)));
-            out = ff > band;
-            unsure = !out && !(ff < -band);
-        }
+        if (t < nt) side32(P, nsum, c.vf[t], c.ev[t], out, unsure);
         if (__any_sync(0xffffffffu, unsure)) {
             if (unsure) {
-                double x, y, z;
+                double nx, ny, nz, d, x, y, z;
+                bisector(F.xs, F.ys, F.zs, sid, F.gx, F.gy, F.gz, nx, ny, nz, d);
                 meet64(c, F, t, x, y, z);
-                out = nx * x + ny * y + nz * z - d > 1e-13 * (double)(nsum * c.vf[t][3] + fabsf(P.w));
+                out = nx * x + ny * y + nz * z - d > 1e-13 * (double)(nsum * c.vf[t].w + fabsf(P.w));
             }
         }
-        if (t < nt) c.side[t] = out ? 1 : 0;
-        any = any || out;
+        mo[it] = __ballot_sync(0xffffffffu, out);
+        any |= mo[it];
     }
-    if (!__any_sync(0xffffffffu, any)) return 0;
-    __syncwarp();
+    if (!any) return 0;
     if (c.np >= WMAXP && wcompact(c) >= WMAXP) return -emv::VS_CAPACITY;
     const int q = c.np;
     // new index of every kept vertex (order kept), in side[]; removed ones listed
     int nk = 0, nout = 0;
-    for (int base = 0; base < nt; base += 32) {
-        const int t = base + lane;
-        const bool in = t < nt;
-        const bool keep = in && !c.side[t];
-        const bool out = in && !keep;
-        const unsigned mk = __ballot_sync(0xffffffffu, keep), mo = __ballot_sync(0xffffffffu, out);
-        if (in) c.side[t] = keep ? (uint8_t)(nk + __popc(mk & lanemask_lt())) : (uint8_t)0xff;
-        if (out) c.out_list[nout + __popc(mo & lanemask_lt())] = (uint8_t)t;
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+        const int t = it * 32 + lane, left = nt - it * 32;
+        const unsigned in = left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1u : 0u), mk = in & ~mo[it];
+        if (t < nt) {
+            const bool out = (mo[it] >> lane) & 1u;
+            c.side[t] = out ? (uint8_t)0xff : (uint8_t)(nk + __popc(mk & lanemask_lt()));
+            if (out) c.out_list[nout + __popc(mo[it] & lanemask_lt())] = (uint8_t)t;
+        }
         nk += __popc(mk);
-        nout += __popc(mo);
+        nout += __popc(mo[it]);
     }
     __syncwarp();
     if (nk == 0) return -emv::VS_TOPOLOGY;
@@ -294,23 +307,30 @@ __device__ int wclip(C &c, const Frame &F, double nx, double ny, double nz, doub
     // across a cut edge are set below); the FP32 copy and its bound move
     // within their buffer (a vertex never moves up, and each round reads
     // before it writes)
-    for (int base = 0; base < nt; base += 32) {
-        const int t = base + lane;
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+        if (it * 32 >= nt) continue;
+        const int t = it * 32 + lane;
         const int pos = t < nt ? c.side[t] : 0xff;
-        float vfk[4], evk = 0.f;
+        float4 v;
+        float e = 0.f;
         if (pos != 0xff) {
-            for (int e = 0; e < 3; ++e) {
-                c.tri[nxt][pos][e] = c.tri[cur][t][e];
-                const int s_ = c.adj[cur][t][e];
-                c.adj[nxt][pos][e] = s_ < nt ? c.side[s_] : (uint8_t)0xff;
+            v = c.vf[t];
+            e = c.ev[t];
+            const uint32_t w = c.adj[cur][t];
+            uint32_t a = 0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int n = byte_of(w, k);
+                a |= (uint32_t)(n < nt ? c.side[n] : (uint8_t)0xff) << (8 * k);
             }
-            for (int e = 0; e < 4; ++e) vfk[e] = c.vf[t][e];
-            evk = c.ev[t];
+            c.tri[nxt][pos] = c.tri[cur][t];
+            c.adj[nxt][pos] = a;
         }
         __syncwarp();
         if (pos != 0xff) {
-            for (int e = 0; e < 4; ++e) c.vf[pos][e] = vfk[e];
-            c.ev[pos] = evk;
+            c.vf[pos] = v;
+            c.ev[pos] = e;
         }
         __syncwarp();
     }
@@ -324,23 +344,23 @@ __device__ int wclip(C &c, const Frame &F, double nx, double ny, double nz, doub
     for (int base = 0; base < 3 * nout; base += 32) {
         const int k = base + lane;
         bool newv = false;
-        uint8_t a = 0, b = 0;
-        int upos = 0, ue = 0;
+        int a = 0, b = 0, upos = 0, ue = 0;
         float px = 0.f, py = 0.f, pz = 0.f, perr = INFINITY;
         if (k < 3 * nout) {
             const int t = c.out_list[k / 3], e = k % 3;
-            a = c.tri[cur][t][e];
-            b = c.tri[cur][t][(e + 1) % 3];
-            const int u = c.adj[cur][t][e];
+            const uint32_t tw = c.tri[cur][t];
+            a = byte_of(tw, e);
+            b = byte_of(tw, e == 2 ? 0 : e + 1);
+            const int u = byte_of(c.adj[cur][t], e);
             if (u >= nt) {
                 bad = true;   // inconsistent neighbours: reported, never followed
             } else if (c.side[u] != 0xff) {
                 newv = true;
                 upos = c.side[u];
                 // the edge of u that is (b, a)
-                const uint8_t *tu = c.tri[cur][u];
-                ue = (tu[0] == b && tu[1] == a) ? 0 : ((tu[1] == b && tu[2] == a) ? 1 : 2);
-                bad = bad || !(tu[ue] == b && tu[(ue + 1) % 3] == a);
+                const uint32_t tu = c.tri[cur][u];
+                ue = (byte_of(tu, 0) == b && byte_of(tu, 1) == a) ? 0 : ((byte_of(tu, 1) == b && byte_of(tu, 2) == a) ? 1 : 2);
+                bad = bad || !(byte_of(tu, ue) == b && byte_of(tu, ue == 2 ? 0 : ue + 1) == a);
                 meet32(c.pf[a], c.pf[b], P, px, py, pz, perr);
             }
         }
@@ -350,10 +370,7 @@ __device__ int wclip(C &c, const Frame &F, double nx, double ny, double nz, doub
                 double PL[3][4];
                 plane64(F, c.sid[a], PL[0][0], PL[0][1], PL[0][2], PL[0][3]);
                 plane64(F, c.sid[b], PL[1][0], PL[1][1], PL[1][2], PL[1][3]);
-                PL[2][0] = nx;
-                PL[2][1] = ny;
-                PL[2][2] = nz;
-                PL[2][3] = d;
+                bisector(F.xs, F.ys, F.zs, sid, F.gx, F.gy, F.gz, PL[2][0], PL[2][1], PL[2][2], PL[2][3]);
                 double x, y, z;
                 meet64p(PL[0], PL[1], PL[2], x, y, z);
                 px = (float)x;
@@ -369,34 +386,32 @@ __device__ int wclip(C &c, const Frame &F, double nx, double ny, double nz, doub
         if (newv) {
             int pos = nn + __popc(m & lanemask_lt());
             if (pos < C::MAXV) {
-                c.tri[nxt][pos][0] = a;
-                c.tri[nxt][pos][1] = b;
-                c.tri[nxt][pos][2] = (uint8_t)q;
-                c.adj[nxt][pos][0] = (uint8_t)upos;
-                c.adj[nxt][upos][ue] = (uint8_t)pos;
-                c.vf[pos][0] = px;
-                c.vf[pos][1] = py;
-                c.vf[pos][2] = pz;
-                c.vf[pos][3] = fabsf(px) + fabsf(py) + fabsf(pz);
+                c.tri[nxt][pos] = (uint32_t)a | (uint32_t)b << 8 | (uint32_t)q << 16;
+                c.adj[nxt][pos] = (uint32_t)upos;   // the edges on the new face follow
+                reinterpret_cast<uint8_t *>(&c.adj[nxt][upos])[ue] = (uint8_t)pos;
+                c.vf[pos] = make_float4(px, py, pz, fabsf(px) + fabsf(py) + fabsf(pz));
                 c.ev[pos] = perr;
+                c.of_a[a] = (uint8_t)pos;
+                c.of_b[b] = (uint8_t)pos;
             }
         }
         nn += __popc(m);
     }
     __syncwarp();
     // the new vertices around the new face q: (a, b, q) meets the one whose
-    // a is this b across (b, q), and the one whose b is this a across (q, a)
+    // a is this b across (b, q), and the one whose b is this a across (q, a);
+    // entries of of_a and of_b that this clip did not write are told apart by
+    // their vertex
     if (nn <= C::MAXV)
         for (int n = nk + lane; n < nn; n += 32) {
-            const uint8_t an = c.tri[nxt][n][0], bn = c.tri[nxt][n][1];
-            int m1 = -1, m2 = -1;
-            for (int o = nk; o < nn; ++o) {
-                if (c.tri[nxt][o][0] == bn) m1 = o;
-                if (c.tri[nxt][o][1] == an) m2 = o;
+            const uint32_t tw = c.tri[nxt][n];
+            const int an = byte_of(tw, 0), bn = byte_of(tw, 1);
+            const int m1 = c.of_a[bn], m2 = c.of_b[an];
+            bad = bad || m1 < nk || m1 >= nn || m2 < nk || m2 >= nn;
+            if (!bad) {
+                bad = byte_of(c.tri[nxt][m1], 0) != bn || byte_of(c.tri[nxt][m2], 1) != an;
+                c.adj[nxt][n] |= (uint32_t)m1 << 8 | (uint32_t)m2 << 16;
             }
-            bad = bad || m1 < 0 || m2 < 0;
-            c.adj[nxt][n][1] = (uint8_t)(m1 < 0 ? 0 : m1);
-            c.adj[nxt][n][2] = (uint8_t)(m2 < 0 ? 0 : m2);
         }
     if (__any_sync(0xffffffffu, bad)) return -emv::VS_TOPOLOGY;
     if (nn > C::MAXV) return -emv::VS_CAPACITY;
@@ -422,8 +437,8 @@ __device__ double wrmax2(const C &c, const Frame &F)
     float r2 = 0.f;
     bool fp64 = false;
     for (int t = lane; t < c.nt; t += 32) {
-        const float *v = c.vf[t];
-        const float r = sqrtf(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]) + 1.7320509f * c.ev[t];
+        const float4 v = c.vf[t];
+        const float r = sqrtf(v.x * v.x + v.y * v.y + v.z * v.z) + 1.7320509f * c.ev[t];
         if (isfinite(r)) r2 = fmaxf(r2, r * r);
         else fp64 = true;
     }
@@ -567,13 +582,14 @@ __device__ int gather_cutting(C &c, const em::ChunkTree &T, const double *__rest
         // lies within 1.8 ev of vf, which moves both squared distances by at
         // most 3.6 ev (|d| + |g|) + 6.5 ev^2)
         for (int t = 0; t < nt; ++t) {
-            const float vx = c.vf[t][0], vy = c.vf[t][1], vz = c.vf[t][2];
+            const float4 v = c.vf[t];
+            const float vx = v.x, vy = v.y, vz = v.z;
             float dx = fmaxf(fmaxf(lx - vx, vx - hx), 0.f);
             float dy = fmaxf(fmaxf(ly - vy, vy - hy), 0.f);
             float dz = fmaxf(fmaxf(lz - vz, vz - hz), 0.f);
             const float db = dx * dx + dy * dy + dz * dz;
             const float dg = vx * vx + vy * vy + vz * vz;
-            const float S = gabs + babs + c.vf[t][3];
+            const float S = gabs + babs + v.w;
             const float e = c.ev[t];
             if (!(db >= dg + 1e-5f * S * S + 7.2f * e * S + 6.5f * e * e)) return true;
         }
@@ -614,9 +630,9 @@ __device__ int gather_cutting(C &c, const em::ChunkTree &T, const double *__rest
                     const float df = 0.5f * rf * rf, rabs = fabsf(ex) + fabsf(ey) + fabsf(ez);
                     bool maybe = false;
                     for (int t = 0; t < nt && !maybe; ++t) {
-                        const float *vf = c.vf[t];
-                        const float ff = ex * vf[0] + ey * vf[1] + ez * vf[2] - df;
-                        maybe = !(ff <= -(1e-5f * (gabs + rabs + vf[3]) * (vf[3] + rabs) + rabs * c.ev[t]));
+                        const float4 vf = c.vf[t];
+                        const float ff = ex * vf.x + ey * vf.y + ez * vf.z - df;
+                        maybe = !(ff <= -(1e-5f * (gabs + rabs + vf.w) * (vf.w + rabs) + rabs * c.ev[t]));
                     }
                     hit = maybe;
                 }
@@ -665,35 +681,44 @@ __device__ int gather_cutting(C &c, const em::ChunkTree &T, const double *__rest
     return n > WCAND ? -1 : n;
 }
 
-// Clip by the first nc (sorted) candidates.  A candidate first meets an FP32
-// side test on the rounded positions (the same margin as in gather_cutting,
-// above the rounding of the coordinates and the vertex bounds): one that
-// every vertex clears cuts nothing and costs no FP64 work.
+// Clip by the first nc (sorted) candidates, 32 at a time: each lane forms its
+// candidate's FP64 bisector and rounds it to FP32 (an FP64 instruction costs
+// the pipe the same on 32 lanes as on one), and the warp clips by the rounded
+// planes in turn; the FP64 one is formed again by the few side tests and meets
+// that need it.  After the first 32 few candidates still cut: each lane tests
+// its own against the cell's vertices, and only those that some vertex does
+// not clear are taken up (a cell only shrinks, so the test stays valid).
 template <class C>
-__device__ int clip_sorted(C &c, const em::ChunkTree &T, const Frame &F, int64_t n, int nc)
+__device__ int clip_sorted(C &c, const Frame &F, int64_t n, int nc)
 {
     const int lane = threadIdx.x & 31;
-    const float gxf = (float)F.gx, gyf = (float)F.gy, gzf = (float)F.gz;
-    const float gabs = fabsf(gxf) + fabsf(gyf) + fabsf(gzf);
-    for (int i = 0; i < nc; ++i) {
-        int k = c.u.k.cid[i];
-        if (k < 0 || k >= n) return emv::VS_BOUNDS;
-        {
-            const float4 pk = T.pts[k];
-            const float ex = pk.x - gxf, ey = pk.y - gyf, ez = pk.z - gzf;
-            const float df = 0.5f * (ex * ex + ey * ey + ez * ez), rabs = fabsf(ex) + fabsf(ey) + fabsf(ez);
-            bool maybe = false;
-            for (int t = lane; t < c.nt; t += 32) {
-                const float *vf = c.vf[t];
-                const float ff = ex * vf[0] + ey * vf[1] + ez * vf[2] - df;
-                maybe = maybe || !(ff <= -(1e-5f * (gabs + rabs + vf[3]) * (vf[3] + rabs) + rabs * c.ev[t]));
-            }
-            if (!__any_sync(0xffffffffu, maybe)) continue;
-        }
+    for (int i0 = 0; i0 < nc; i0 += 32) {
+        const int k = i0 + lane < nc ? c.u.k.cid[i0 + lane] : 0;
+        if (__any_sync(0xffffffffu, k < 0 || k >= n)) return emv::VS_BOUNDS;
         double nx, ny, nz, d;
         bisector(F.xs, F.ys, F.zs, k, F.gx, F.gy, F.gz, nx, ny, nz, d);
-        int r = wclip(c, F, nx, ny, nz, d, k);
-        if (r < 0) return -r;
+        const float4 P = make_float4(em::f32_rn(nx), em::f32_rn(ny), em::f32_rn(nz), em::f32_rn(d));
+        bool maybe = i0 + lane < nc;
+        if (i0 > 0) {
+            const float nsum = fabsf(P.x) + fabsf(P.y) + fabsf(P.z);
+            bool cut = false;
+            const int nt = c.nt;
+            for (int t = 0; t < nt; ++t) {
+                bool out, unsure;
+                side32(P, nsum, c.vf[t], c.ev[t], out, unsure);
+                cut = cut || out || unsure;
+            }
+            maybe = maybe && cut;
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, maybe);
+        while (todo) {
+            const int l = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const float4 Q = make_float4(__shfl_sync(0xffffffffu, P.x, l), __shfl_sync(0xffffffffu, P.y, l),
+                                         __shfl_sync(0xffffffffu, P.z, l), __shfl_sync(0xffffffffu, P.w, l));
+            const int r = wclip(c, F, Q, __shfl_sync(0xffffffffu, k, l));
+            if (r < 0) return -r;
+        }
     }
     return 0;
 }
@@ -784,7 +809,7 @@ __device__ int wbuild_cell(C &c, const em::ChunkTree &T, const Frame &F, int64_t
         }
         if (m > 0) {
             sort_cand(c, m);
-            int st = clip_sorted(c, T, F, n, m);
+            int st = clip_sorted(c, F, n, m);
             if (st) return status | st;
         }
         skip2 = hi2;
@@ -818,16 +843,18 @@ __device__ int wface_loop(const C &c, int q, uint8_t *loop, int maxn)
 {
     const int cur = c.cur, nt = c.nt;
     int t0 = -1;
-    for (int t = 0; t < nt && t0 < 0; ++t)
-        if (c.tri[cur][t][0] == q || c.tri[cur][t][1] == q || c.tri[cur][t][2] == q) t0 = t;
+    for (int t = 0; t < nt && t0 < 0; ++t) {
+        const uint32_t w = c.tri[cur][t];
+        if (byte_of(w, 0) == q || byte_of(w, 1) == q || byte_of(w, 2) == q) t0 = t;
+    }
     if (t0 < 0) return 0;
     int n = 0, t = t0;
     do {
         if (n >= maxn) return -1;
         loop[n++] = (uint8_t)t;
-        const uint8_t *tr = c.tri[cur][t];
-        const int r = tr[0] == q ? 0 : (tr[1] == q ? 1 : 2);
-        const int nx = c.adj[cur][t][(r + 2) % 3];
+        const uint32_t w = c.tri[cur][t];
+        const int r = byte_of(w, 0) == q ? 0 : (byte_of(w, 1) == q ? 1 : 2);
+        const int nx = byte_of(c.adj[cur][t], r == 0 ? 2 : r - 1);
         if (nx >= nt) return -1;
         t = nx;
     } while (t != t0);
