@@ -740,7 +740,7 @@ __global__ void __launch_bounds__(32 * FW_WARPS) k_map_fp64(
 // every weight above 1e-14 / tol, absolute 1e-14 below); so does a face plane
 // through P.
 //
-// 24.06 M pairs of the 1e6-particle cloud: 71.2 ms (3.4e8 pairs/s), against
+// 24.06 M pairs of the 1e6-particle cloud: 70.2 ms (3.4e8 pairs/s), against
 // 111 ms with 4- and 8-point rules in s = asinh(tau / A), an asinh per
 // segment and an exponential per node, the two sides of every edge queued in
 // turn, and correctly rounded or subnormal-safe reciprocals; the error against
@@ -776,6 +776,7 @@ static_assert(MQ_CHUNK % 32 == 0, "whole rounds of the warp");
 constexpr int MQ_NOSLOT = 4095;
 static_assert(MQ_SLOTS * 56 < MQ_NOSLOT, "slot indices fit in 12 bits");
 constexpr unsigned FULL_MASK = 0xffffffffu;
+constexpr unsigned MQ_EDGE_DONE = 32;   // mq_edge: every segment of the edge is queued
 
 struct SegQueue {
     float ts[MQ_SLOTS][32], len[MQ_SLOTS][32], A[MQ_SLOTS][32];
@@ -965,8 +966,8 @@ __device__ __forceinline__ void mq_push(SegQueue &q, int lane, int sl, int piece
 // A range across the foot is taken as its two sides.  Most edges yield one
 // segment: the loop runs once for each that the warp's busiest lane has, with
 // the lanes converged.
-__device__ __forceinline__ void mq_edge(SegQueue &q, int lane, int &cnt, emq::ff T0x, emq::ff T1x, float dT, float A,
-                                        emq::ff B2, float sc, const FaceState &fs, bool tilde, emq::ff &acc,
+__device__ __forceinline__ void mq_edge(SegQueue &q, int lane, int &cnt, unsigned &queued, emq::ff T0x,
+                                        emq::ff T1x, float dT, float A, emq::ff B2, float sc, const FaceState &fs, bool tilde, emq::ff &acc,
                                         float &mag)
 {
     const float A2 = A * A, B2f = fmaxf(B2.hi, A2);
@@ -984,16 +985,20 @@ __device__ __forceinline__ void mq_edge(SegQueue &q, int lane, int &cnt, emq::ff
     // the other side's: piece 1 up to x1, piece 2 from t1 to x2
     const float x1 = fminf(xo, t1), x2 = fminf(xo, t2);
     unsigned todo = (e1 > 0.f ? 1u : 0u) | (e2 > s2 ? 2u : 0u) | (x1 > 0.f ? 4u : 0u) | (x2 > t1 ? 8u : 0u);
-    while (todo) {
+    const bool first = queued == 0;   // the part beyond 2h is added once
+    todo &= ~queued;
+    while (todo && cnt < MQ_SLOTS) {
         const int k = __ffs(todo) - 1;
         todo &= todo - 1;
+        queued |= 1u << k;
         // start: ua, ua + s2, 0 or t1
         emq::ff t = emq::ff_two_sum(k < 2 ? ua : 0.f, k == 1 ? s2 : (k == 3 ? t1 : 0.f));
         if (k < 2) t.lo += ualo;
         const float len = k == 0 ? e1 : (k == 1 ? e2 - s2 : (k == 2 ? x1 : x2 - t1));
         mq_push(q, lane, cnt++, (k & 1) ? 2 : 1, t, len, A, A2, B2f, B2, sc, fs, tilde);
     }
-    if (tilde) {   // beyond 2h: K~(Q) = 0, the integrand is -K~(R) >= 0
+    queued = todo ? queued | 16u : MQ_EDGE_DONE;
+    if (tilde && first) {   // beyond 2h: K~(Q) = 0, the integrand is -K~(R) >= 0
         auto far = [&](float u, float l) {   // tau from u over length l
             const emq::ff v = emq::ff_two_prod(sc, -fs.KR * emq::angle_q1(l * A, fmaf(u, u + l, A2)));
             const emq::ff s = emq::ff_two_sum(acc.hi, v.hi);
@@ -1129,8 +1134,9 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_map_fp32(int64_t npairs, c
                 }
             }
         }
-        for (int ei = 0; last ? ei == 0 : __any_sync(FULL_MASK, ei < ne); ++ei) {
-            if (ei < ne) {
+        unsigned queued = 0;   // of the lane's current edge: the segments queued (mq_edge)
+        for (int ei = 0; last ? ei == 0 : __any_sync(FULL_MASK, ei < ne);) {
+            if (ei < ne && queued != MQ_EDGE_DONE) {
                 // edge geometry in float-float (see quad32.cuh): A, T0, T1 and
                 // B^2, each rounded once to FP32 where it is used so
                 const EdgeF H = edge_f[e0 + ei], Lo = edge_fl[e0 + ei];
@@ -1147,14 +1153,24 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_map_fp32(int64_t npairs, c
                     // signed factor: D/pi, face orientation, side of the edge line
                     // (T1 >= T0: the edge runs along its direction)
                     const float sc = fs.sign * (a.hi > 0.f ? 1.f : -1.f) * fs.Df * 0.31830988618379067154f;
-                    mq_edge(q, lane, cnt, t0, t1, lh.hi, A, emq::ff_add(fs.D2, emq::ff_mul(a, a)), sc, fs, tilde,
-                            acc_far, mag_far);
+                    mq_edge(q, lane, cnt, queued, t0, t1, lh.hi, A, emq::ff_add(fs.D2, emq::ff_mul(a, a)), sc, fs,
+                            tilde, acc_far, mag_far);
+                } else {
+                    queued = MQ_EDGE_DONE;
                 }
             }
-            // an edge queues at most four segments
-            if (__any_sync(FULL_MASK, cnt > (last ? 0 : MQ_SLOTS - 4))) {
+            // almost every edge queues one or two segments: the queue is evaluated
+            // when a lane has no room for two (71.2 ms on the 1e6-particle cloud where
+            // it was when a lane had no room for four, 70.2 so), and an edge that
+            // found too little room is taken up again after that
+            const bool rest = ei < ne && queued != MQ_EDGE_DONE;
+            if (__any_sync(FULL_MASK, rest || cnt > (last ? 0 : MQ_SLOTS - 2))) {
                 mq_flush(q, lane, cnt, acc, mag);
                 cnt = 0;
+            }
+            if (!__any_sync(FULL_MASK, rest)) {
+                queued = 0;
+                ++ei;
             }
         }
         if (last) break;
