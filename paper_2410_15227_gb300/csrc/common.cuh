@@ -120,7 +120,6 @@ struct em_tree {
     int64_t n = 0, nnode = 0;
     int depth = 0;
     double box[6];
-    std::vector<int64_t> level_off;   // host: first node index of each level, + end
     int32_t *perm = nullptr;          // [n] original index of Morton position k
     uint64_t *key = nullptr;          // [n] sorted keys
     double *xs = nullptr, *ys = nullptr, *zs = nullptr, *ms = nullptr;   // [n] Morton order
