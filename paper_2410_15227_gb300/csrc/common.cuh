@@ -198,7 +198,8 @@ struct em_pairs {
 // ---- helpers shared across translation units -------------------------------------
 
 int em_prepare_cells(em_ctx *ctx, em_voronoi *v);                 // derived geometry
-int em_build_pair_index(em_ctx *ctx, em_pairs *pr);               // CSR offsets + transpose
+int em_build_transpose(em_ctx *ctx, em_pairs *pr, int *bad);      // (i, j) order
+int em_build_pair_index(em_ctx *ctx, em_pairs *pr);               // CSR offsets + transpose of a given list
 // map_exact's body (mapping.cu); d_flag_buf / d_flag_count: optional scratch
 // for the mixed pass's flagged pairs (npairs entries), read back by map_batch
 int em_map_exact_impl(em_ctx *ctx, const em_pairs *pr, const double *d_x, const double *d_y, const double *d_z,

@@ -249,22 +249,16 @@ __global__ void k_check_within_cell(int64_t n, const int32_t *__restrict__ pi, c
     if (k > 0 && pj[k] == pj[k - 1] && pi[k] <= pi[k - 1]) atomicOr(bad, 8);
 }
 
-int em_build_pair_index(em_ctx *ctx, em_pairs *pr)
+// The (i, j)-ordered transpose of a list ordered by (j, i): a stable sort by i.
+// bad (or null): raised where the sorted keys are out of range.
+int em_build_transpose(em_ctx *ctx, em_pairs *pr, int *bad)
 {
-    int64_t n = pr->npairs;
+    const int64_t n = pr->npairs;
     DevArena tmp(ctx->stream, true);
-    int *bad;
-    EM_TRY(tmp.alloc(&bad, 1));
-    EM_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream));
-    EM_TRY(pr->mem.alloc(&pr->cell_pair_off, pr->ncell + 1));
+    int *ignored;
+    EM_TRY(tmp.alloc(&ignored, 1));
     EM_TRY(pr->mem.alloc(&pr->part_pair_off, pr->np + 1));
     EM_TRY(pr->mem.alloc(&pr->part_pair_idx, n));
-    k_segment_offsets<<<em_grid(n + 1, 256), 256, 0, ctx->stream>>>(n, pr->pair_j, pr->ncell, pr->cell_pair_off, bad);
-    EM_LAUNCHED(ctx);
-    if (n) {
-        k_check_within_cell<<<em_grid(n, 256), 256, 0, ctx->stream>>>(n, pr->pair_i, pr->pair_j, pr->np, bad);
-        EM_LAUNCHED(ctx);
-    }
     uint32_t *keys;
     EM_TRY(tmp.alloc(&keys, n));
     if (n) {
@@ -273,8 +267,27 @@ int em_build_pair_index(em_ctx *ctx, em_pairs *pr)
         EM_TRY(em_sort_pairs_u32(ctx, keys, pr->part_pair_idx, n, em_nbits((uint64_t)pr->np)));
     }
     k_segment_offsets<<<em_grid(n + 1, 256), 256, 0, ctx->stream>>>(n, (const int32_t *)keys, pr->np,
-                                                                      pr->part_pair_off, bad);
+                                                                      pr->part_pair_off, bad ? bad : ignored);
     EM_LAUNCHED(ctx);
+    return EM_OK;
+}
+
+// Cell offsets and transpose of a given list, which is checked.
+int em_build_pair_index(em_ctx *ctx, em_pairs *pr)
+{
+    int64_t n = pr->npairs;
+    DevArena tmp(ctx->stream, true);
+    int *bad;
+    EM_TRY(tmp.alloc(&bad, 1));
+    EM_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), ctx->stream));
+    EM_TRY(pr->mem.alloc(&pr->cell_pair_off, pr->ncell + 1));
+    k_segment_offsets<<<em_grid(n + 1, 256), 256, 0, ctx->stream>>>(n, pr->pair_j, pr->ncell, pr->cell_pair_off, bad);
+    EM_LAUNCHED(ctx);
+    if (n) {
+        k_check_within_cell<<<em_grid(n, 256), 256, 0, ctx->stream>>>(n, pr->pair_i, pr->pair_j, pr->np, bad);
+        EM_LAUNCHED(ctx);
+    }
+    EM_TRY(em_build_transpose(ctx, pr, bad));
     int hbad = 0;
     EM_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     EM_CUDA(cudaStreamSynchronize(ctx->stream));

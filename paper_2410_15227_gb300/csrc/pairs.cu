@@ -13,9 +13,10 @@
 // inside the band take the exact FP64 test, which also sets the near flag.
 // The pair set is therefore the FP64 predicate's.  Hits are compacted with a
 // warp ballot into a per-warp buffer and written, unordered, at positions
-// reserved with an atomic add; one radix sort by (j, i) puts them in order.
-// 24.06 M pairs of the 1e6-particle cloud, index included: 8.4 ms, against 12.1
-// with every candidate of the ball classified.
+// reserved with an atomic add; a second kernel orders each cell's (k_place_pairs).
+// 24.06 M pairs of the 1e6-particle cloud, index included: 7.1 ms, against 8.4
+// with a radix sort of all hits and 12.1 with every candidate of the ball
+// classified as well.
 #include <vector>
 
 #include "common.cuh"
@@ -108,17 +109,32 @@ __device__ __forceinline__ float cell_dist2_f32(float rx, float ry, float rz, in
 
 // One warp per cell: candidate particles from the sphere hierarchy, FP32
 // classification, exact FP64 test inside the band, ballot compaction into a
-// per-warp buffer in shared memory.  A full (or the final) buffer is written
-// at a position reserved with one atomic add on the global hit counter, as
-// (j << 32 | i) keys and near flags: unordered, the caller sorts them.  Hits
+// per-warp buffer in shared memory.  A full (or the final) buffer is written as
+// a segment of the cell's hits at a position reserved with one atomic add on
+// the global hit counter, each the particle index with the near flag in bit 31,
+// and linked to the cell's other segments: k_place_pairs orders them.  Hits
 // past the capacity are counted but not written; the caller then repeats the
 // pass with room for all of them.
 #ifndef EM_PAIRS_WARPS
 #define EM_PAIRS_WARPS 1   // warps (cells) per block: a finished cell frees its slot at once (12.4 against 13.0 ms with 4)
 #endif
 constexpr int PAIRS_WARPS = EM_PAIRS_WARPS;
-constexpr int PAIRS_BUF = 128;   // hits a warp holds before writing them out
+constexpr int PAIRS_BUF = 256;   // hits a warp holds before writing them out
 constexpr int PAIRS_LEAVES = 2;  // 32-particle leaves a walk reads together
+
+// The hits of a pass: `hits` in segments, seg[s] = {first hit, count, the
+// cell's previous segment or -1, the cell}, head[j] the cell's last segment.
+// A segment that is not a cell's last holds more than PAIRS_BUF - 32 hits, so
+// ncell + capacity / (PAIRS_BUF - 32) + 1 segments suffice.  counter: hits
+// found, segments, 1 if some cell has more than PLACE_MAX hits.
+struct HitLists {
+    unsigned long long *counter;
+    int64_t capacity;
+    uint32_t *hits;
+    int4 *seg;
+    int32_t *head;
+};
+constexpr int PLACE_MAX = 2048;   // hits of a cell that k_place_pairs orders in shared memory
 
 __global__ void __launch_bounds__(32 * PAIRS_WARPS)
     k_cell_pairs(int64_t cell0, int64_t cell1, em::ChunkTree T, const double *__restrict__ xs, const double *__restrict__ ys,
@@ -126,11 +142,9 @@ __global__ void __launch_bounds__(32 * PAIRS_WARPS)
                  const double *__restrict__ gen, const double *__restrict__ radius, const int64_t *__restrict__ cfo,
                  const int64_t *__restrict__ fvo, const PlaneD *__restrict__ plane, const EdgeD *__restrict__ edge,
                  const PlaneF *__restrict__ plane_f, const EdgeF *__restrict__ edge_f, float margin,
-                 unsigned long long *__restrict__ counter, int64_t capacity, uint64_t *__restrict__ keys,
-                 int32_t *__restrict__ nearf, int64_t *__restrict__ cell_count)
+                 HitLists H, int64_t *__restrict__ cell_count)
 {
-    __shared__ uint64_t buf_key[PAIRS_WARPS][PAIRS_BUF];
-    __shared__ int32_t buf_near[PAIRS_WARPS][PAIRS_BUF];
+    __shared__ uint32_t buf[PAIRS_WARPS][PAIRS_BUF];
     __shared__ int32_t cand_buf[PAIRS_WARPS][64];   // a chunk adds at most 32 to fewer than 32
     const int w = threadIdx.x >> 5;
     int64_t j = cell0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
@@ -138,17 +152,19 @@ __global__ void __launch_bounds__(32 * PAIRS_WARPS)
     const int lane = threadIdx.x & 31;
     int nb = 0;   // hits in the warp's buffer (the same on every lane)
     int64_t ncell_hits = 0;
+    int32_t head = -1;   // the cell's last segment
     // with capacity 0 the pass only counts (cell_count)
     auto write_out = [&]() {
-        if (capacity > 0) {
+        if (H.capacity > 0) {
             unsigned long long at = 0;
-            if (lane == 0) at = atomicAdd(counter, (unsigned long long)nb);
+            if (lane == 0) at = atomicAdd(&H.counter[0], (unsigned long long)nb);
             at = __shfl_sync(0xffffffffu, at, 0);
-            for (int t = lane; t < nb; t += 32) {
-                const unsigned long long pos = at + (unsigned long long)t;
-                if (pos < (unsigned long long)capacity) {
-                    keys[pos] = buf_key[w][t];
-                    nearf[pos] = buf_near[w][t];
+            if (at + (unsigned long long)nb <= (unsigned long long)H.capacity) {
+                for (int t = lane; t < nb; t += 32) H.hits[at + t] = buf[w][t];
+                if (lane == 0) {
+                    const int32_t seg = (int32_t)atomicAdd(&H.counter[1], 1ull);   // < nseg: see HitLists
+                    H.seg[seg] = make_int4((int)at, nb, head, (int)j);
+                    head = seg;
                 }
             }
         }
@@ -168,8 +184,7 @@ __global__ void __launch_bounds__(32 * PAIRS_WARPS)
         if (nb + __popc(b) > PAIRS_BUF) write_out();
         if (hit) {
             const int pos = nb + __popc(b & ((1u << lane) - 1u));
-            buf_key[w][pos] = ((uint64_t)j << 32) | (uint32_t)perm[k];
-            buf_near[w][pos] = nearb ? 1 : 0;
+            buf[w][pos] = (uint32_t)perm[k] | (nearb ? 0x80000000u : 0u);
         }
         __syncwarp();
         nb += __popc(b);
@@ -280,7 +295,75 @@ __global__ void __launch_bounds__(32 * PAIRS_WARPS)
         });
     if (nc > 0) classify(lane < nc ? cb[lane] : 0, lane < nc);
     if (nb > 0) write_out();
-    if (cell_count && lane == 0) cell_count[j - cell0] = ncell_hits;
+    if (lane == 0) {
+        if (cell_count) cell_count[j] = ncell_hits;
+        if (H.capacity > 0) {
+            H.head[j] = head;
+            if (ncell_hits > PLACE_MAX) atomicMax(&H.counter[2], 1ull);
+        }
+    }
+}
+
+// One warp per cell: its segments into shared memory, ordered by particle
+// (bitonic, the near flag carried below the index), and out at the cell's
+// offset.  A radix sort of all hits by (cell, particle) took 7 passes over 12 B
+// a pair, 1.7 ms for 24 M pairs; the cells need only be ordered within.
+__global__ void __launch_bounds__(32) k_place_pairs(HitLists H, const int64_t *__restrict__ off,
+                                                    int32_t *__restrict__ pi, int32_t *__restrict__ pj,
+                                                    uint8_t *__restrict__ nearo)
+{
+    extern __shared__ uint32_t v[];
+    const int64_t j = blockIdx.x;
+    const int lane = threadIdx.x;
+    const int64_t o = off[j];
+    const int n = (int)(off[j + 1] - o);
+    if (n == 0) return;
+    int at = 0;
+    for (int32_t s = H.head[j]; s >= 0;) {
+        const int4 g = H.seg[s];
+        for (int t = lane; t < g.y; t += 32) {
+            const uint32_t h = H.hits[g.x + t];
+            v[at + t] = (h << 1) | (h >> 31);
+        }
+        at += g.y;
+        s = g.z;
+    }
+    int len = 2;
+    while (len < n) len <<= 1;
+    for (int t = n + lane; t < len; t += 32) v[t] = 0xffffffffu;
+    __syncwarp();
+    for (int size = 2; size <= len; size <<= 1)
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            for (int t = lane; t < len / 2; t += 32) {
+                const int lo = 2 * t - (t & (stride - 1)), hi = lo + stride;
+                const uint32_t a = v[lo], b = v[hi];
+                if ((a > b) == ((lo & size) == 0)) {
+                    v[lo] = b;
+                    v[hi] = a;
+                }
+            }
+            __syncwarp();
+        }
+    for (int t = lane; t < n; t += 32) {
+        const uint32_t a = v[t];
+        pi[o + t] = (int32_t)(a >> 1);
+        pj[o + t] = (int32_t)j;
+        nearo[o + t] = (uint8_t)(a & 1u);
+    }
+}
+
+// For cells of more than PLACE_MAX hits: every hit as a (cell, particle) key
+// and its near flag, one warp per segment, for a radix sort.
+__global__ void k_segment_keys(int64_t nseg, HitLists H, uint64_t *__restrict__ keys, int32_t *__restrict__ nearf)
+{
+    const int64_t s = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (s >= nseg) return;
+    const int4 g = H.seg[s];
+    for (int t = threadIdx.x & 31; t < g.y; t += 32) {
+        const uint32_t h = H.hits[g.x + t];
+        keys[g.x + t] = ((uint64_t)(uint32_t)g.w << 32) | (h & 0x7fffffffu);
+        nearf[g.x + t] = (int32_t)(h >> 31);
+    }
 }
 
 __global__ void k_split_keys(int64_t n, const uint64_t *__restrict__ keys, const int32_t *__restrict__ nearf,
@@ -377,12 +460,11 @@ static int prepare_particles(em_ctx *ctx, DevArena &tmp, int64_t np, const doubl
 }
 
 static void launch_cell_pairs(em_ctx *ctx, const PairParticles &P, const em_voronoi *v, int64_t cell0, int64_t cell1,
-                              unsigned long long *counter, int64_t capacity, uint64_t *keys, int32_t *nearf,
-                              int64_t *cell_count)
+                              const HitLists &H, int64_t *cell_count)
 {
     k_cell_pairs<<<em_grid((cell1 - cell0) * 32, 32 * PAIRS_WARPS), 32 * PAIRS_WARPS, 0, ctx->stream>>>(
         cell0, cell1, P.T, P.xs, P.ys, P.zs, P.hs, P.perm, v->gen, v->radius, v->cell_face_off, v->face_vert_off,
-        v->plane, v->edge, v->plane_f, v->edge_f, P.margin, counter, capacity, keys, nearf, cell_count);
+        v->plane, v->edge, v->plane_f, v->edge_f, P.margin, H, cell_count);
 }
 
 // The pairs of the cells [cell0, cell1) into pr (all of v's cells indexed,
@@ -401,34 +483,35 @@ static int find_pairs_impl(em_ctx *ctx, int64_t np, const double *x, const doubl
     // one pass into an unsorted buffer sized from the hint (or the last call,
     // or a guess on the first), repeated once with the exact size if it
     // overflowed
-    unsigned long long *counter;
-    EM_TRY(tmp.alloc(&counter, 1));
-    int64_t capacity = capacity_hint > 0 ? capacity_hint
-                                         : (ctx->pairs_hint > 0 ? ctx->pairs_hint : 64 * np + (1 << 20));
+    HitLists H;
+    int64_t *count;
+    EM_TRY(tmp.alloc(&H.counter, 3));
+    EM_TRY(tmp.alloc(&H.head, nc));
+    EM_TRY(tmp.alloc(&count, nc + 1));
+    EM_CUDA(cudaMemsetAsync(count, 0, (nc + 1) * sizeof(int64_t), st));
+    H.capacity = capacity_hint > 0 ? capacity_hint : (ctx->pairs_hint > 0 ? ctx->pairs_hint : 64 * np + (1 << 20));
     int64_t total = 0;
-    uint64_t *keys = nullptr;
-    int32_t *nearf = nullptr;
+    unsigned long long found[3] = {0, 0, 0};
     for (int attempt = 0; attempt < 2; ++attempt) {
         DevArena buf(st, true);   // released on an early return
-        EM_TRY(buf.alloc(&keys, capacity));
-        EM_TRY(buf.alloc(&nearf, capacity));
-        EM_CUDA(cudaMemsetAsync(counter, 0, sizeof *counter, st));
+        EM_TRY(buf.alloc(&H.hits, H.capacity));
+        EM_TRY(buf.alloc(&H.seg, nc + H.capacity / (PAIRS_BUF - 32) + 1));
+        EM_CUDA(cudaMemsetAsync(H.counter, 0, 3 * sizeof *H.counter, st));
         if (cell1 > cell0) {
-            launch_cell_pairs(ctx, P, v, cell0, cell1, counter, capacity, keys, nearf, nullptr);
+            launch_cell_pairs(ctx, P, v, cell0, cell1, H, count);
             EM_LAUNCHED(ctx);
         }
-        unsigned long long hits = 0;
-        EM_CUDA(cudaMemcpyAsync(&hits, counter, sizeof hits, cudaMemcpyDeviceToHost, st));
+        EM_CUDA(cudaMemcpyAsync(found, H.counter, sizeof found, cudaMemcpyDeviceToHost, st));
         EM_CUDA(cudaStreamSynchronize(st));
-        total = (int64_t)hits;
-        if (total <= capacity || total >= INT32_MAX) {
+        total = (int64_t)found[0];
+        if (total <= H.capacity || total >= INT32_MAX) {
             // keep the buffers: they belong to the call's scratch from here on
             for (void *q : buf.ptrs) tmp.ptrs.push_back(q);
             buf.ptrs.clear();
             break;
         }
         buf.release();
-        capacity = total;
+        H.capacity = total;
     }
     if (total >= INT32_MAX) {
         em_set_error("find_pairs: %lld pairs exceed the 2^31 limit of one pair list", (long long)total);
@@ -436,15 +519,28 @@ static int find_pairs_impl(em_ctx *ctx, int64_t np, const double *x, const doubl
     }
     if (capacity_hint <= 0) ctx->pairs_hint = total + total / 8 + 1024;
     pr->npairs = total;
-    if (total) EM_TRY(em_sort_pairs_u64(ctx, keys, nearf, total, 32 + em_nbits((uint64_t)nc)));
     EM_TRY(pr->mem.alloc(&pr->pair_i, total));
     EM_TRY(pr->mem.alloc(&pr->pair_j, total));
     EM_TRY(pr->mem.alloc(&pr->near, total));
-    if (total) {
+    EM_TRY(pr->mem.alloc(&pr->cell_pair_off, nc + 1));
+    EM_TRY(em_exclusive_scan_i64(ctx, count, pr->cell_pair_off, nc + 1));
+    if (total && !found[2]) {
+        // the cells outside [cell0, cell1) have no pairs, and no head to read
+        k_place_pairs<<<(unsigned)nc, 32, PLACE_MAX * sizeof(uint32_t), st>>>(H, pr->cell_pair_off, pr->pair_i,
+                                                                             pr->pair_j, pr->near);
+        EM_LAUNCHED(ctx);
+    } else if (total) {
+        uint64_t *keys;
+        int32_t *nearf;
+        EM_TRY(tmp.alloc(&keys, total));
+        EM_TRY(tmp.alloc(&nearf, total));
+        k_segment_keys<<<em_grid((int64_t)found[1] * 32, 256), 256, 0, st>>>((int64_t)found[1], H, keys, nearf);
+        EM_LAUNCHED(ctx);
+        EM_TRY(em_sort_pairs_u64(ctx, keys, nearf, total, 32 + em_nbits((uint64_t)nc)));
         k_split_keys<<<em_grid(total, 256), 256, 0, st>>>(total, keys, nearf, pr->pair_i, pr->pair_j, pr->near);
         EM_LAUNCHED(ctx);
     }
-    return em_build_pair_index(ctx, pr);
+    return em_build_transpose(ctx, pr, nullptr);
 }
 
 static int new_pairs(em_ctx *ctx, int64_t np, const double *d_x, const double *d_y, const double *d_z,
@@ -482,7 +578,7 @@ EM_EXPORT int find_pairs_plan(em_ctx *ctx, int64_t np, const double *d_x, const 
     if (nc > 0) {
         int64_t *d_cnt;
         EM_TRY(tmp.alloc(&d_cnt, nc));
-        launch_cell_pairs(ctx, P, v, 0, nc, nullptr, 0, nullptr, nullptr, d_cnt);
+        launch_cell_pairs(ctx, P, v, 0, nc, HitLists{nullptr, 0, nullptr, nullptr, nullptr}, d_cnt);
         EM_LAUNCHED(ctx);
         EM_CUDA(cudaMemcpyAsync(cnt.data(), d_cnt, nc * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
         EM_CUDA(cudaStreamSynchronize(st));
