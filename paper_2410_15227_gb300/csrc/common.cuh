@@ -73,11 +73,17 @@ void em_set_error(const char *fmt, ...);
 cudaMemPool_t em_device_pool(int device);
 
 // Stream-ordered device allocations released together (handle memory, or a
-// call's scratch when used as a local).
+// call's scratch when used as a local).  Requests of up to kSmall bytes share
+// slabs of kSlab: a stage makes 20 to 30 of them, and with small snapshots the
+// pool's calls, 1 to 2 us each under one lock for all streams, were a tenth of
+// its time.
 struct DevArena {
+    static constexpr size_t kAlign = 256, kSmall = 1 << 18, kSlab = 1 << 20;
     cudaStream_t stream = nullptr;
     std::vector<void *> ptrs;
     bool scoped = false;
+    char *slab = nullptr;   // the rest of the last slab
+    size_t left = 0;
 
     explicit DevArena(cudaStream_t s = nullptr, bool scoped_ = false) : stream(s), scoped(scoped_) {}
     DevArena(const DevArena &) = delete;
@@ -91,17 +97,17 @@ struct DevArena {
     int alloc(T **p, size_t n)
     {
         *p = nullptr;
-        size_t bytes = (n ? n : 1) * sizeof(T);
-        int dev = 0;
-        cudaMemPool_t pool = cudaGetDevice(&dev) == cudaSuccess ? em_device_pool(dev) : nullptr;
-        cudaError_t e = pool ? cudaMallocFromPoolAsync((void **)p, bytes, pool, stream)
-                             : cudaMallocAsync((void **)p, bytes, stream);
-        if (e != cudaSuccess) {
-            em_set_error("device allocation of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
-            cudaGetLastError();
-            return EM_ENOMEM;
+        const size_t bytes = ((n ? n : 1) * sizeof(T) + kAlign - 1) / kAlign * kAlign;
+        if (bytes > kSmall) return block((void **)p, bytes);
+        if (left < bytes) {
+            void *s;
+            if (block(&s, kSlab) != EM_OK) return block((void **)p, bytes);
+            slab = (char *)s;
+            left = kSlab;
         }
-        ptrs.push_back((void *)*p);
+        *p = (T *)slab;
+        slab += bytes;
+        left -= bytes;
         return EM_OK;
     }
 
@@ -109,6 +115,24 @@ struct DevArena {
     {
         for (void *p : ptrs) cudaFreeAsync(p, stream);
         ptrs.clear();
+        slab = nullptr;
+        left = 0;
+    }
+
+private:
+    int block(void **p, size_t bytes)
+    {
+        *p = nullptr;
+        int dev = 0;
+        cudaMemPool_t pool = cudaGetDevice(&dev) == cudaSuccess ? em_device_pool(dev) : nullptr;
+        cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, stream) : cudaMallocAsync(p, bytes, stream);
+        if (e != cudaSuccess) {
+            em_set_error("device allocation of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
+            cudaGetLastError();
+            return EM_ENOMEM;
+        }
+        ptrs.push_back(*p);
+        return EM_OK;
     }
 };
 
