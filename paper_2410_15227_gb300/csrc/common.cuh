@@ -180,8 +180,9 @@ struct __align__(16) PlaneF {
 struct __align__(16) EdgeD {
     double mx, my, mz, cm, ex, ey, ez, ce, L, pad;
 };
+// (In FP32 m and e by component, for packed arithmetic on both: quad32.cuh.)
 struct __align__(16) EdgeF {
-    float mx, my, mz, cm, ex, ey, ez, ce, L, pad0, pad1, pad2;
+    float mx, ex, my, ey, mz, ez, cm, ce, L, pad0, pad1, pad2;
 };
 
 struct em_voronoi {

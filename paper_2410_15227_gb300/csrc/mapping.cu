@@ -1153,11 +1153,10 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_map_fp32(int64_t npairs, c
                 // edge geometry in float-float (see quad32.cuh): A, T0, T1 and
                 // B^2, each rounded once to FP32 where it is used so
                 const EdgeF H = edge_f[e0 + ei], Lo = edge_fl[e0 + ei];
-                const emq::ff ah = emq::ff_offset_dot(H.cm, Lo.cm, H.mx, Lo.mx, H.my, Lo.my, H.mz, Lo.mz, rxx, ryy, rzz);
-                const emq::ff a = emq::ff_mul(ah, ihh);
+                const emq::ff2 at = emq::ff2_mul(emq::edge_offsets(H, Lo, rxx, ryy, rzz), ihh);
+                const emq::ff a{at.hi.x, at.lo.x};
                 if (a.hi != 0.f) {
-                    const emq::ff th = emq::ff_offset_dot(H.ce, Lo.ce, H.ex, Lo.ex, H.ey, Lo.ey, H.ez, Lo.ez, rxx, ryy, rzz);
-                    const emq::ff t0 = emq::ff_mul(th, ihh);
+                    const emq::ff t0{at.hi.y, at.lo.y};
                     const emq::ff lh = emq::ff_mul(emq::ff{H.L, Lo.L}, ihh);   // L/h
                     const emq::ff t1 = emq::ff_add(t0, lh);
                     // A below 1e-18 h changes the integral by ~1e-18 relative and would
