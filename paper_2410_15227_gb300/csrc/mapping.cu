@@ -1268,6 +1268,68 @@ __device__ __forceinline__ void pair_sums(int64_t k0, int64_t k1, const int32_t 
     }
 }
 
+// The same sums by ROW_LANES lanes per row: each gathers one pair of eight, four
+// groups of eight in flight, and all of them add the row's terms in order, as
+// they come by shuffles.  For a short list of rows, where a thread per row
+// leaves most SMs without one and waits on its row's chain of gathers: 1,000
+// rows of about 90 pairs, k_map_back 63 -> 25.5 us, k_particle_wsum 27 -> 16.  Called with the warp converged, n = 0 for
+// a lane without a row.
+constexpr int ROW_LANES = 8;
+template <bool WITH_F>
+__device__ __forceinline__ void group_sums(int64_t k0, int n, const int32_t *__restrict__ idx,
+                                           const int32_t *__restrict__ pj, const double *__restrict__ w,
+                                           const double *__restrict__ f, double &num, double &den)
+{
+    constexpr int U = 4;
+    const int l = threadIdx.x & (ROW_LANES - 1);
+    int nmax = n;
+#pragma unroll
+    for (int o = ROW_LANES; o < 32; o <<= 1) nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
+    for (int c = 0; c < nmax; c += U * ROW_LANES) {
+        int32_t q[U];
+        double wq[U], pq[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) q[u] = c + u * ROW_LANES + l < n ? __ldg(idx + k0 + c + u * ROW_LANES + l) : -1;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            wq[u] = q[u] >= 0 ? __ldg(w + q[u]) : 0.0;
+            pq[u] = WITH_F && q[u] >= 0 ? __dmul_rn(wq[u], __ldg(f + __ldg(pj + q[u]))) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+#pragma unroll
+            for (int t = 0; t < ROW_LANES; ++t) {
+                const double wt = __shfl_sync(0xffffffffu, wq[u], t, ROW_LANES);
+                const double pt = WITH_F ? __shfl_sync(0xffffffffu, pq[u], t, ROW_LANES) : 0.0;
+                if (c + u * ROW_LANES + t < n) {
+                    if (WITH_F) num = __dadd_rn(num, pt);
+                    den = __dadd_rn(den, wt);
+                }
+            }
+        }
+    }
+}
+
+// Row i's sums in one pass, by one thread or by ROW_LANES lanes; false for a
+// thread that has none to write.
+template <bool GROUP, bool WITH_F>
+__device__ __forceinline__ bool row_sums(int64_t np, const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
+                                         const int32_t *__restrict__ pj, const double *__restrict__ w,
+                                         const double *__restrict__ f, int64_t &i, double &num, double &den)
+{
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    num = den = 0.0;
+    i = GROUP ? t / ROW_LANES : t;
+    if (!GROUP) {
+        if (i >= np) return false;
+        pair_sums<WITH_F>(off[i], off[i + 1], idx, pj, w, f, num, den);
+        return true;
+    }
+    const int64_t k0 = i < np ? off[i] : 0;
+    group_sums<WITH_F>(k0, i < np ? (int)(off[i + 1] - k0) : 0, idx, pj, w, f, num, den);
+    return i < np && threadIdx.x % ROW_LANES == 0;
+}
+
 // The same sums for many pairs, in two passes.  One thread walking a row of
 // the transpose is bound by the longest row's chain of dependent gathers
 // (3,832 pairs where the mean is 234: about 1.0 of k_map_back's 1.5 ms on the
@@ -1396,15 +1458,27 @@ static int two_pass_sums(em_ctx *ctx, const em_pairs *pr, const double *w, const
     return EM_OK;
 }
 
-// u_i = sum_j w_ij (ascending j), one thread per particle
+// u_i = sum_j w_ij (ascending j)
+template <bool GROUP>
 __global__ void k_particle_wsum(int64_t np, const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
                                 const double *__restrict__ w, double *__restrict__ u)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= np) return;
-    double num = 0.0, s = 0.0;
-    pair_sums<false>(off[i], off[i + 1], idx, nullptr, w, nullptr, num, s);
-    u[i] = s;
+    int64_t i;
+    double num, den;
+    if (row_sums<GROUP, false>(np, off, idx, nullptr, w, nullptr, i, num, den)) u[i] = den;
+}
+
+// One pass: ROW_LANES lanes per row where the rows have at least as many pairs
+// on average, else a thread per row.
+static bool lanes_per_row(const em_pairs *pr) { return pr->npairs >= ROW_LANES * pr->np; }
+template <class... K, class... A>
+static void launch_rows(em_ctx *ctx, const em_pairs *pr, void (*group)(K...), void (*single)(K...), A... args)
+{
+    if (lanes_per_row(pr))
+        group<<<em_grid(pr->np * ROW_LANES, 64), 64, 0, ctx->stream>>>(pr->np, pr->part_pair_off, pr->part_pair_idx,
+                                                                       args...);
+    else
+        single<<<em_grid(pr->np, 256), 256, 0, ctx->stream>>>(pr->np, pr->part_pair_off, pr->part_pair_idx, args...);
 }
 
 // The FP32 pass in launch shape `variant` (see MQ_VARIANT_*).
@@ -1520,8 +1594,7 @@ int em_map_exact_impl(em_ctx *ctx, const em_pairs *pr, const double *d_x, const 
     bool summed = !(d_wsum_out && pr->np);
     if (!summed && !fixed) EM_TRY(two_pass_sums<0>(ctx, pr, d_w_out, nullptr, d_wsum_out, nullptr, &summed));
     if (!summed) {
-        k_particle_wsum<<<em_grid(pr->np, 256), 256, 0, ctx->stream>>>(pr->np, pr->part_pair_off, pr->part_pair_idx,
-                                                                        d_w_out, d_wsum_out);
+        launch_rows(ctx, pr, k_particle_wsum<true>, k_particle_wsum<false>, d_w_out, d_wsum_out);
         EM_LAUNCHED(ctx);
     }
     return EM_OK;
@@ -1655,18 +1728,17 @@ EM_EXPORT int map_exact_noalloc(em_ctx *ctx, const em_pairs *pr, const double *d
 // Inverse mapping
 // ---------------------------------------------------------------------------
 
+template <bool GROUP>
 __global__ void k_map_back(int64_t np, const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
                            const int32_t *__restrict__ pj, const double *__restrict__ w,
                            const double *__restrict__ f_cell, double *__restrict__ f_out)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= np) return;
-    // ascending j, each product and each sum rounded on its own (pair_sums),
+    // ascending j, each product and each sum rounded on its own (row_sums),
     // so that equal weights give bit-identical results on any implementation
     // that sums in the same order
-    double num = 0.0, den = 0.0;
-    pair_sums<true>(off[i], off[i + 1], idx, pj, w, f_cell, num, den);
-    f_out[i] = num / den;
+    int64_t i;
+    double num, den;
+    if (row_sums<GROUP, true>(np, off, idx, pj, w, f_cell, i, num, den)) f_out[i] = num / den;
 }
 
 // every SPH particle takes the value of the pseudo-particle it belongs to
@@ -1682,16 +1754,17 @@ __global__ void k_inherit(int64_t npseudo, const int32_t *__restrict__ first, co
 
 // The two sums of map_back per particle, added into num and den (ascending
 // j, every product and sum rounded on its own, as k_map_back).
+template <bool GROUP>
 __global__ void k_map_back_sums(int64_t np, const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
                                 const int32_t *__restrict__ pj, const double *__restrict__ w,
                                 const double *__restrict__ f_cell, double *__restrict__ num, double *__restrict__ den)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= np) return;
-    double a = 0.0, b = 0.0;
-    pair_sums<true>(off[i], off[i + 1], idx, pj, w, f_cell, a, b);
-    num[i] = __dadd_rn(num[i], a);
-    den[i] = __dadd_rn(den[i], b);
+    int64_t i;
+    double a, b;
+    if (row_sums<GROUP, true>(np, off, idx, pj, w, f_cell, i, a, b)) {
+        num[i] = __dadd_rn(num[i], a);
+        den[i] = __dadd_rn(den[i], b);
+    }
 }
 
 EM_EXPORT int map_back_sums(em_ctx *ctx, const em_pairs *pr, const double *d_w, const double *d_f_cell,
@@ -1701,9 +1774,7 @@ EM_EXPORT int map_back_sums(em_ctx *ctx, const em_pairs *pr, const double *d_w, 
     bool done = pr->np == 0;
     if (!done) EM_TRY(two_pass_sums<2>(ctx, pr, d_w, d_f_cell, d_num, d_den, &done));
     if (!done) {
-        k_map_back_sums<<<em_grid(pr->np, 256), 256, 0, ctx->stream>>>(pr->np, pr->part_pair_off,
-                                                                        pr->part_pair_idx, pr->pair_j, d_w,
-                                                                        d_f_cell, d_num, d_den);
+        launch_rows(ctx, pr, k_map_back_sums<true>, k_map_back_sums<false>, pr->pair_j, d_w, d_f_cell, d_num, d_den);
         EM_LAUNCHED(ctx);
     }
     return EM_OK;
@@ -1730,8 +1801,7 @@ EM_EXPORT int map_back(em_ctx *ctx, const em_pairs *pr, const double *d_w, const
     bool done = pr->np == 0;
     if (!done) EM_TRY(two_pass_sums<1>(ctx, pr, d_w, d_f_cell, d_f_out, nullptr, &done));
     if (!done) {
-        k_map_back<<<em_grid(pr->np, 256), 256, 0, ctx->stream>>>(pr->np, pr->part_pair_off, pr->part_pair_idx,
-                                                                   pr->pair_j, d_w, d_f_cell, d_f_out);
+        launch_rows(ctx, pr, k_map_back<true>, k_map_back<false>, pr->pair_j, d_w, d_f_cell, d_f_out);
         EM_LAUNCHED(ctx);
     }
     if (inherit && ps->n) {
