@@ -43,30 +43,35 @@ __global__ void k_prepare_faces(int64_t nface, int64_t ncell, const double *__re
     plane[f] = PlaneD{nx, ny, nz, c};
     // hi and low parts: the plane = hi + lo to about 2^-48 relative (float-float)
     PlaneF F, G;
-    split_df(nx, F.x, G.x);
-    split_df(ny, F.y, G.y);
-    split_df(nz, F.z, G.z);
-    split_df(c, F.w, G.w);
+    split_all<4>({nx, ny, nz, c}, {&F.x, &F.y, &F.z, &F.w}, {&G.x, &G.y, &G.z, &G.w});
     plane_f[f] = F;
     plane_fl[f] = G;
     cell_of_face[f] = (int32_t)j;
     for (int64_t k = v0; k < v1; ++k) face_of_fv[k] = (int32_t)f;
 }
 
-// Per face-vertex k (one thread each, so that the records are written by
-// adjacent threads): the edge from vertex k to the next vertex of its face, in
-// the generator's frame, as FP64 and FP32 hi/lo records.  The cell radius is
-// the largest |V - g| over its vertices: every vertex raises its cell's r^2
-// with an atomic max on the bit pattern (non-negative doubles order like their
-// bits), so the result does not depend on the order.
-__global__ void k_prepare_edges(int64_t nfv, const double *__restrict__ gen, const int64_t *__restrict__ fvo,
-                                const double *__restrict__ verts, const double *__restrict__ normals,
-                                const int32_t *__restrict__ face_of_fv, const int32_t *__restrict__ cell_of_face,
-                                unsigned long long *__restrict__ r2bits, EdgeD *__restrict__ edge,
-                                EdgeF *__restrict__ edge_f, EdgeF *__restrict__ edge_fl)
+// Per face-vertex k, one thread each: the edge from vertex k to the next vertex
+// of its face, in the generator's frame, as FP64 and FP32 hi/lo records.  Bound
+// by the FP64 pipe (about 36 operations a vertex): 21.2 M vertices 3.01 ms with
+// the splits' conversions if-converted (split.cuh: split_all) and the records
+// written 80 and 48 B apart, 2.08 ms so.  The records, 176 B a thread, are put
+// together in shared memory and written out by adjacent threads.  The cell
+// radius is the largest |V - g| over its
+// vertices: the largest of a warp's lanes on one cell (a cell's vertices lie
+// together) raises the cell's r^2 with an atomic max on the bit pattern
+// (non-negative doubles order like their bits), so the result does not depend
+// on the order.
+constexpr int PREP_EDGES = 128;   // threads per block
+__global__ void __launch_bounds__(PREP_EDGES)
+    k_prepare_edges(int64_t nfv, const double *__restrict__ gen, const int64_t *__restrict__ fvo,
+                    const double *__restrict__ verts, const double *__restrict__ normals,
+                    const int32_t *__restrict__ face_of_fv, const int32_t *__restrict__ cell_of_face,
+                    unsigned long long *__restrict__ r2bits, EdgeD *__restrict__ edge, EdgeF *__restrict__ edge_f,
+                    EdgeF *__restrict__ edge_fl)
 {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= nfv) return;
+    __shared__ EdgeD sd[PREP_EDGES];
+    __shared__ EdgeF sf[2][PREP_EDGES];
+    const int64_t kb = blockIdx.x * (int64_t)PREP_EDGES, k = min(kb + (int64_t)threadIdx.x, nfv - 1);
     const int64_t f = face_of_fv[k];
     const int64_t j = cell_of_face[f];
     const double gx = gen[3 * j], gy = gen[3 * j + 1], gz = gen[3 * j + 2];
@@ -78,15 +83,16 @@ __global__ void k_prepare_edges(int64_t nfv, const double *__restrict__ gen, con
     double q = ax * ax + ay * ay + az * az;
     double ex = bx - ax, ey = by - ay, ez = bz - az;
     // L and 1/L from one reciprocal square root: an FP32 seed (on the bits,
-    // split.cuh) and two FP64 Newton steps, within about an ulp, for fewer
-    // FP64 instructions than a square root and a division
+    // split.cuh) and the series of (1 - e)^(-1/2), e = 1 - s2 r0^2 of at most
+    // 2^-20, to e^2 (the next term is below 2^-61), within about an ulp, for
+    // fewer FP64 instructions than a square root and a division
     const double s2 = ex * ex + ey * ey + ez * ez;
     double L = 0.0;
     EdgeD E;
-    if (s2 > 1e-30 && s2 < 1e30) {   // the seed in float's normal range
-        double r = f64_of(rsqrtf(f32_rn(s2)));
-        r = r * (1.5 - 0.5 * s2 * r * r);
-        r = r * (1.5 - 0.5 * s2 * r * r);
+    const int e2 = __double2hiint(s2) >> 20;   // the exponent: s2 >= 0 (a comparison would issue at the FP64 rate)
+    if (e2 >= 1023 - 99 && e2 < 1023 + 99) {   // the seed in float's normal range
+        const double r0 = f64_of(rsqrtf(f32_of(s2))), e = fma(-(s2 * r0), r0, 1.0);
+        const double r = fma(r0 * e, fma(0.375, e, 0.5), r0);
         L = s2 * r;
         ex *= r;
         ey *= r;
@@ -107,23 +113,35 @@ __global__ void k_prepare_edges(int64_t nfv, const double *__restrict__ gen, con
     E.cm = E.mx * ax + E.my * ay + E.mz * az;
     E.ce = ex * ax + ey * ay + ez * az;
     E.pad = 0.0;
-    edge[k] = E;
+    sd[threadIdx.x] = E;
     // hi and low parts: E = hi + lo to about 2^-48 relative (float-float)
     EdgeF F, G;
-    split_df(E.mx, F.mx, G.mx);
-    split_df(E.my, F.my, G.my);
-    split_df(E.mz, F.mz, G.mz);
-    split_df(E.cm, F.cm, G.cm);
-    split_df(E.ex, F.ex, G.ex);
-    split_df(E.ey, F.ey, G.ey);
-    split_df(E.ez, F.ez, G.ez);
-    split_df(E.ce, F.ce, G.ce);
-    split_df(E.L, F.L, G.L);
+    split_all<9>({E.mx, E.my, E.mz, E.cm, E.ex, E.ey, E.ez, E.ce, E.L},
+                 {&F.mx, &F.my, &F.mz, &F.cm, &F.ex, &F.ey, &F.ez, &F.ce, &F.L},
+                 {&G.mx, &G.my, &G.mz, &G.cm, &G.ex, &G.ey, &G.ez, &G.ce, &G.L});
     F.pad0 = F.pad1 = F.pad2 = 0.f;
     G.pad0 = G.pad1 = G.pad2 = 0.f;
-    edge_f[k] = F;
-    edge_fl[k] = G;
-    atomicMax(r2bits + j, (unsigned long long)__double_as_longlong(q));
+    sf[0][threadIdx.x] = F;
+    sf[1][threadIdx.x] = G;
+    // the last threads past nfv repeat its vertex: they change no maximum
+    const int lane = threadIdx.x & 31;
+    unsigned long long qb = (unsigned long long)__double_as_longlong(q);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long qo = __shfl_down_sync(0xffffffffu, qb, o);
+        const int jo = __shfl_down_sync(0xffffffffu, (int)j, o);
+        if (lane + o < 32 && jo == (int)j) qb = max(qb, qo);
+    }
+    const int jp = __shfl_up_sync(0xffffffffu, (int)j, 1);
+    if (lane == 0 || jp != (int)j) atomicMax(r2bits + j, qb);
+    __syncthreads();
+    const int n = (int)min((int64_t)PREP_EDGES, nfv - kb);
+    constexpr int ND = sizeof(EdgeD) / 16, NF = sizeof(EdgeF) / 16;
+    for (int i = threadIdx.x; i < n * ND; i += PREP_EDGES) ((float4 *)(edge + kb))[i] = ((const float4 *)sd)[i];
+    for (int i = threadIdx.x; i < n * NF; i += PREP_EDGES) {
+        ((float4 *)(edge_f + kb))[i] = ((const float4 *)sf[0])[i];
+        ((float4 *)(edge_fl + kb))[i] = ((const float4 *)sf[1])[i];
+    }
 }
 
 __global__ void k_radius_finish(int64_t ncell, double *__restrict__ radius)
@@ -153,7 +171,7 @@ int em_prepare_cells(em_ctx *ctx, em_voronoi *v)
                 v->nface, v->ncell, v->gen, v->cell_face_off, v->face_vert_off, v->verts, v->normals, v->plane,
                 v->plane_f, v->plane_fl, face_of_fv, cell_of_face);
             EM_LAUNCHED(ctx);
-            k_prepare_edges<<<em_grid(v->nfv, 256), 256, 0, ctx->stream>>>(
+            k_prepare_edges<<<em_grid(v->nfv, PREP_EDGES), PREP_EDGES, 0, ctx->stream>>>(
                 v->nfv, v->gen, v->face_vert_off, v->verts, v->normals, face_of_fv, cell_of_face,
                 (unsigned long long *)v->radius, v->edge, v->edge_f, v->edge_fl);
             EM_LAUNCHED(ctx);

@@ -692,9 +692,7 @@ __device__ __forceinline__ bool solve_node(const em::ChunkTree &T, const Populat
     L.xa = px[a];
     L.ya = py[a];
     L.za = pz[a];
-    em::split_df(L.xa, L.xh, L.xl);
-    em::split_df(L.ya, L.yh, L.yl);
-    em::split_df(L.za, L.zh, L.zl);
+    em::split_all<3>({L.xa, L.ya, L.za}, {&L.xh, &L.yh, &L.zh}, {&L.xl, &L.yl, &L.zl});
     L.r = 0.f;
     L.n = -1;
     L.heavy = false;

@@ -9,22 +9,25 @@
 
 namespace em {
 
+// By the conversions themselves, for any x.
+__device__ __forceinline__ void split_cvt(double x, float &hi, float &lo)
+{
+    hi = __double2float_rn(x);
+    lo = __double2float_rn(x - (double)hi);
+}
+
 // The significand M (53 bits) of x = +-M 2^k, k = e - 1075, is cut after its
 // top 24 bits; hi keeps them, rounded to nearest even (a carry to 2^24 moves
 // hi to the next binade), and x - hi = +-R 2^k exactly with |R| <= 2^28.
 // (float)R rounds R to 24 bits as (float)(x - hi) would, and the power of two
 // scales it exactly, since |R 2^k| >= 2^-112 stays a normal float for
-// |x| >= 2^-60.  Smaller values, and those beyond float's range (with 0,
-// infinities and NaN), take the conversions.
-__device__ __forceinline__ void split_df(double x, float &hi, float &lo)
+// |x| >= 2^-60.  False, with hi and lo not set, for smaller values but zero and
+// those beyond float's range (with infinities and NaN): they take the
+// conversions.
+__device__ __forceinline__ bool split_bits(double x, float &hi, float &lo)
 {
     const unsigned long long u = (unsigned long long)__double_as_longlong(x);
     const int e = (int)((u >> 52) & 0x7ff);
-    if (e < 963 || e > 1149) {
-        hi = __double2float_rn(x);
-        lo = __double2float_rn(x - (double)hi);
-        return;
-    }
     const unsigned long long M = (u & 0xfffffffffffffull) | 0x10000000000000ull;
     unsigned long long Mh = M >> 29;
     const unsigned long long r = M & 0x1fffffffull;
@@ -33,9 +36,31 @@ __device__ __forceinline__ void split_df(double x, float &hi, float &lo)
     const unsigned sign = (unsigned)(u >> 63) << 31;
     const unsigned eh = (unsigned)(e - 1023 + 127);
     const unsigned hb = (Mh >> 24) ? (eh + 1u) << 23 : (eh << 23) | (unsigned)(Mh & 0x7fffffull);
-    hi = __uint_as_float(hb | sign);
+    const bool zero = (u << 1) == 0;
+    hi = __uint_as_float((zero ? 0u : hb) | sign);
     const float l = (float)R * __int_as_float((e - 1075 + 127) << 23);
-    lo = R == 0 ? 0.f : (sign ? -l : l);
+    lo = zero || R == 0 ? 0.f : (sign ? -l : l);
+    return zero || (e >= 963 && e <= 1149);
+}
+
+__device__ __forceinline__ void split_df(double x, float &hi, float &lo)
+{
+    if (!split_bits(x, hi, lo)) split_cvt(x, hi, lo);
+}
+
+// Several at once, one branch for all: behind a branch of its own each value's
+// few conversions are if-converted, and the FP64 pipe is given them for every
+// value, taken or not (k_prepare_edges: half of that pipe's time).
+template <int N>
+__device__ __forceinline__ void split_all(const double (&x)[N], float *const (&hi)[N], float *const (&lo)[N])
+{
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < N; ++i) ok = split_bits(x[i], *hi[i], *lo[i]) && ok;
+    if (!ok) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) split_cvt(x[i], *hi[i], *lo[i]);
+    }
 }
 
 // (float)x, rounded to nearest even, for 2^-100 <= |x| < 2^100 (the caller's
