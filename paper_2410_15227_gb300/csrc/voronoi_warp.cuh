@@ -153,7 +153,7 @@ template <class C>
 __device__ void meet64(const C &c, const Frame &F, int t, double &x, double &y, double &z)
 {
     double P[3][4];
-#pragma unroll
+#pragma unroll 1
     for (int e = 0; e < 3; ++e) plane64(F, c.sid[byte_of(c.tri[c.cur][t], e)], P[e][0], P[e][1], P[e][2], P[e][3]);
     meet64p(P[0], P[1], P[2], x, y, z);
 }
@@ -215,11 +215,14 @@ __device__ int wcompact(C &c)
     const int lane = threadIdx.x & 31;
     if (lane == 0) {
         int map[WMAXP];
+#pragma unroll 1
         for (int q = 0; q < c.np; ++q) map[q] = -1;
         const int cur = c.cur;
+#pragma unroll 1
         for (int t = 0; t < c.nt; ++t)
             for (int e = 0; e < 3; ++e) map[byte_of(c.tri[cur][t], e)] = 0;
         int n = 0;
+#pragma unroll 1
         for (int q = 0; q < c.np; ++q) {
             if (map[q] < 0) continue;
             map[q] = n;
@@ -227,6 +230,8 @@ __device__ int wcompact(C &c)
             c.pf[n] = c.pf[q];
             ++n;
         }
+#pragma unroll 1
+#pragma unroll 1
         for (int t = 0; t < c.nt; ++t) {
             const uint32_t w = c.tri[cur][t];
             c.tri[cur][t] = (uint32_t)map[byte_of(w, 0)] | (uint32_t)map[byte_of(w, 1)] << 8 | (uint32_t)map[byte_of(w, 2)] << 16;
@@ -254,7 +259,6 @@ __device__ __forceinline__ void side32(float4 P, float nsum, float4 v, float ev,
 template <class C>
 __device__ int wclip(C &c, const Frame &F, float4 P, int sid)
 {
-    constexpr int IT = (C::MAXV + 31) / 32;
     const int lane = threadIdx.x & 31;
     const int cur = c.cur, nxt = cur ^ 1, nt = c.nt;
     // The side of each vertex (side32).  Inside the band the vertex's
@@ -264,42 +268,54 @@ __device__ int wclip(C &c, const Frame &F, float4 P, int sid)
     // through existing vertices, as in degenerate (lattice) site sets, cuts
     // no sliver off.
     const float nsum = fabsf(P.x) + fabsf(P.y) + fabsf(P.z);
-    unsigned mo[IT];   // the removed vertices
-    unsigned any = 0;
-#pragma unroll
-    for (int it = 0; it < IT; ++it) {
-        mo[it] = 0;
-        if (it * 32 >= nt) continue;
+    // lane i holds round i's masks: the removed vertices, and those FP64 decides
+    unsigned mo = 0, mu = 0, any = 0, anyu = 0;
+#pragma unroll 1
+    for (int it = 0; it * 32 < nt; ++it) {
         const int t = it * 32 + lane;
         bool out = false, unsure = false;
         if (t < nt) side32(P, nsum, c.vf[t], c.ev[t], out, unsure);
-        if (__any_sync(0xffffffffu, unsure)) {
-            if (unsure) {
+        const unsigned bo = __ballot_sync(0xffffffffu, out && !unsure), bu = __ballot_sync(0xffffffffu, unsure);
+        if (lane == it) {
+            mo = bo;
+            mu = bu;
+        }
+        any |= bo;
+        anyu |= bu;
+    }
+    if (anyu) {
+#pragma unroll 1
+        for (int it = 0; it * 32 < nt; ++it) {
+            const int t = it * 32 + lane;
+            bool out = false;
+            if ((__shfl_sync(0xffffffffu, mu, it) >> lane) & 1u) {
                 double nx, ny, nz, d, x, y, z;
                 bisector(F.xs, F.ys, F.zs, sid, F.gx, F.gy, F.gz, nx, ny, nz, d);
                 meet64(c, F, t, x, y, z);
                 out = nx * x + ny * y + nz * z - d > 1e-13 * (double)(nsum * c.vf[t].w + fabsf(P.w));
             }
+            const unsigned b = __ballot_sync(0xffffffffu, out);
+            any |= b;
+            if (lane == it) mo |= b;
         }
-        mo[it] = __ballot_sync(0xffffffffu, out);
-        any |= mo[it];
     }
     if (!any) return 0;
     if (c.np >= WMAXP && wcompact(c) >= WMAXP) return -emv::VS_CAPACITY;
     const int q = c.np;
     // new index of every kept vertex (order kept), in side[]; removed ones listed
     int nk = 0, nout = 0;
-#pragma unroll
-    for (int it = 0; it < IT; ++it) {
+#pragma unroll 1
+    for (int it = 0; it * 32 < nt; ++it) {
         const int t = it * 32 + lane, left = nt - it * 32;
-        const unsigned in = left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1u : 0u), mk = in & ~mo[it];
+        const unsigned m = __shfl_sync(0xffffffffu, mo, it);
+        const unsigned mk = (left >= 32 ? 0xffffffffu : (1u << left) - 1u) & ~m;
         if (t < nt) {
-            const bool out = (mo[it] >> lane) & 1u;
+            const bool out = (m >> lane) & 1u;
             c.side[t] = out ? (uint8_t)0xff : (uint8_t)(nk + __popc(mk & lanemask_lt()));
-            if (out) c.out_list[nout + __popc(mo[it] & lanemask_lt())] = (uint8_t)t;
+            if (out) c.out_list[nout + __popc(m & lanemask_lt())] = (uint8_t)t;
         }
         nk += __popc(mk);
-        nout += __popc(mo[it]);
+        nout += __popc(m);
     }
     __syncwarp();
     if (nk == 0) return -emv::VS_TOPOLOGY;
@@ -307,9 +323,8 @@ __device__ int wclip(C &c, const Frame &F, float4 P, int sid)
     // across a cut edge are set below); the FP32 copy and its bound move
     // within their buffer (a vertex never moves up, and each round reads
     // before it writes)
-#pragma unroll
-    for (int it = 0; it < IT; ++it) {
-        if (it * 32 >= nt) continue;
+#pragma unroll 1
+    for (int it = 0; it * 32 < nt; ++it) {
         const int t = it * 32 + lane;
         const int pos = t < nt ? c.side[t] : 0xff;
         float4 v;
@@ -341,6 +356,7 @@ __device__ int wclip(C &c, const Frame &F, float4 P, int sid)
     // uncertain to be of use (planes near a common line)
     int nn = nk;
     bool bad = false;
+#pragma unroll 1
     for (int base = 0; base < 3 * nout; base += 32) {
         const int k = base + lane;
         bool newv = false;
@@ -403,6 +419,7 @@ __device__ int wclip(C &c, const Frame &F, float4 P, int sid)
     // entries of of_a and of_b that this clip did not write are told apart by
     // their vertex
     if (nn <= C::MAXV)
+#pragma unroll 1
         for (int n = nk + lane; n < nn; n += 32) {
             const uint32_t tw = c.tri[nxt][n];
             const int an = byte_of(tw, 0), bn = byte_of(tw, 1);
@@ -436,6 +453,7 @@ __device__ double wrmax2(const C &c, const Frame &F)
     const int lane = threadIdx.x & 31;
     float r2 = 0.f;
     bool fp64 = false;
+#pragma unroll 1
     for (int t = lane; t < c.nt; t += 32) {
         const float4 v = c.vf[t];
         const float r = sqrtf(v.x * v.x + v.y * v.y + v.z * v.z) + 1.7320509f * c.ev[t];
@@ -444,6 +462,7 @@ __device__ double wrmax2(const C &c, const Frame &F)
     }
     double q2 = (double)r2 * (1.0 + 1e-5);
     if (__any_sync(0xffffffffu, fp64)) {
+#pragma unroll 1
         for (int t = lane; t < c.nt; t += 32) {
             if (isfinite(c.ev[t])) continue;
             double x, y, z;
@@ -515,14 +534,19 @@ __device__ void sort_cand(C &c, int n)
     float *cd2 = c.u.k.cd2;
     int *cid = c.u.k.cid;
     int len = 2;
+#pragma unroll 1
     while (len < n) len <<= 1;
+#pragma unroll 1
     for (int i = n + lane; i < len; i += 32) {
         cd2[i] = INFINITY;
         cid[i] = 0x7fffffff;
     }
     __syncwarp();
+#pragma unroll 1
     for (int size = 2; size <= len; size <<= 1) {
+#pragma unroll 1
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
+#pragma unroll 1
             for (int i = lane; i < len / 2; i += 32) {
                 int lo = 2 * i - (i & (stride - 1));
                 int hi = lo + stride;
@@ -581,6 +605,7 @@ __device__ int gather_cutting(C &c, const em::ChunkTree &T, const double *__rest
         // some vertex nearer to the box than to the site (the exact vertex
         // lies within 1.8 ev of vf, which moves both squared distances by at
         // most 3.6 ev (|d| + |g|) + 6.5 ev^2)
+#pragma unroll 1
         for (int t = 0; t < nt; ++t) {
             const float4 v = c.vf[t];
             const float vx = v.x, vy = v.y, vz = v.z;
@@ -595,15 +620,13 @@ __device__ int gather_cutting(C &c, const em::ChunkTree &T, const double *__rest
         }
         return false;
     };
-    uint32_t mask[em::kMaxLevels + 1];
-    int64_t base[em::kMaxLevels + 1];
-    const int top = T.nlev;
+    // a level above the top, of one node, so that the box test has one call site
+    uint32_t mask[em::kMaxLevels + 2];
+    int64_t base[em::kMaxLevels + 2];
+    const int top = T.nlev + 1;
     int n = 0;
-    {
-        bool hit = lane < T.count[top] && box_can_cut(T.lo[top][lane], T.hi[top][lane]);
-        mask[top] = __ballot_sync(0xffffffffu, hit);
-        base[top] = 0;
-    }
+    mask[top] = 1;
+    base[top] = 0;
     int lvl = top;
     while (true) {
         if (mask[lvl] == 0) {
@@ -629,6 +652,7 @@ __device__ int gather_cutting(C &c, const em::ChunkTree &T, const double *__rest
                 if (hit) {
                     const float df = 0.5f * rf * rf, rabs = fabsf(ex) + fabsf(ey) + fabsf(ez);
                     bool maybe = false;
+#pragma unroll 1
                     for (int t = 0; t < nt && !maybe; ++t) {
                         const float4 vf = c.vf[t];
                         const float ff = ex * vf.x + ey * vf.y + ez * vf.z - df;
@@ -650,6 +674,7 @@ __device__ int gather_cutting(C &c, const em::ChunkTree &T, const double *__rest
                 const float pf = nextafterf(kth, 0.f);
                 const double p2 = (double)pf;
                 int keep = 0;   // the sorted prefix below the median key
+#pragma unroll 1
                 for (int b = 0; b < n; b += 32) {
                     const int i = b + lane;
                     keep += __popc(__ballot_sync(0xffffffffu, i < n && cd2[i] < kth));
@@ -692,6 +717,7 @@ template <class C>
 __device__ int clip_sorted(C &c, const Frame &F, int64_t n, int nc)
 {
     const int lane = threadIdx.x & 31;
+#pragma unroll 1
     for (int i0 = 0; i0 < nc; i0 += 32) {
         const int k = i0 + lane < nc ? c.u.k.cid[i0 + lane] : 0;
         if (__any_sync(0xffffffffu, k < 0 || k >= n)) return emv::VS_BOUNDS;
@@ -703,6 +729,7 @@ __device__ int clip_sorted(C &c, const Frame &F, int64_t n, int nc)
             const float nsum = fabsf(P.x) + fabsf(P.y) + fabsf(P.z);
             bool cut = false;
             const int nt = c.nt;
+#pragma unroll 1
             for (int t = 0; t < nt; ++t) {
                 bool out, unsure;
                 side32(P, nsum, c.vf[t], c.ev[t], out, unsure);
@@ -753,6 +780,7 @@ __device__ int wbuild_cell(C &c, const em::ChunkTree &T, const Frame &F, int64_t
             d2 = dx * dx + dy * dy + dz * dz;
         }
         float kthf = INFINITY;
+#pragma unroll 1
         for (int r = 0; r < 8; ++r) {
             float m = d2;
 #pragma unroll
@@ -773,12 +801,14 @@ __device__ int wbuild_cell(C &c, const em::ChunkTree &T, const Frame &F, int64_t
     // round -1 is stage 1, rounds 0.. stage 2; both clip through the one call
     // site below (one inlined copy of the clip keeps the code small)
     double skip2 = -1.0;
+#pragma unroll 1
     for (int round = -1; round < 256; ++round) {
         int m = -1;
         double hi2 = 0.0;
         if (round < 0) {
             // stage 1: shrink or grow R until the candidates fit and number at least K
             double lo_ok = 0.0, hi_bad = INFINITY;
+#pragma unroll 1
             for (int it = 0; it < 48; ++it) {
                 m = gather(c, T, xs, ys, zs, s, gx, gy, gz, -1.0, R2, margin, status);
                 if (status & emv::VS_COINCIDENT) return status;
@@ -800,6 +830,7 @@ __device__ int wbuild_cell(C &c, const em::ChunkTree &T, const Frame &F, int64_t
             const double lim2 = 4.0 * wrmax2(c, F) * (1.0 + 1e-12);   // no generator beyond 2 R_max can cut
             if (skip2 >= lim2) return status;
             hi2 = lim2;
+#pragma unroll 1
             for (int h = 0; h < 64; ++h) {
                 m = gather_cutting(c, T, xs, ys, zs, s, gx, gy, gz, skip2, hi2);
                 if (m >= 0) break;
@@ -824,6 +855,7 @@ __device__ void finish_vertices(C &c, const Frame &F)
 {
     const int lane = threadIdx.x & 31;
     __syncwarp();
+#pragma unroll 1
     for (int t = lane; t < c.nt; t += 32) {
         double x, y, z;
         meet64(c, F, t, x, y, z);
@@ -843,6 +875,7 @@ __device__ int wface_loop(const C &c, int q, uint8_t *loop, int maxn)
 {
     const int cur = c.cur, nt = c.nt;
     int t0 = -1;
+#pragma unroll 1
     for (int t = 0; t < nt && t0 < 0; ++t) {
         const uint32_t w = c.tri[cur][t];
         if (byte_of(w, 0) == q || byte_of(w, 1) == q || byte_of(w, 2) == q) t0 = t;
