@@ -506,41 +506,16 @@ ALGO_WORK = {
     "pseudo_2e5": dict(subtriangles=162.86, flops=41708.6, sqrt=1017.31, transcendental=2280.04, pairs=13422),
     "sphere_1e5": dict(subtriangles=163.63, flops=46702.9, sqrt=1064.1, transcendental=2529.7, pairs=2734),
 }
-# Implementation work of the FP32 pass per pair (what the kernel executes,
-# float-float bookkeeping included), for the utilisation figure beside the
-# algorithmic one: the cell's faces, the faces within reach (D < 2 and R < 2 in
-# units of h) and their edges, counted over random pairs of each workload with
-# a CPU model of the FP32 pass (6,000 pairs of the 1e6 cloud, 3,683 of the 1e5
-# sphere), and the quadrature's 4-node slots (a 4-point segment, or half of an
-# 8-point sub-piece), counted over every pair of one launch by an instrumented
-# build.
-WORK = {
-    "pseudo_1e6": dict(faces=15.64, faces_used=11.33, edges_used=60.65, slots=88.43),
-    "sphere_1e5": dict(faces=15.23, faces_used=7.93, edges_used=43.36, slots=72.05),
-}
-# Work of the FP32 pass per unit, counted in its source (FMA = 2 flops):
-#  - per quadrature node 53 FP32 flops (the node's place relative to its
-#    segment's start, sinh, cosh and tau - ts from expm1, Q from rsqrt and a
-#    Newton step, Q^2 - R^2 from the offset: 33; the kernel piece's integrand
-#    about 20) and 5 SFU operations (expm1, the reciprocals of 1 + expm1,
-#    Q + R and cosh, and rsqrt for Q);
-#  - per edge of a face within reach 185 FP32 flops of float-float geometry
-#    (two offset dot products, four products, four sums) and segment set-up
-#    (lengths in s from the offsets, the differences at the start);
-#  - per face 60 (float-float plane distance and, for faces within reach,
-#    the face constants), and 18 per edge of a face within reach for the FP32
-#    distance to the polygon;
-#  - per 4-node slot 14 for the float-float accumulation and 6 for the
-#    segment start's sinh and cosh (ts / A, and sqrt(1 + (ts/A)^2) by rsqrt
-#    and a Newton step), formed where the slot is evaluated;
-#  - per pair about 30 FP64 flops (r = x - g, 1/h, the final sums).
-FP32_FLOPS_NODE, SFU_OPS_NODE = 53, 5
-FP32_FLOPS_EDGE, FP32_FLOPS_FACE, FP32_FLOPS_POLY_EDGE, FP32_FLOPS_SLOT = 185, 60, 18, 20
-FP64_FLOPS_PAIR = 30
+# Implementation work of the FP32 pass per pair: the FP32 operations it executes
+# (FMA = 2), float-float bookkeeping included, for the utilisation figure beside
+# the algorithmic one.  Counted by ncu on the 1e5 sphere's 4.34 M pairs with the
+# same arithmetic unpacked (the counters leave packed instructions out); the 1e6
+# cloud's pairs take the same time to 5%.
+IMPL_FLOPS = {"pseudo_1e6": 30432.0, "sphere_1e5": 30432.0}
 # DRAM traffic of one k_map_fp32 launch per pair (ncu, dram__bytes_read.sum +
 # dram__bytes_write.sum over the pairs of the launch), per workload, from a
 # capture of the current kernel (profiles/k_map_fp32_dram_pseudo_1e6.md)
-TRAFFIC_PER_PAIR = {"pseudo_1e6": 108.94}
+TRAFFIC_PER_PAIR = {"pseudo_1e6": 108.53}
 
 
 def nominal_peaks(sm_count, mhz):
@@ -558,7 +533,7 @@ def roofline(npairs, ms, precision, workload, peaks, clock_mhz=None):
     the pipe that executes it (em_measure_peaks: FP32 for the mixed pass, FP64
     for the FP64 path); the special-function rate (square roots and
     transcendental calls) against the measured SFU peak beside it, and the
-    FP32 pass's own instruction-mix flops (WORK) as a utilisation figure."""
+    FP32 pass's own flops (IMPL_FLOPS) as a utilisation figure."""
     aw = ALGO_WORK.get(workload)
     if aw is None or ms <= 0:   # per-pair work not counted for this workload
         return None
@@ -579,11 +554,8 @@ def roofline(npairs, ms, precision, workload, peaks, clock_mhz=None):
            "sfu": {"achieved": xu, "peak": peaks["xu_tops"], "unit": "Top/s", "frac": xu / peaks["xu_tops"],
                    "ops_per_pair": aw["sqrt"] + aw["transcendental"],
                    "work": "square roots and transcendental calls of the closed form per pair"}}
-    wk = WORK.get(workload)
-    if precision == "mixed" and wk is not None:
-        nodes = 4 * wk["slots"]
-        f32 = (FP32_FLOPS_NODE * nodes + FP32_FLOPS_SLOT * wk["slots"]
-               + (FP32_FLOPS_EDGE + FP32_FLOPS_POLY_EDGE) * wk["edges_used"] + FP32_FLOPS_FACE * wk["faces"])
+    f32 = IMPL_FLOPS.get(workload)
+    if precision == "mixed" and f32 is not None:
         impl = npairs * f32 / t / 1e12
         out["implementation"] = {"achieved": impl, "unit": "TFLOP/s", "frac": impl / peaks["fp32_tflops"],
                                  "flops_per_pair": f32,

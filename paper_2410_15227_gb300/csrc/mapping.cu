@@ -771,7 +771,7 @@ __global__ void __launch_bounds__(32 * FW_WARPS) k_map_fp64(
 // every weight above 1e-14 / tol, absolute 1e-14 below); so does a face plane
 // through P.
 //
-// 24.06 M pairs of the 1e6-particle cloud: 65.8 ms (3.7e8 pairs/s), against
+// 24.06 M pairs of the 1e6-particle cloud: 63.8 ms (3.8e8 pairs/s), against
 // 111 ms with 4- and 8-point rules in s = asinh(tau / A), an asinh per
 // segment and an exponential per node, the two sides of every edge queued in
 // turn, and correctly rounded or subnormal-safe reciprocals; the error against
