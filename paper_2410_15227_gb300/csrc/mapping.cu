@@ -37,9 +37,10 @@ __global__ void k_prepare_faces(int64_t nface, int64_t ncell, const double *__re
     }
     const int64_t j = lo;
     const double gx = gen[3 * j], gy = gen[3 * j + 1], gz = gen[3 * j + 2];
-    const double nx = normals[3 * f], ny = normals[3 * f + 1], nz = normals[3 * f + 2];
+    double nx = normals[3 * f], ny = normals[3 * f + 1], nz = normals[3 * f + 2], c = 0.0;
     const int64_t v0 = fvo[f], v1 = fvo[f + 1];
-    const double c = nx * (verts[3 * v0] - gx) + ny * (verts[3 * v0 + 1] - gy) + nz * (verts[3 * v0 + 2] - gz);
+    if (v0 < v1) c = nx * (verts[3 * v0] - gx) + ny * (verts[3 * v0 + 1] - gy) + nz * (verts[3 * v0 + 2] - gz);
+    else nx = ny = nz = 0.0;   // an imported face of no vertices lies nowhere and bounds nothing
     plane[f] = PlaneD{nx, ny, nz, c};
     // hi and low parts: the plane = hi + lo to about 2^-48 relative (float-float)
     PlaneF F, G;
@@ -171,10 +172,12 @@ int em_prepare_cells(em_ctx *ctx, em_voronoi *v)
                 v->nface, v->ncell, v->gen, v->cell_face_off, v->face_vert_off, v->verts, v->normals, v->plane,
                 v->plane_f, v->plane_fl, face_of_fv, cell_of_face);
             EM_LAUNCHED(ctx);
-            k_prepare_edges<<<em_grid(v->nfv, PREP_EDGES), PREP_EDGES, 0, ctx->stream>>>(
-                v->nfv, v->gen, v->face_vert_off, v->verts, v->normals, face_of_fv, cell_of_face,
-                (unsigned long long *)v->radius, v->edge, v->edge_f, v->edge_fl);
-            EM_LAUNCHED(ctx);
+            if (v->nfv) {   // its last threads repeat vertex nfv - 1
+                k_prepare_edges<<<em_grid(v->nfv, PREP_EDGES), PREP_EDGES, 0, ctx->stream>>>(
+                    v->nfv, v->gen, v->face_vert_off, v->verts, v->normals, face_of_fv, cell_of_face,
+                    (unsigned long long *)v->radius, v->edge, v->edge_f, v->edge_fl);
+                EM_LAUNCHED(ctx);
+            }
         }
         k_radius_finish<<<em_grid(v->ncell, 256), 256, 0, ctx->stream>>>(v->ncell, v->radius);
         EM_LAUNCHED(ctx);

@@ -268,6 +268,7 @@ __global__ void k_cell_centroid(int64_t ncell, const double *__restrict__ gen, c
     double v6 = 0.0, mx = 0.0, my = 0.0, mz = 0.0;
     for (int64_t f = cfo[j] + lane; f < cfo[j + 1]; f += 32) {
         const int64_t k0 = fvo[f], k1 = fvo[f + 1];
+        if (k1 - k0 < 3) continue;   // (of imported cells)
         const double ax = verts[3 * k0] - gx, ay = verts[3 * k0 + 1] - gy, az = verts[3 * k0 + 2] - gz;
         double bx = verts[3 * k0 + 3] - gx, by = verts[3 * k0 + 4] - gy, bz = verts[3 * k0 + 5] - gz;
         for (int64_t k = k0 + 2; k < k1; ++k) {
