@@ -626,7 +626,7 @@ __device__ __forceinline__ void fp64_pairs_warp(int64_t n, const int32_t *__rest
             continue;
         }
         // inside test over all faces, then the form
-        bool ins = true;
+        bool ins = nface > 0;   // nothing lies in a cell without faces: it weighs 0
         if (code >= 0)
             for (int f = lane; f < nface; f += 32) {
                 const PlaneD pl = plane[f0 + f];
@@ -635,6 +635,8 @@ __device__ __forceinline__ void fp64_pairs_warp(int64_t n, const int32_t *__rest
         ins = __all_sync(0xffffffffu, ins);
         const bool full = code < 0 || (ins && sqrt(rx * rx + ry * ry + rz * rz) + radius[j] < 2.0 * hh);
         // faces: distance, coefficients, and how many edges each contributes
+        if (lane == 0) p.pre[0] = 0;   // also where there is no face (a cell that a range build left out)
+        __syncwarp();
         for (int base = 0; base < nface; base += 32) {
             const int f = base + lane;
             int cnt = 0;
@@ -652,9 +654,7 @@ __device__ __forceinline__ void fp64_pairs_warp(int64_t n, const int32_t *__rest
                 const int y = __shfl_up_sync(0xffffffffu, xs, o);
                 if (lane >= o) xs += y;
             }
-            const int carry = base == 0 ? 0 : p.pre[base];
-            __syncwarp();
-            if (lane == 0 && base == 0) p.pre[0] = 0;
+            const int carry = p.pre[base];
             if (f < nface) p.pre[f + 1] = carry + xs;
             __syncwarp();
         }
@@ -1105,7 +1105,7 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_map_fp32(int64_t npairs, c
     // the full kernel applies when P is inside a cell that lies entirely
     // within 2h of it; otherwise the complement form, and whether P is inside
     // is read off the face loop's own plane distances
-    bool inside = valid, full = false;
+    bool inside = f1 > f, full = false;   // nothing lies in a cell without faces: it weighs 0
     if (valid && sqrt(rx * rx + ry * ry + rz * rz) + rad < 2.0 * hh) {
         for (int64_t g = f; g < f1; ++g) inside = inside && !(plane_dist(g).hi < 0.f);
         full = inside;
