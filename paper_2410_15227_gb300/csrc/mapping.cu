@@ -249,7 +249,8 @@ __global__ void k_segment_offsets(int64_t n, const int32_t *__restrict__ key, in
         atomicOr(bad, 2);
         return;
     }
-    for (int64_t c = prev + 1; c <= cur; ++c) off[c] = k;
+    // (a negative key before this one is an error that its own thread raises)
+    for (int64_t c = prev < -1 ? 0 : prev + 1; c <= cur; ++c) off[c] = k;
 }
 
 __global__ void k_iota_keys(int64_t n, const int32_t *__restrict__ src, uint32_t *__restrict__ key,
