@@ -134,6 +134,11 @@ struct HitLists {
     int4 *seg;
     int32_t *head;
 };
+// FP32 decides only on lengths whose squares keep their precision: below FINE32
+// (squares of 1e-32, 13 digits above the smallest subnormal) and where squares
+// overflow to infinity, a comparison leaves the pair to the FP64 predicate, so
+// that the list does not depend on the caller's unit of length.
+constexpr float FINE32 = 1e-16f;
 constexpr int PLACE_MAX = 2048;   // hits of a cell that k_place_pairs orders in shared memory
 
 __global__ void __launch_bounds__(32 * PAIRS_WARPS)
@@ -201,12 +206,12 @@ __global__ void __launch_bounds__(32 * PAIRS_WARPS)
             const float rr = sqrtf(rxf * rxf + ryf * ryf + rzf * rzf);
             const float band = 1e-5f * (Rf + rr + h2f);
             // the cell lies inside the ball of radius R_j around g: dist >= |r| - R_j
-            if (rr < Rf + h2f + band) {
+            if (rr <= fmaxf(Rf + h2f + band, FINE32)) {
                 const float lo = h2f - band, hi = h2f + band;
                 const float d2f = cell_dist2_f32(rxf, ryf, rzf, f0, f1, fvo, plane_f, edge_f, hi + band);
-                if (lo > 0.f && d2f < lo * lo) {
+                if (lo > FINE32 && d2f < lo * lo) {
                     hit = true;
-                } else if (!(d2f > hi * hi)) {   // inside the band: exact FP64 test
+                } else if (!(d2f > fmaxf(hi, FINE32) * fmaxf(hi, FINE32))) {   // inside the band: exact FP64 test
                     const double d2 = cell_dist2(rx, ry, rz, f0, f1, fvo, plane, edge, 2.0 * h2);
                     hit = d2 < h2 * h2;
                     if (hit) nearb = fabs(sqrt(d2) - h2) < 0.5e-9 * h2;
@@ -271,12 +276,13 @@ __global__ void __launch_bounds__(32 * PAIRS_WARPS)
                 const float ex = p[u].x - gxf, ey = p[u].y - gyf, ez = p[u].z - gzf, h2f = p[u].w;
                 const float d2 = ex * ex + ey * ey + ez * ez;
                 const float slack = 1e-5f * (gscale + Rf + h2f);
-                const float in = h2f - slack - 1e-5f * h2f, out = (Rf + h2f + slack) * 1.00003f, box = h2f + 2.f * slack;
+                const float in = h2f - slack - 1e-5f * h2f, reach = (Rf + h2f + slack) * 1.00003f;
+                const float out = fmaxf(reach, FINE32), box = fmaxf(h2f + 2.f * slack, FINE32);
                 const float dx = fmaxf(fmaxf(bl[0] - ex, ex - bh[0]), 0.f), dy = fmaxf(fmaxf(bl[1] - ey, ey - bh[1]), 0.f),
                             dz = fmaxf(fmaxf(bl[2] - ez, ez - bh[2]), 0.f);
-                const bool sure = k[u] >= 0 && ginside && in > 0.f && d2 < in * in;
-                const bool cand = k[u] >= 0 && !sure && out > 0.f && d2 < out * out &&
-                                  dx * dx + dy * dy + dz * dz < box * box;
+                const bool sure = k[u] >= 0 && ginside && in > FINE32 && d2 < in * in;
+                const bool cand = k[u] >= 0 && !sure && reach > 0.f && d2 <= out * out &&
+                                  dx * dx + dy * dy + dz * dz <= box * box;
                 if (__any_sync(0xffffffffu, sure)) emit(k[u], sure, false);
                 const unsigned cm = __ballot_sync(0xffffffffu, cand);
                 if (cand) cb[nc + __popc(cm & ((1u << lane) - 1u))] = k[u];
