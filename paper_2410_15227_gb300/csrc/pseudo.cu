@@ -260,35 +260,30 @@ struct HsList {
     int n;
     int32_t *k;
     int32_t *buf;      // HS_BUF entries of the warp's own
-    double (*red)[2];  // the team's partial sums
+    double (*red)[3];  // the team's partial sums
     int part;
     bool heavy;        // one warp alone: the walk was given up
 };
 
-// a and b summed over the team's lanes, the same on all of them
-template <int TEAM, class Real>
-__device__ __forceinline__ void team_sum(const HsList &L, Real &a, Real &b)
+// N values summed over the team's lanes, the same on all of them
+template <int TEAM, int N, class Real>
+__device__ __forceinline__ void team_sum(const HsList &L, Real (&v)[N])
 {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-    }
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
     if (TEAM > 1) {
-        if ((threadIdx.x & 31) == 0) {
-            L.red[L.part][0] = (double)a;
-            L.red[L.part][1] = (double)b;
-        }
+        if ((threadIdx.x & 31) == 0)
+            for (int i = 0; i < N; ++i) L.red[L.part][i] = (double)v[i];
         __syncthreads();
-        a = b = Real(0);
-        for (int t = 0; t < TEAM; ++t) {
-            a += (Real)L.red[t][0];
-            b += (Real)L.red[t][1];
+        for (int i = 0; i < N; ++i) {
+            v[i] = Real(0);
+            for (int t = 0; t < TEAM; ++t) v[i] += (Real)L.red[t][i];
         }
         __syncthreads();
     }
 }
-
 
 // The population within 2h of the node, 32 entries at a time from a compacted
 // buffer: batch(k, in) on every lane, in false on the lanes without one; it
@@ -334,18 +329,18 @@ __device__ __forceinline__ bool term64(const Population &P, const HsList &L, int
 template <int TEAM>
 __device__ Density warp_density(const em::ChunkTree &T, const Population &P, HsList &L, double h, float margin)
 {
-    double s = 0.0, ds = 0.0;
+    double s[2] = {0.0, 0.0};
     const double ih = rcp64(h), ih2 = ih * ih, norm = ih2 * ih * 0.31830988618379067154;   // 1/(pi h^3)
     walk_neighbours<TEAM>(T, L, h, margin, [&](int32_t k, bool in) {
         double w, g;
         if (in && term64(P, L, k, ih2, w, g)) {
-            s += w;
-            ds += g;
+            s[0] += w;
+            s[1] += g;
         }
         return true;
     });
-    team_sum<TEAM>(L, s, ds);
-    return Density{s * norm, -ds * norm * ih};
+    team_sum<TEAM>(L, s);
+    return Density{s[0] * norm, -s[1] * norm * ih};
 }
 
 // Sign of f(h) = h_fact n(h)^(-1/3) - h (Eq. 8) for the bisection, which uses
@@ -359,51 +354,55 @@ template <int TEAM>
 __device__ int warp_f_sign(const em::ChunkTree &T, const Population &P, HsList &L, double h, double h_fact,
                            float margin)
 {
-    double s = 0.0, over = 0.0;
+    double s[2] = {0.0, 0.0};   // the sum; warps that ended their walk
     const double ih = rcp64(h), ih2 = ih * ih, norm = ih2 * ih * 0.31830988618379067154;   // 1/(pi h^3)
     const double t = h_fact * ih, thr = t * t * t * (1.0 + 1e-9);
     // the sum of w; the walk stops once norm sum w exceeds thr
     const double thrw = thr * (3.14159265358979323846 * h * h * h);   // thr / norm
     const bool full = walk_neighbours<TEAM>(T, L, h, margin, [&](int32_t k, bool in) {
         double w, g;
-        if (in && term64(P, L, k, ih2, w, g)) s += w;
-        double tot = s;
+        if (in && term64(P, L, k, ih2, w, g)) s[0] += w;
+        double tot = s[0];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
         return !(tot > thrw);
     });
-    if (!full) over = 1.0;
-    team_sum<TEAM>(L, s, over);
-    if (over > 0.0) return -1;
-    const double f = h_fact * rcbrt(s * norm) - h;   // n^(-1/3) as a reciprocal cube root
+    if (!full) s[1] = 1.0;
+    team_sum<TEAM>(L, s);
+    if (s[1] > 0.0) return -1;
+    const double f = h_fact * rcbrt(s[0] * norm) - h;   // n^(-1/3) as a reciprocal cube root
     return f > 0.0 ? 1 : (f < 0.0 ? -1 : 0);
 }
 
+// Sums of w, of g = 3 w + q w' and of e = q g': dS / dlog h = 3 S - G,
+// dG / dlog h = -E.
 struct Sum32 {
-    float S, G;   // sums of w and of g = 3 w + q w'
+    float S, G, E;
 };
 
-// w and g of the M4 spline at q2 = q^2 < 4, branch-free
-__device__ __forceinline__ void m4_wg32(float q2, float &w, float &g)
+// w, g and e of the M4 spline at q2 = q^2 < 4, branch-free
+__device__ __forceinline__ void m4_wge32(float q2, float &w, float &g, float &e)
 {
     const float q = q2 * rsqrtf(fmaxf(q2, 1e-30f));   // 0 at the particle itself
     const float t = 2.f - q, t2 = t * t;
     w = q < 1.f ? fmaf(q2, fmaf(0.75f, q, -1.5f), 1.f) : 0.25f * t2 * t;
     g = q < 1.f ? fmaf(q2, fmaf(4.5f, q, -7.5f), 3.f) : 0.75f * t2 * (t - q);
+    e = q < 1.f ? q2 * fmaf(13.5f, q, -15.f) : q * t * fmaf(4.5f, q, -6.f);
 }
 
 // Add one entry's terms (none if !in).  No branches, so that the entries of a
 // batch overlap: a lone warp walking a large node's 2 h_0, which may hold the
 // whole population, is bound by the latency of this chain.
-__device__ __forceinline__ void add32(const HsList &L, bool in, float4 p, float4 lo, float ih2, float &S, float &G)
+__device__ __forceinline__ void add32(const HsList &L, bool in, float4 p, float4 lo, float ih2, float (&s)[3])
 {
     const float ex = (p.x - L.xh) + (lo.x - L.xl), ey = (p.y - L.yh) + (lo.y - L.yl), ez = (p.z - L.zh) + (lo.z - L.zl);
     const float q2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) * ih2;
-    float w, g;
-    m4_wg32(q2, w, g);
+    float w, g, e;
+    m4_wge32(q2, w, g, e);
     const bool add = in && q2 < 4.f;
-    S += add ? w : 0.f;
-    G += add ? g : 0.f;
+    s[0] += add ? w : 0.f;
+    s[1] += add ? g : 0.f;
+    s[2] += add ? e : 0.f;
 }
 
 // The sums at h in FP32 (the same on every lane), from the list where it
@@ -413,9 +412,9 @@ __device__ Sum32 warp_sum32(const em::ChunkTree &T, const Population &P, HsList 
 {
     const int lane = threadIdx.x & 31;
     const float ih2 = 1.f / (h * h);
-    float S = 0.f, G = 0.f;
+    float s[3] = {0.f, 0.f, 0.f};
     if (L.n >= 0 && 2.0002f * h <= L.r) {
-        for (int t = lane; t < L.n; t += 32) add32(L, true, T.pts[L.k[t]], P.lo[L.k[t]], ih2, S, G);
+        for (int t = lane; t < L.n; t += 32) add32(L, true, T.pts[L.k[t]], P.lo[L.k[t]], ih2, s);
     } else {
         const float r = 2.f * HS_COVER * h;
         const float lim = r + 1e-5f * (fabsf(L.xh) + fabsf(L.yh) + fabsf(L.zh) + r), lim2 = lim * lim;
@@ -438,7 +437,7 @@ __device__ Sum32 warp_sum32(const em::ChunkTree &T, const Population &P, HsList 
             for (int u = 0; u < HS_LEAVES; ++u) {
                 const float ex = p[u].x - L.xh, ey = p[u].y - L.yh, ez = p[u].z - L.zh;
                 const bool in = k[u] >= 0 && ex * ex + ey * ey + ez * ez < lim2;
-                add32(L, in, p[u], lo[u], ih2, S, G);
+                add32(L, in, p[u], lo[u], ih2, s);
                 b[u] = __ballot_sync(0xffffffffu, in);
             }
 #pragma unroll
@@ -453,8 +452,8 @@ __device__ Sum32 warp_sum32(const em::ChunkTree &T, const Population &P, HsList 
         L.r = r;
         L.n = TEAM == 1 && n <= HS_LIST && !L.heavy ? n : -1;
     }
-    team_sum<TEAM>(L, S, G);
-    return Sum32{S, G};
+    team_sum<TEAM>(L, s);
+    return Sum32{s[0], s[1], s[2]};
 }
 
 // Make the list the population within 2h and a margin for h's last digits, so
@@ -491,20 +490,21 @@ template <int TEAM>
 __device__ Density list_density(const em::ChunkTree &T, const Population &P, HsList &L, double h, float margin)
 {
     if (!(L.n >= 0 && 2.0002f * (float)h <= L.r)) return warp_density<TEAM>(T, P, L, h, margin);
-    double s = 0.0, ds = 0.0;
+    double s[2] = {0.0, 0.0};
     const double ih = rcp64(h), ih2 = ih * ih, norm = ih2 * ih * 0.31830988618379067154;   // 1/(pi h^3)
     for (int t = threadIdx.x & 31; t < L.n; t += 32) {
         double w, g;
         if (term64(P, L, L.k[t], ih2, w, g)) {
-            s += w;
-            ds += g;
+            s[0] += w;
+            s[1] += g;
         }
     }
-    team_sum<TEAM>(L, s, ds);
-    return Density{s * norm, -ds * norm * ih};
+    team_sum<TEAM>(L, s);
+    return Density{s[0] * norm, -s[1] * norm * ih};
 }
 
-// One Newton step of Eqs. 8-10 from n and dn/dh at h.
+// The step f / f' of Newton's iteration (Eqs. 8-10: the next iterate is h less
+// the step) from n and dn/dh at h.
 __device__ __forceinline__ double newton_step(Density d, double h, double h_fact)
 {
     // n^(-1/3) as a reciprocal cube root and n^(-4/3) as its fourth power:
@@ -514,7 +514,7 @@ __device__ __forceinline__ double newton_step(Density d, double h, double h_fact
     const double c = rcbrt(d.n);
     const double f = h_fact * c - h;                                              // Eq. 8
     const double fp = -h_fact * d.dn * ((c * c) * (c * c)) * (1.0 / 3.0) - 1.0;   // Eq. 9 (a product, not a division)
-    return h - f * rcp64(fp);                                                     // Eq. 10
+    return f * rcp64(fp);                                                         // Eq. 10
 }
 
 // Newton (Eq. 10) from h_0 (Eq. 11) until |dh|/h_0 < tol, every evaluation in
@@ -527,7 +527,7 @@ __device__ bool newton64(const em::ChunkTree &T, const Population &P, HsList &L,
     const double ih0 = rcp64(h0), blo = 1e-2 * h0, bhi = 1e2 * h0;
     double h = h0;
     for (int it = 0; it < max_newton; ++it) {
-        const double hn = newton_step(warp_density<TEAM>(T, P, L, h, margin), h, h_fact);
+        const double hn = h - newton_step(warp_density<TEAM>(T, P, L, h, margin), h, h_fact);
         if (L.heavy) return false;
         if (!(hn >= blo && hn <= bhi)) return false;
         const double step = fabs(hn - h) * ih0;   // |dh| / h_0
@@ -563,21 +563,42 @@ __device__ double bisect64(const em::ChunkTree &T, const Population &P, HsList &
     return 0.5 * (lo + hi);
 }
 
-// The root of f near h (an FP32 root) by Newton in FP64: the step after which
-// the quadratic convergence leaves less than a tenth of tol is the last.
+// One Newton step from FP32 sums at h, in relative terms (x = log h,
+// a = h_fact n^(-1/3) / h): f = h (a - 1), f' = c - 1, h f'' = dc/dx.
+struct Step32 {
+    float s;      // the step f / f', over h: the next iterate is h (1 - s)
+    float c;      // f' + 1
+    float K;      // h f'' / (2 f'): Newton's remaining error is K s^2
+};
+__device__ __forceinline__ Step32 step32(Sum32 u, float hf)
+{
+    const float a = hf * cbrtf(3.14159265f / u.S), iS = 1.f / (3.f * u.S);
+    Step32 r;
+    r.c = a * u.G * iS;
+    const float i = 1.f / (r.c - 1.f);
+    const float dc = (r.c - a) * u.G * iS - a * iS * (u.E + u.G * (3.f - u.G / u.S));
+    r.s = (a - 1.f) * i;
+    r.K = 0.5f * dc * i;
+    return r;
+}
+
+// The root of f near h (an FP32 root, K of Step32 there) in FP64, to its
+// rounding whatever the tolerance: Newton's step and the next term of its
+// series, h K s^2, after which what is left is K^2 s^3 and s^2 times the change
+// of K over the step.  So one evaluation suffices in nine cases of ten.
 // Returns false where it does not settle at once.
 template <int TEAM>
-__device__ bool polish64(const em::ChunkTree &T, const Population &P, HsList &L, double &h, double h_fact, double tol,
+__device__ bool polish64(const em::ChunkTree &T, const Population &P, HsList &L, double &h, double h_fact, float K,
                          float margin)
 {
     settle_list<TEAM>(T, P, L, (float)h, margin);
     for (int it = 0; it < 5; ++it) {
-        const double hn = newton_step(list_density<TEAM>(T, P, L, h, margin), h, h_fact);
+        const double d = newton_step(list_density<TEAM>(T, P, L, h, margin), h, h_fact);
         if (L.heavy) return false;
-        const double d = fabs(hn - h);
-        if (!(d <= 1e-3 * h)) return false;
-        h = hn;
-        if (d * d <= 0.1 * tol * h * h) return true;
+        const float s = (float)(d * rcp64(h)), q = K * s * s;
+        if (!(fabsf(s) <= 1e-3f)) return false;
+        h = h - d - h * (double)q;
+        if (fabsf(q) <= 1e-13f && fabsf(s) <= 1e-5f) return true;
     }
     return false;
 }
@@ -598,26 +619,25 @@ __device__ int newton32(const em::ChunkTree &T, const Population &P, HsList &L, 
     for (int it = 0; it + 4 < max_newton; ++it) {
         const Sum32 u = warp_sum32<TEAM>(T, P, L, h, margin);
         if (L.heavy) return -1;
-        const float a = hf * cbrtf(3.14159265f / u.S);   // h_fact n^(-1/3) / h
-        const float hn = h * (1.f - (a - 1.f) / (a * u.G / (3.f * u.S) - 1.f));
+        const Step32 r = step32(u, hf);
+        const float hn = h * (1.f - r.s);
         if (!(fabsf(hn) < 1e30f)) return -1;
         if (hn < 0.9f * blo || hn > 1.1f * bhi) return 0;
         if (hn < 1.1f * blo || hn > 0.9f * bhi) return -1;
-        const float d = fabsf(hn - h);
-        h = hn;
-        if (d < 3e-4f * h) {
-            hout = h;
-            return polish64<TEAM>(T, P, L, hout, h_fact, tol, margin) ? 1 : -1;
+        if (fabsf(r.s) < 3e-4f) {
+            hout = hn - h * (r.K * r.s * r.s);
+            return polish64<TEAM>(T, P, L, hout, h_fact, r.K, margin) ? 1 : -1;
         }
+        h = hn;
     }
     return -1;
 }
 
 // bisect64's result where FP32 decides it (else false): f's sign is that of
 // pi h_fact^3 - S(h), S = sum w increasing in h, so its one root r in the
-// bracket is found by a bracketed Newton in log h, polished, and the
-// bisection's decisions are comparisons with r; only a midpoint within 2e-14 r
-// of it (the rounding of either) takes an FP64 evaluation.
+// bracket is found by a bracketed Newton in log h, polished to FP64's rounding
+// (about 1e-15 r / |f'|), and the bisection's decisions are comparisons with r;
+// only a midpoint within ten times that of it takes an FP64 evaluation.
 template <int TEAM>
 __device__ bool bisect32(const em::ChunkTree &T, const Population &P, HsList &L, double h0, double h_fact, double tol,
                          float margin, double &hout, int &st)
@@ -667,9 +687,10 @@ __device__ bool bisect32(const em::ChunkTree &T, const Population &P, HsList &L,
         if ((in && d < 3e-4f * h) || hi - lo < 1e-6f * h) break;
     }
     double r = h;
-    if (!polish64<TEAM>(T, P, L, r, h_fact, tol, margin)) return false;
+    const Step32 v = step32(u, hf);   // within 3e-4 of the root, or so
+    if (!polish64<TEAM>(T, P, L, r, h_fact, v.K, margin)) return false;
     double dlo = 1e-2 * h0, dhi = 1e2 * h0;
-    const double near = 2e-14 * r, width = tol * h0;
+    const double near = 1e-14 * r * (1.0 + 1.0 / (double)fabsf(v.c - 1.f)), width = tol * h0;
     for (int k = 0; k < 200 && (dhi - dlo) > width && !L.heavy; ++k) {
         const double mid = 0.5 * (dlo + dhi), e = mid - r;
         const bool below = fabs(e) > near ? e < 0.0
@@ -739,13 +760,13 @@ __global__ void __launch_bounds__(32 * HS_WARPS, 6) k_h_solve(
 
 // The listed nodes, a block of HS_TEAM warps each (grid-stride; the count is
 // read on the device).
-__global__ void __launch_bounds__(32 * HS_TEAM) k_h_solve_heavy(
+__global__ void __launch_bounds__(32 * HS_TEAM, 2) k_h_solve_heavy(
     em::ChunkTree T, Population P, const double *__restrict__ px, const double *__restrict__ py,
     const double *__restrict__ pz, double h_fact, double tol, int max_newton, float margin, double *__restrict__ ph,
     int32_t *__restrict__ status, const int *__restrict__ nheavy, const int32_t *__restrict__ heavy)
 {
     __shared__ int32_t bufs[HS_TEAM][HS_BUF];
-    __shared__ double red[HS_TEAM][2];
+    __shared__ double red[HS_TEAM][3];
     HsList L;
     L.k = nullptr;
     L.buf = bufs[threadIdx.x >> 5];
