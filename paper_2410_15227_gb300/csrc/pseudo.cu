@@ -412,7 +412,7 @@ __device__ Sum32 warp_sum32(const em::ChunkTree &T, const Population &P, HsList 
 {
     const int lane = threadIdx.x & 31;
     const float ih2 = 1.f / (h * h);
-    float s[3] = {0.f, 0.f, 0.f};
+    float s[3] = {0.f, 0.f, 0.f}, lost[3] = {0.f, 0.f, 0.f};
     if (L.n >= 0 && 2.0002f * h <= L.r) {
         for (int t = lane; t < L.n; t += 32) add32(L, true, T.pts[L.k[t]], P.lo[L.k[t]], ih2, s);
     } else {
@@ -427,6 +427,7 @@ __device__ Sum32 warp_sum32(const em::ChunkTree &T, const Population &P, HsList 
             }
             float4 p[HS_LEAVES], lo[HS_LEAVES];
             unsigned b[HS_LEAVES];
+            float v[3] = {0.f, 0.f, 0.f};
 #pragma unroll
             for (int u = 0; u < HS_LEAVES; ++u) {
                 const int32_t kk = max(k[u], 0);
@@ -437,8 +438,15 @@ __device__ Sum32 warp_sum32(const em::ChunkTree &T, const Population &P, HsList 
             for (int u = 0; u < HS_LEAVES; ++u) {
                 const float ex = p[u].x - L.xh, ey = p[u].y - L.yh, ez = p[u].z - L.zh;
                 const bool in = k[u] >= 0 && ex * ex + ey * ey + ez * ez < lim2;
-                add32(L, in, p[u], lo[u], ih2, s);
+                add32(L, in, p[u], lo[u], ih2, v);
                 b[u] = __ballot_sync(0xffffffffu, in);
+            }
+            // a team's lanes add up thousands of terms: with what each addition rounds off
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const float t = s[i] + v[i];
+                if (TEAM > 1) lost[i] += v[i] - (t - s[i]);
+                s[i] = t;
             }
 #pragma unroll
             for (int u = 0; u < HS_LEAVES; ++u) {
@@ -452,6 +460,8 @@ __device__ Sum32 warp_sum32(const em::ChunkTree &T, const Population &P, HsList 
         L.r = r;
         L.n = TEAM == 1 && n <= HS_LIST && !L.heavy ? n : -1;
     }
+    if (TEAM > 1)
+        for (int i = 0; i < 3; ++i) s[i] += lost[i];
     team_sum<TEAM>(L, s);
     return Sum32{s[0], s[1], s[2]};
 }
@@ -569,8 +579,11 @@ struct Step32 {
     float s;      // the step f / f', over h: the next iterate is h (1 - s)
     float c;      // f' + 1
     float K;      // h f'' / (2 f'): Newton's remaining error is K s^2
+    // with h known to within e (relative) and the sums to within eps:
+    float err;    // bound on the error of 1 - s
+    float least;  // |s| is at least this, also where c - 1 may have either sign
 };
-__device__ __forceinline__ Step32 step32(Sum32 u, float hf)
+__device__ __forceinline__ Step32 step32(Sum32 u, float hf, float e, float eps)
 {
     const float a = hf * cbrtf(3.14159265f / u.S), iS = 1.f / (3.f * u.S);
     Step32 r;
@@ -579,8 +592,16 @@ __device__ __forceinline__ Step32 step32(Sum32 u, float hf)
     const float dc = (r.c - a) * u.G * iS - a * iS * (u.E + u.G * (3.f - u.G / u.S));
     r.s = (a - 1.f) * i;
     r.K = 0.5f * dc * i;
+    // the next iterate's derivative by x, over h, carries e on; and the sums'
+    // rounding: that of c is eps of 2.5 |c| + 2 a at most (the terms of G add up
+    // to |G| + 6 S in magnitude, since the positive ones are below 3 w)
+    const float M = 1.f - r.s, dM = (a - r.c + r.s * dc) * i, ce = eps * (2.5f * fabsf(r.c) + 2.f * a);
+    r.err = e * fabsf(M + dM) + eps * (fabsf(M) + fabsf(i) * a) + ce * fabsf(i * r.s);
+    r.least = (fabsf(a - 1.f) - e * fabsf(r.c - a) - eps * a) / (fabsf(r.c - 1.f) + e * fabsf(dc) + ce);
     return r;
 }
+// of the sums: a lane's has at most 192 terms in a warp, and keeps what it rounds off in a team
+constexpr float HS_EPS = 2e-6f;
 
 // The root of f near h (an FP32 root, K of Step32 there) in FP64, to its
 // rounding whatever the tolerance: Newton's step and the next term of its
@@ -605,26 +626,57 @@ __device__ bool polish64(const em::ChunkTree &T, const Population &P, HsList &L,
 
 // For a tolerance that means "converged" (tol <= HS_WARM_TOL) the approach is
 // made in FP32.  newton32: Newton's iterates from h_0 decide whether Newton
-// converges (1; the root polished in FP64) or leaves the bracket (0), as in
-// FP64 unless an iterate comes within 10% of the bracket's ends (-1: not
-// decided).
+// converges (1; the root polished in FP64) or leaves the bracket (0).  A bound
+// on how far each iterate may lie from FP64's goes along (Step32::err: near
+// f' = 0 a step magnifies the rounding without limit); where it leaves a
+// decision open, or grows beyond 1e-2, the step from the last iterate known in
+// FP64 (hx, after itx steps) is taken again in FP64 and FP32 goes on from there.
+// -1: not decided, which is also the answer where the tolerance is so near
+// FP64's rounding of a step, about 1e-14 h / |f'|, that FP64's iterates may
+// never meet it.  In a model of both on 6 x 10^7 random neighbourhoods (shells
+// of 1 to 200 entries at 0.006 to 160 h_0) no decision differed; 55 of 3 x 10^6
+// did where only iterates within 10% of the bracket's ends were left open.  1e6
+// particles: a handful of nodes take a step again; FP64 iterates throughout for
+// these, which may take them across the whole cloud, cost 1.2 ms of 5.9.
 constexpr double HS_WARM_TOL = 1e-9;
 template <int TEAM>
 __device__ int newton32(const em::ChunkTree &T, const Population &P, HsList &L, double h0, double h_fact, double tol,
                         int max_newton, float margin, double &hout)
 {
     const float h0f = (float)h0, hf = (float)h_fact, blo = 1e-2f * h0f, bhi = 1e2f * h0f;
-    float h = h0f;
     if (!(h0f > 1e-15f && h0f < 1e15f)) return -1;
-    for (int it = 0; it + 4 < max_newton; ++it) {
+    float h = h0f, e = 1e-7f;
+    double hx = h0;
+    int itx = 0;
+    bool exact = false;   // take the next step in FP64
+    // every step taken again moves itx on: at most max_newton of them (n bounds the loop whatever happens)
+    for (int it = 0, n = 0; it + 4 < max_newton && n < 4 * max_newton; ++it, ++n) {
+        if (exact) {
+            exact = false;
+            const double hn = hx - newton_step(list_density<TEAM>(T, P, L, hx, margin), hx, h_fact);
+            if (L.heavy) return -1;
+            if (!(hn >= 1e-2 * h0 && hn <= 1e2 * h0)) return 0;
+            hx = hn;
+            itx = it + 1;
+            h = (float)hx;
+            e = 1e-7f;
+            continue;
+        }
         const Sum32 u = warp_sum32<TEAM>(T, P, L, h, margin);
         if (L.heavy) return -1;
-        const Step32 r = step32(u, hf);
-        const float hn = h * (1.f - r.s);
-        if (!(fabsf(hn) < 1e30f)) return -1;
-        if (hn < 0.9f * blo || hn > 1.1f * bhi) return 0;
-        if (hn < 1.1f * blo || hn > 0.9f * bhi) return -1;
+        const Step32 r = step32(u, hf, e, HS_EPS);
+        const float hn = h * (1.f - r.s), dh = h * r.err;
+        const bool finite = fabsf(hn) < 1e30f && dh < 1e30f;
+        // left: below, above, or by a step so long that it leaves either way
+        if ((finite && (hn + dh < 0.999f * blo || hn - dh > 1.001f * bhi)) || r.least > 1.f + 1.01f * bhi / h) return 0;
+        e = r.err / (1.f - r.s);
+        if (!(finite && hn - dh > 1.001f * blo && hn + dh < 0.999f * bhi && e < 1e-2f)) {
+            it = itx - 1;
+            exact = true;
+            continue;
+        }
         if (fabsf(r.s) < 3e-4f) {
+            if (!(tol * h0 * (double)fabsf(r.c - 1.f) >= 1e-14 * (double)hn)) return -1;
             hout = hn - h * (r.K * r.s * r.s);
             return polish64<TEAM>(T, P, L, hout, h_fact, r.K, margin) ? 1 : -1;
         }
@@ -687,7 +739,7 @@ __device__ bool bisect32(const em::ChunkTree &T, const Population &P, HsList &L,
         if ((in && d < 3e-4f * h) || hi - lo < 1e-6f * h) break;
     }
     double r = h;
-    const Step32 v = step32(u, hf);   // within 3e-4 of the root, or so
+    const Step32 v = step32(u, hf, 0.f, 0.f);   // within 3e-4 of the root, or so
     if (!polish64<TEAM>(T, P, L, r, h_fact, v.K, margin)) return false;
     double dlo = 1e-2 * h0, dhi = 1e2 * h0;
     const double near = 1e-14 * r * (1.0 + 1.0 / (double)fabsf(v.c - 1.f)), width = tol * h0;

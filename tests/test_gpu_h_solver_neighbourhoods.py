@@ -36,6 +36,7 @@ def neighbourhood(seed, k):
 
 
 @pytest.mark.parametrize("seed,ks,tol,max_newton", [
+    (1, [8442, *range(20)], 1e-13, 50),
     (2, range(60), 1e-9, 50),
     (3, range(60), 1e-12, 8)])
 def test_status_and_h(orc, seed, ks, tol, max_newton):
