@@ -249,8 +249,9 @@ int voronoi_destroy(em_voronoi *v);
  *   d_x, d_y, d_z, d_h: np (pseudo-)particles (device).
  *   npairs (host, may be NULL): the pair count.
  * One pass writes the hits, unordered, into a buffer sized from the
- * context's previous pair count (plus 1/8; a guess on the first call) and a
- * radix sort orders them; a call that finds more pairs than the buffer holds
+ * context's previous pair count (plus 1/8; a guess on the first call); each
+ * cell's are then ordered by a warp, or all by a radix sort where some cell
+ * has more than 2,048.  A call that finds more pairs than the buffer holds
  * repeats the pass once with the exact size.  Synchronises the stream to
  * read the count.  EM_ECAPACITY if the pairs reach 2^31. */
 int find_pairs(em_ctx *ctx, int64_t np, const double *d_x, const double *d_y, const double *d_z,
