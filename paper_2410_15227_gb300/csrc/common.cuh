@@ -208,6 +208,13 @@ struct em_voronoi {
     explicit em_voronoi(cudaStream_t s) : mem(s) {}
 };
 
+// A particle's row of the transpose is summed by one thread up to this many
+// pairs, by a block with others of like length beyond (mapping.cu).  With 64 the
+// rows of a direct mapping, 43 on average, are partly long (4.3 M pairs: 78 us,
+// 68 so); with 128 the thread's chain shows in a pseudo-particle list (24.0 M:
+// 480 us, 466 so).
+constexpr int EM_ROW_LONG = 96;
+
 struct em_pairs {
     int device;
     DevArena mem;
@@ -217,6 +224,10 @@ struct em_pairs {
     int64_t *cell_pair_off = nullptr;               // [ncell + 1]
     int64_t *part_pair_off = nullptr;               // [np + 1]
     int32_t *part_pair_idx = nullptr;               // [npairs] pair ids sorted by (i, j)
+    // rows of the transpose with more than EM_ROW_LONG pairs (npairs > EM_ROW_LONG
+    // only), longest first, and on the device their number and that of the very long
+    int *nlong = nullptr;
+    int32_t *long_rows = nullptr;
     explicit em_pairs(cudaStream_t s) : mem(s) {}
 };
 

@@ -271,6 +271,62 @@ __global__ void k_check_within_cell(int64_t n, const int32_t *__restrict__ pi, c
     if (k > 0 && pj[k] == pj[k - 1] && pi[k] <= pi[k - 1]) atomicOr(bad, 8);
 }
 
+// The rows of the transpose with more than EM_ROW_LONG pairs, which long_rows
+// sums 32 at a time, longest first and like lengths together (four classes an
+// octave; the order within one is of no account).  k_long_count: rows per class.
+constexpr int ROW_CLASSES = 32, VERY_CLASS = 14;
+constexpr int ROW_VERY = 1086, ROW_FEW = 8;   // EM_ROW_LONG 2^(VERY_CLASS / 4), rounded down; rows a block has of them
+__device__ __forceinline__ int row_class(int64_t n)
+{
+    return ROW_CLASSES - 1 - min(ROW_CLASSES - 1, (int)(4.f * log2f((float)n * (1.f / EM_ROW_LONG))));
+}
+
+__global__ void k_long_count(int64_t np, const int64_t *__restrict__ off, int *__restrict__ count)
+{
+    __shared__ int c[ROW_CLASSES];
+    if (threadIdx.x < ROW_CLASSES) c[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t n = i < np ? off[i + 1] - off[i] : 0;
+    if (n > EM_ROW_LONG) atomicAdd(&c[row_class(n)], 1);
+    __syncthreads();
+    if (threadIdx.x < ROW_CLASSES && c[threadIdx.x]) atomicAdd(count + threadIdx.x, c[threadIdx.x]);
+}
+
+// Into rows (of that capacity: the offsets of a list that is refused afterwards
+// may be anything), with their number to nlong[0] and that of those of at least
+// about ROW_VERY pairs to nlong[1].
+__global__ void k_long_place(int64_t np, const int64_t *__restrict__ off, const int *__restrict__ count,
+                             int *__restrict__ cursor, int capacity, int32_t *__restrict__ rows, int *__restrict__ nlong)
+{
+    __shared__ int c[ROW_CLASSES], base[ROW_CLASSES];
+    const int t = threadIdx.x;
+    if (t < ROW_CLASSES) c[t] = 0;
+    __syncthreads();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + t;
+    const int64_t n = i < np ? off[i + 1] - off[i] : 0;
+    int k = 0, r = 0;
+    if (n > EM_ROW_LONG) {
+        k = row_class(n);
+        r = atomicAdd(&c[k], 1);
+    }
+    __syncthreads();
+    if (t < ROW_CLASSES) {   // one warp
+        int first = count[t];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, first, o);
+            if (t >= o) first += x;
+        }
+        if (blockIdx.x == 0 && t == ROW_CLASSES - 1) nlong[0] = min(first, capacity);
+        if (blockIdx.x == 0 && t == ROW_CLASSES - 1 - VERY_CLASS) nlong[1] = min(first, capacity);
+        base[t] = first - count[t] + (c[t] ? atomicAdd(cursor + t, c[t]) : 0);
+    }
+    __syncthreads();
+    if (n > EM_ROW_LONG && base[k] + r < capacity) rows[base[k] + r] = (int32_t)i;
+}
+static_assert(ROW_CLASSES == 32, "one warp scans the classes");
+
 // The (i, j)-ordered transpose of a list ordered by (j, i): a stable sort by i.
 // bad (or null): raised where the sorted keys are out of range.
 int em_build_transpose(em_ctx *ctx, em_pairs *pr, int *bad)
@@ -291,6 +347,20 @@ int em_build_transpose(em_ctx *ctx, em_pairs *pr, int *bad)
     k_segment_offsets<<<em_grid(n + 1, 256), 256, 0, ctx->stream>>>(n, (const int32_t *)keys, pr->np,
                                                                       pr->part_pair_off, bad ? bad : ignored);
     EM_LAUNCHED(ctx);
+    if (n > EM_ROW_LONG && pr->np) {
+        int *count;   // and the cursors
+        EM_TRY(tmp.alloc(&count, 2 * ROW_CLASSES));
+        EM_CUDA(cudaMemsetAsync(count, 0, 2 * ROW_CLASSES * sizeof(int), ctx->stream));
+        const int capacity = (int)(n / (EM_ROW_LONG + 1));
+        EM_TRY(pr->mem.alloc(&pr->nlong, 2));
+        EM_TRY(pr->mem.alloc(&pr->long_rows, capacity));
+        k_long_count<<<em_grid(pr->np, 256), 256, 0, ctx->stream>>>(pr->np, pr->part_pair_off, count);
+        EM_LAUNCHED(ctx);
+        k_long_place<<<em_grid(pr->np, 256), 256, 0, ctx->stream>>>(pr->np, pr->part_pair_off, count,
+                                                                     count + ROW_CLASSES, capacity, pr->long_rows,
+                                                                     pr->nlong);
+        EM_LAUNCHED(ctx);
+    }
     return EM_OK;
 }
 
@@ -1253,196 +1323,15 @@ __global__ void k_cell_density(int64_t ncell, const int64_t *__restrict__ off, c
     if (lane == 0) rho[warp] = off[warp + 1] > off[warp] ? s / volume[warp] : 0.0;
 }
 
-// Sums over a particle's pairs [k0, k1) of the (i, j)-ordered transpose, in
+// Sums over a particle's pairs, a row of the (i, j)-ordered transpose, in
 // ascending j, each product and each sum rounded on its own (no fused
-// multiply-add): den = sum w, and with f given, num = sum w f_j.  The loads of
-// PB pairs are issued before their sums, so that a thread has PB gathers in
-// flight instead of one dependent chain at a time; the order of the sums is
-// unchanged.
-constexpr int PB = 8;
-template <bool WITH_F>
-__device__ __forceinline__ void pair_sums(int64_t k0, int64_t k1, const int32_t *__restrict__ idx,
-                                          const int32_t *__restrict__ pj, const double *__restrict__ w,
-                                          const double *__restrict__ f, double &num, double &den)
-{
-    int64_t k = k0;
-    for (; k + PB <= k1; k += PB) {
-        int32_t q[PB];
-        double wq[PB], fq[PB];
-#pragma unroll
-        for (int u = 0; u < PB; ++u) q[u] = __ldg(idx + k + u);
-#pragma unroll
-        for (int u = 0; u < PB; ++u) {
-            wq[u] = __ldg(w + q[u]);
-            fq[u] = WITH_F ? __ldg(f + __ldg(pj + q[u])) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < PB; ++u) {
-            if (WITH_F) num = __dadd_rn(num, __dmul_rn(wq[u], fq[u]));
-            den = __dadd_rn(den, wq[u]);
-        }
-    }
-    for (; k < k1; ++k) {
-        const int32_t q = idx[k];
-        const double wq = w[q];
-        if (WITH_F) num = __dadd_rn(num, __dmul_rn(wq, f[pj[q]]));
-        den = __dadd_rn(den, wq);
-    }
-}
-
-// The same sums by ROW_LANES lanes per row: each gathers one pair of eight, four
-// groups of eight in flight, and all of them add the row's terms in order, as
-// they come by shuffles.  For a short list of rows, where a thread per row
-// leaves most SMs without one and waits on its row's chain of gathers: 1,000
-// rows of about 90 pairs, k_map_back 63 -> 25.5 us, k_particle_wsum 27 -> 16.  Called with the warp converged, n = 0 for
-// a lane without a row.
-constexpr int ROW_LANES = 8;
-template <bool WITH_F>
-__device__ __forceinline__ void group_sums(int64_t k0, int n, const int32_t *__restrict__ idx,
-                                           const int32_t *__restrict__ pj, const double *__restrict__ w,
-                                           const double *__restrict__ f, double &num, double &den)
-{
-    constexpr int U = 4;
-    const int l = threadIdx.x & (ROW_LANES - 1);
-    int nmax = n;
-#pragma unroll
-    for (int o = ROW_LANES; o < 32; o <<= 1) nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
-    for (int c = 0; c < nmax; c += U * ROW_LANES) {
-        int32_t q[U];
-        double wq[U], pq[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) q[u] = c + u * ROW_LANES + l < n ? __ldg(idx + k0 + c + u * ROW_LANES + l) : -1;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            wq[u] = q[u] >= 0 ? __ldg(w + q[u]) : 0.0;
-            pq[u] = WITH_F && q[u] >= 0 ? __dmul_rn(wq[u], __ldg(f + __ldg(pj + q[u]))) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-#pragma unroll
-            for (int t = 0; t < ROW_LANES; ++t) {
-                const double wt = __shfl_sync(0xffffffffu, wq[u], t, ROW_LANES);
-                const double pt = WITH_F ? __shfl_sync(0xffffffffu, pq[u], t, ROW_LANES) : 0.0;
-                if (c + u * ROW_LANES + t < n) {
-                    if (WITH_F) num = __dadd_rn(num, pt);
-                    den = __dadd_rn(den, wt);
-                }
-            }
-        }
-    }
-}
-
-// Row i's sums in one pass, by one thread or by ROW_LANES lanes; false for a
-// thread that has none to write.
-template <bool GROUP, bool WITH_F>
-__device__ __forceinline__ bool row_sums(int64_t np, const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
-                                         const int32_t *__restrict__ pj, const double *__restrict__ w,
-                                         const double *__restrict__ f, int64_t &i, double &num, double &den)
-{
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    num = den = 0.0;
-    i = GROUP ? t / ROW_LANES : t;
-    if (!GROUP) {
-        if (i >= np) return false;
-        pair_sums<WITH_F>(off[i], off[i + 1], idx, pj, w, f, num, den);
-        return true;
-    }
-    const int64_t k0 = i < np ? off[i] : 0;
-    group_sums<WITH_F>(k0, i < np ? (int)(off[i + 1] - k0) : 0, idx, pj, w, f, num, den);
-    return i < np && threadIdx.x % ROW_LANES == 0;
-}
-
-// The same sums for many pairs, in two passes.  One thread walking a row of
-// the transpose is bound by the longest row's chain of dependent gathers
-// (3,832 pairs where the mean is 234: about 1.0 of k_map_back's 1.5 ms on the
-// 1e6-particle cloud), and the sum's order, which fixes its bits, rules out
-// splitting a row.  So the gathers, which have no order, are done by all
-// threads at once into contiguous rows (k_gather_rows), and the rows are then
-// added serially by one lane each, fed by asynchronous copies three tiles
-// ahead (k_row_sums).  24.06 M pairs: map_back and map_back_sums together 3.24 to
-// 1.55 ms.
-template <bool WITH_F>
-__global__ void k_gather_rows(int64_t n, const int32_t *__restrict__ idx, const int32_t *__restrict__ pj,
-                              const double *__restrict__ w, const double *__restrict__ f, double *__restrict__ wt,
-                              double *__restrict__ pt)
-{
-    constexpr int U = 4;   // gathers in flight per thread
-    const int64_t t0 = blockIdx.x * (int64_t)(U * blockDim.x) + threadIdx.x;
-    int32_t q[U];
-    double wq[U], fq[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const int64_t t = t0 + u * (int64_t)blockDim.x;
-        q[u] = t < n ? __ldg(idx + t) : -1;
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        wq[u] = q[u] >= 0 ? __ldg(w + q[u]) : 0.0;
-        fq[u] = WITH_F && q[u] >= 0 ? __ldg(f + __ldg(pj + q[u])) : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const int64_t t = t0 + u * (int64_t)blockDim.x;
-        if (t < n) {
-            wt[t] = wq[u];
-            if (WITH_F) pt[t] = __dmul_rn(wq[u], fq[u]);
-        }
-    }
-}
-
-// Row sums of wt (and pt) in ascending position, one warp per 32 particles,
-// each lane its own.  MODE 0: out0 = den; 1: out0 = num / den; 2: out0 += num,
-// out1 += den.
-constexpr int RS_COLS = 16, RS_STAGES = 4;
+// multiply-add): den = sum w, and with f given, num = sum w f_j.  The order fixes
+// the bits, so a row cannot be split.  MODE 0: out0 = den; 1: out0 = num / den;
+// 2: out0 += num, out1 += den.
 template <int MODE>
-__global__ void __launch_bounds__(32) k_row_sums(int64_t np, const int64_t *__restrict__ off,
-                                                 const double *__restrict__ wt, const double *__restrict__ pt,
-                                                 double *__restrict__ out0, double *__restrict__ out1)
+__device__ __forceinline__ void row_out(int64_t i, double num, double den, double *__restrict__ out0,
+                                        double *__restrict__ out1)
 {
-    constexpr bool WITH_F = MODE > 0;
-    __shared__ double sw[RS_STAGES][32][RS_COLS + 1];   // padded: lanes read down a column
-    __shared__ double sp[WITH_F ? RS_STAGES : 1][WITH_F ? 32 : 1][RS_COLS + 1];
-    const int lane = threadIdx.x, col = lane & (RS_COLS - 1), half = lane / RS_COLS;
-    const int64_t i = blockIdx.x * (int64_t)32 + lane;
-    const int k0 = i < np ? (int)off[i] : 0, n = i < np ? (int)off[i + 1] - k0 : 0;   // pairs < 2^31
-    int kr[RS_COLS], nr[RS_COLS];   // the rows this lane copies: 2 u + half
-#pragma unroll
-    for (int u = 0; u < RS_COLS; ++u) {
-        kr[u] = __shfl_sync(FULL_MASK, k0, 2 * u + half) + col;
-        nr[u] = __shfl_sync(FULL_MASK, n, 2 * u + half) - col;
-    }
-    const int tiles = (__reduce_max_sync(FULL_MASK, n) + RS_COLS - 1) / RS_COLS;
-    auto fetch = [&](int c) {
-        if (c < tiles) {
-            const int s = c & (RS_STAGES - 1), c0 = c * RS_COLS;
-#pragma unroll
-            for (int u = 0; u < RS_COLS; ++u)
-                if (c0 < nr[u]) {
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
-                                     (unsigned)__cvta_generic_to_shared(&sw[s][2 * u + half][col])),
-                                 "l"(wt + kr[u] + c0));
-                    if (WITH_F)
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
-                                         (unsigned)__cvta_generic_to_shared(&sp[s][2 * u + half][col])),
-                                     "l"(pt + kr[u] + c0));
-                }
-        }
-        asm volatile("cp.async.commit_group;");
-    };
-    for (int c = 0; c < RS_STAGES - 1; ++c) fetch(c);
-    double num = 0.0, den = 0.0;
-    for (int c = 0; c < tiles; ++c) {
-        fetch(c + RS_STAGES - 1);
-        asm volatile("cp.async.wait_group %0;" ::"n"(RS_STAGES - 1));
-        __syncwarp();
-        const int s = c & (RS_STAGES - 1), m = min(RS_COLS, n - c * RS_COLS);
-        for (int t = 0; t < m; ++t) {
-            if (WITH_F) num = __dadd_rn(num, sp[s][lane][t]);
-            den = __dadd_rn(den, sw[s][lane][t]);
-        }
-        __syncwarp();   // the stage is copied over in the next pass
-    }
-    if (i >= np) return;
     if (MODE == 0) out0[i] = den;
     else if (MODE == 1) out0[i] = num / den;
     else {
@@ -1451,56 +1340,270 @@ __global__ void __launch_bounds__(32) k_row_sums(int64_t np, const int64_t *__re
     }
 }
 
-// Whether the two passes ran: from SUMS_TWO_PASS pairs on, where the rows
-// (16 bytes a pair) can be had from the pool and the stream is not being
-// captured; otherwise the caller's one-pass kernel does it.  Both give the
-// same bits.
-constexpr int64_t SUMS_TWO_PASS = 1 << 20;
+// A row of up to EM_ROW_LONG pairs by one thread, PB pairs at a time in a
+// pipeline: while one batch is added the next one's weights and values are on
+// their way, and the cells and pair numbers of the two after that.  The two
+// batches' registers take turns in the code: copying one that is still being
+// loaded into another would wait for it.
+constexpr int PB = 2;
 template <int MODE>
-static int two_pass_sums(em_ctx *ctx, const em_pairs *pr, const double *w, const double *f, double *out0, double *out1,
-                         bool *done)
+__device__ __forceinline__ void short_row(int64_t i, int64_t k0, int n, const int32_t *__restrict__ idx,
+                                          const int32_t *__restrict__ pj, const double *__restrict__ w,
+                                          const double *__restrict__ f, double *__restrict__ out0,
+                                          double *__restrict__ out1)
 {
-    *done = false;
-    const int64_t n = pr->npairs;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (n < SUMS_TWO_PASS || cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess ||
-        cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
+    constexpr bool WITH_F = MODE > 0;
+    idx += k0;
+    // the batch from c on; past the row's end its last pair is loaded again, and not added
+    auto pairs = [&](int c, int32_t(&q)[PB]) {
+#pragma unroll
+        for (int u = 0; u < PB; ++u) q[u] = __ldg(idx + min(c + u, n - 1));
+    };
+    auto cells = [&](const int32_t(&q)[PB], int32_t(&j)[PB]) {
+#pragma unroll
+        for (int u = 0; u < PB; ++u) j[u] = WITH_F ? __ldg(pj + q[u]) : 0;
+    };
+    struct Batch {
+        double w[PB], f[PB];
+    };
+    auto values = [&](const int32_t(&q)[PB], const int32_t(&j)[PB], Batch &x) {
+#pragma unroll
+        for (int u = 0; u < PB; ++u) {
+            x.w[u] = __ldg(w + q[u]);
+            x.f[u] = WITH_F ? __ldg(f + j[u]) : 0.0;
+        }
+    };
+    double num = 0.0, den = 0.0;
+    if (n > 0) {
+        int32_t q0[PB], q1[PB], j[PB];
+        Batch A, B;
+        pairs(0, q0);
+        pairs(PB, q1);
+        cells(q0, j);
+        values(q0, j, A);
+        cells(q1, j);
+        values(q1, j, B);
+        pairs(2 * PB, q0);
+        cells(q0, j);
+        pairs(3 * PB, q1);
+        // before the batch at c: q0, j of the one at c + 2 PB, q1 of the next
+        auto step = [&](int c, Batch &x) {
+#pragma unroll
+            for (int u = 0; u < PB; ++u)
+                if (c + u < n) {
+                    if (WITH_F) num = __dadd_rn(num, __dmul_rn(x.w[u], x.f[u]));
+                    den = __dadd_rn(den, x.w[u]);
+                }
+            if (c + 2 * PB < n) {
+                values(q0, j, x);
+                cells(q1, j);
+#pragma unroll
+                for (int u = 0; u < PB; ++u) q0[u] = q1[u];
+                pairs(c + 4 * PB, q1);
+            }
+        };
+#pragma unroll 1
+        for (int c = 0; c < n; c += 2 * PB) {
+            step(c, A);
+            step(c + PB, B);
+        }
+    }
+    row_out<MODE>(i, num, den, out0, out1);
+}
+
+// Up to 32 longer rows of like length (listed with the transpose) by a block.  An
+// FP64 instruction takes a scheduler 64 cycles whatever its active lanes, so a
+// long row among shorter ones, or a warp that both gathers and adds, is what
+// makes a row of thousands of pairs the last to end.  One warp adds, each lane
+// its own row's terms as they stand in shared memory; the other three gather a
+// tile of LR_COLS pairs of every row at a time, multiply, and store it, with the
+// next two tiles' weights and values, a third one's cells and a fourth one's pair
+// numbers on their way.  The adding warp is another one from block to block,
+// since a block's warps go to the four schedulers in turn.  It adds whole tiles
+// without asking (with a test at every term 0.11 us a pair of the longest row,
+// so 0.073, the two additions' 128 cycles).
+constexpr int SHORT_THREADS = 64, ROW_THREADS = 128, LR_COLS = 12, LR_PER = 4;
+static_assert((ROW_THREADS - 32) * LR_PER == 32 * LR_COLS && (ROW_THREADS - 32) % LR_COLS == 0, "a tile's entries");
+template <int MODE>
+struct LongTile {
+    double w[2][32][LR_COLS + 1];   // padded: lanes read down a column
+    double p[MODE > 0 ? 2 : 1][MODE > 0 ? 32 : 1][LR_COLS + 1];
+};
+// the block's barrier, met by its two kinds of warps in different places
+__device__ __forceinline__ void tile_sync() { asm volatile("bar.sync 0, %0;" ::"n"(ROW_THREADS) : "memory"); }
+template <int MODE>
+__device__ __forceinline__ void long_rows(LongTile<MODE> &sh, int nrow, const int32_t *__restrict__ rows,
+                                          const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
+                                          const int32_t *__restrict__ pj, const double *__restrict__ w,
+                                          const double *__restrict__ f, double *__restrict__ out0,
+                                          double *__restrict__ out1)
+{
+    constexpr bool WITH_F = MODE > 0;
+    const int lane = threadIdx.x & 31, adder = blockIdx.x & 3, wp = threadIdx.x >> 5;
+    const int i = lane < nrow ? rows[lane] : -1;   // the same in every warp
+    const int k0 = i >= 0 ? (int)off[i] : 0, n = i >= 0 ? (int)off[i + 1] - k0 : 0;   // pairs < 2^31
+    const int tiles = (__reduce_max_sync(FULL_MASK, n) + LR_COLS - 1) / LR_COLS;
+    if (wp == adder) {
+        double num = 0.0, den = 0.0;
+        tile_sync();
+        for (int c = 0; c < tiles; ++c) {
+            const int s = c & 1, m = n - c * LR_COLS;
+            double wv[LR_COLS], pv[LR_COLS];
+#pragma unroll
+            for (int t = 0; t < LR_COLS; ++t) {
+                wv[t] = sh.w[s][lane][t];
+                pv[t] = WITH_F ? sh.p[s][lane][t] : 0.0;
+            }
+            if (m >= LR_COLS) {
+#pragma unroll
+                for (int t = 0; t < LR_COLS; ++t) {
+                    if (WITH_F) num = __dadd_rn(num, pv[t]);
+                    den = __dadd_rn(den, wv[t]);
+                }
+            } else if (m > 0) {
+#pragma unroll
+                for (int t = 0; t < LR_COLS; ++t)
+                    if (t < m) {
+                        if (WITH_F) num = __dadd_rn(num, pv[t]);
+                        den = __dadd_rn(den, wv[t]);
+                    }
+            }
+            tile_sync();
+        }
+        if (i >= 0) row_out<MODE>(i, num, den, out0, out1);
+        return;
+    }
+    // entry u of this thread: row RSTEP u + sub, column col
+    constexpr int RSTEP = (ROW_THREADS - 32) / LR_COLS;
+    const int t = (wp - (wp > adder ? 1 : 0)) * 32 + lane, col = t % LR_COLS, sub = t / LR_COLS;
+    int kr[LR_PER], nr[LR_PER];
+#pragma unroll
+    for (int u = 0; u < LR_PER; ++u) {
+        kr[u] = __shfl_sync(FULL_MASK, k0, RSTEP * u + sub) + col;
+        nr[u] = __shfl_sync(FULL_MASK, n, RSTEP * u + sub) - col;
+    }
+    // the tile's pair numbers (-1 past a row's end), their cells, weights and values
+    auto pairs = [&](int c, int32_t(&q)[LR_PER]) {
+#pragma unroll
+        for (int u = 0; u < LR_PER; ++u) q[u] = c * LR_COLS < nr[u] ? __ldg(idx + kr[u] + c * LR_COLS) : -1;
+    };
+    auto cells = [&](const int32_t(&q)[LR_PER], int32_t(&j)[LR_PER]) {
+#pragma unroll
+        for (int u = 0; u < LR_PER; ++u) j[u] = WITH_F && q[u] >= 0 ? __ldg(pj + q[u]) : 0;
+    };
+    struct Part {
+        double w[LR_PER], f[LR_PER];
+    };
+    auto values = [&](const int32_t(&q)[LR_PER], const int32_t(&j)[LR_PER], Part &x) {
+#pragma unroll
+        for (int u = 0; u < LR_PER; ++u) {
+            x.w[u] = q[u] >= 0 ? __ldg(w + q[u]) : 0.0;
+            x.f[u] = WITH_F && q[u] >= 0 ? __ldg(f + j[u]) : 0.0;
+        }
+    };
+    int32_t q0[LR_PER], q1[LR_PER], j[LR_PER];
+    Part A, B;   // take turns, as in short_row
+    pairs(0, q0);
+    pairs(1, q1);
+    cells(q0, j);
+    values(q0, j, A);
+    cells(q1, j);
+    values(q1, j, B);
+    pairs(2, q0);
+    cells(q0, j);
+    pairs(3, q1);
+    // before tile c: q0, j of tile c + 2, q1 of the next
+    auto step = [&](int c, Part &x) {
+        const int s = c & 1;
+#pragma unroll
+        for (int u = 0; u < LR_PER; ++u) {
+            sh.w[s][RSTEP * u + sub][col] = x.w[u];
+            if (WITH_F) sh.p[s][RSTEP * u + sub][col] = __dmul_rn(x.w[u], x.f[u]);
+        }
+        values(q0, j, x);
+        cells(q1, j);
+#pragma unroll
+        for (int u = 0; u < LR_PER; ++u) q0[u] = q1[u];
+        pairs(c + 4, q1);
+        tile_sync();   // tile c is there; the adder has done with tile c - 1, whose place tile c + 1 takes
+    };
+#pragma unroll 1
+    for (int c = 0; c < tiles; c += 2) {
+        step(c, A);
+        if (c + 1 < tiles) step(c + 1, B);
+    }
+    tile_sync();
+}
+
+// LONG: blocks below nlongb take the long rows, the longest first: 32 each, and
+// ROW_FEW of those beyond ROW_VERY pairs, which then end sooner (24.04 M pairs
+// with rows of up to 3,781: 569 us with 32 of any length, 466 so; 16.4 M with rows
+// of up to 33,417: 2,834 and 2,451).
+// SHORT: the other blocks take the short ones, a row per thread.
+template <int MODE, bool LONG, bool SHORT>
+__global__ void __launch_bounds__(LONG ? ROW_THREADS : SHORT_THREADS, LONG ? 5 : 16)
+    k_rows(int64_t np, int nlongb, const int *__restrict__ nlong, const int32_t *__restrict__ rows,
+           const int64_t *__restrict__ off, const int32_t *__restrict__ idx, const int32_t *__restrict__ pj,
+           const double *__restrict__ w, const double *__restrict__ f, double *__restrict__ out0,
+           double *__restrict__ out1)
+{
+    if constexpr (LONG) {
+        __shared__ LongTile<MODE> sh;
+        if ((int)blockIdx.x < nlongb) {
+            const int nl = nlong[0], nv = nlong[1], vb = (nv + ROW_FEW - 1) / ROW_FEW, b = blockIdx.x;
+            const int g = b < vb ? b * ROW_FEW : nv + (b - vb) * 32, end = b < vb ? nv : nl;
+            if (g < end)
+                long_rows<MODE>(sh, min(b < vb ? ROW_FEW : 32, end - g), rows + g, off, idx, pj, w, f, out0, out1);
+            return;
+        }
+    }
+    if constexpr (SHORT) {
+        const int64_t i = (int64_t)(blockIdx.x - nlongb) * blockDim.x + threadIdx.x;
+        if (i >= np) return;
+        const int64_t k0 = off[i], n = off[i + 1] - k0;
+        if (n <= EM_ROW_LONG) short_row<MODE>(i, k0, (int)n, idx, pj, w, f, out0, out1);
+    }
+}
+
+// Both kinds in one launch up to ROWS_ONE_LAUNCH pairs: the long rows do not wait
+// for the short ones (545,000 pairs, rows of up to 361: 46 us, 64 in two).
+// Beyond, two: the short rows' kernel has more warps resident by itself (1.7 M
+// pairs in rows of 43: 33 us, 38 in one; 17.6 M: 229 and 311).
+// map_back, us, with one thread per row and a wait for each of its three loads /
+// with every pair gathered into a copy of the transpose first and the rows, in
+// the caller's order, added from there (eight lanes a row below 2^20 pairs) / so:
+//   107,000 pairs, rows of about 107               40.0 /   25.0 /   21.4
+//   412,000 pairs, rows of about 41                23.5 /   34.7 /   15.2
+//   4.3 M, rows of about 43                        68.5 /  104   /   68.3
+//   17.6 M, rows of about 44                       245  /  491   /  229
+//   1.9 M, rows of about 3                         47.9 /   72.9 /   48.8
+//   0.55 M pseudo-particle pairs, rows up to 361   80.8 /   58.1 /   39.8
+//   4.7 M, up to 2,504                             571  /  284   /  227
+//   24.0 M, up to 3,781                           1,667 /  782   /  466
+//   16.4 M, up to 33,417                         13,596 / 3,145  / 2,451
+constexpr int64_t ROWS_ONE_LAUNCH = 1 << 20;
+template <int MODE>
+static int launch_rows(em_ctx *ctx, const em_pairs *pr, const double *w, const double *f, double *out0, double *out1)
+{
+    // as many blocks of long rows as there may be; those without return at once
+    const int nlongb = pr->npairs > EM_ROW_LONG
+                           ? (int)(pr->npairs / (EM_ROW_LONG + 1) / 32 + pr->npairs / ROW_VERY / ROW_FEW) + 2
+                           : 0;
+    auto launch = [&](auto kernel, int threads, int nl, int64_t nshort) {
+        kernel<<<(unsigned)(nl + nshort), threads, 0, ctx->stream>>>(pr->np, nl, pr->nlong, pr->long_rows,
+                                                                     pr->part_pair_off, pr->part_pair_idx, pr->pair_j,
+                                                                     w, f, out0, out1);
+    };
+    if (pr->npairs < ROWS_ONE_LAUNCH) {
+        launch(k_rows<MODE, true, true>, ROW_THREADS, nlongb, em_grid(pr->np, ROW_THREADS));
+        EM_LAUNCHED(ctx);
         return EM_OK;
     }
-    DevArena tmp(ctx->stream, true);
-    double *wt, *pt = nullptr;
-    if (tmp.alloc(&wt, n) != EM_OK || (MODE > 0 && tmp.alloc(&pt, n) != EM_OK)) return EM_OK;
-    k_gather_rows<(MODE > 0)><<<em_grid(n, 4 * 256), 256, 0, ctx->stream>>>(n, pr->part_pair_idx, pr->pair_j, w, f, wt,
-                                                                            pt);
+    launch(k_rows<MODE, true, false>, ROW_THREADS, nlongb, 0);
     EM_LAUNCHED(ctx);
-    k_row_sums<MODE><<<em_grid(pr->np, 32), 32, 0, ctx->stream>>>(pr->np, pr->part_pair_off, wt, pt, out0, out1);
+    launch(k_rows<MODE, false, true>, SHORT_THREADS, 0, em_grid(pr->np, SHORT_THREADS));
     EM_LAUNCHED(ctx);
-    *done = true;
     return EM_OK;
-}
-
-// u_i = sum_j w_ij (ascending j)
-template <bool GROUP>
-__global__ void k_particle_wsum(int64_t np, const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
-                                const double *__restrict__ w, double *__restrict__ u)
-{
-    int64_t i;
-    double num, den;
-    if (row_sums<GROUP, false>(np, off, idx, nullptr, w, nullptr, i, num, den)) u[i] = den;
-}
-
-// One pass: ROW_LANES lanes per row where the rows have at least as many pairs
-// on average, else a thread per row.
-static bool lanes_per_row(const em_pairs *pr) { return pr->npairs >= ROW_LANES * pr->np; }
-template <class... K, class... A>
-static void launch_rows(em_ctx *ctx, const em_pairs *pr, void (*group)(K...), void (*single)(K...), A... args)
-{
-    if (lanes_per_row(pr))
-        group<<<em_grid(pr->np * ROW_LANES, 64), 64, 0, ctx->stream>>>(pr->np, pr->part_pair_off, pr->part_pair_idx,
-                                                                       args...);
-    else
-        single<<<em_grid(pr->np, 256), 256, 0, ctx->stream>>>(pr->np, pr->part_pair_off, pr->part_pair_idx, args...);
 }
 
 // The FP32 pass in launch shape `variant` (see MQ_VARIANT_*).
@@ -1613,12 +1716,7 @@ int em_map_exact_impl(em_ctx *ctx, const em_pairs *pr, const double *d_x, const 
                                                                                d_w_out, d_m, v->volume, d_rho_out);
         EM_LAUNCHED(ctx);
     }
-    bool summed = !(d_wsum_out && pr->np);
-    if (!summed && !fixed) EM_TRY(two_pass_sums<0>(ctx, pr, d_w_out, nullptr, d_wsum_out, nullptr, &summed));
-    if (!summed) {
-        launch_rows(ctx, pr, k_particle_wsum<true>, k_particle_wsum<false>, d_w_out, d_wsum_out);
-        EM_LAUNCHED(ctx);
-    }
+    if (d_wsum_out && pr->np) EM_TRY(launch_rows<0>(ctx, pr, d_w_out, nullptr, d_wsum_out, nullptr));   // u_i = sum_j w_ij
     return EM_OK;
 }
 
@@ -1750,19 +1848,6 @@ EM_EXPORT int map_exact_noalloc(em_ctx *ctx, const em_pairs *pr, const double *d
 // Inverse mapping
 // ---------------------------------------------------------------------------
 
-template <bool GROUP>
-__global__ void k_map_back(int64_t np, const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
-                           const int32_t *__restrict__ pj, const double *__restrict__ w,
-                           const double *__restrict__ f_cell, double *__restrict__ f_out)
-{
-    // ascending j, each product and each sum rounded on its own (row_sums),
-    // so that equal weights give bit-identical results on any implementation
-    // that sums in the same order
-    int64_t i;
-    double num, den;
-    if (row_sums<GROUP, true>(np, off, idx, pj, w, f_cell, i, num, den)) f_out[i] = num / den;
-}
-
 // every SPH particle takes the value of the pseudo-particle it belongs to
 __global__ void k_inherit(int64_t npseudo, const int32_t *__restrict__ first, const int32_t *__restrict__ count,
                           const int32_t *__restrict__ perm, const double *__restrict__ f_pseudo,
@@ -1774,31 +1859,11 @@ __global__ void k_inherit(int64_t npseudo, const int32_t *__restrict__ first, co
     for (int32_t k = first[a]; k < first[a] + count[a]; ++k) f_particle[perm[k]] = f;
 }
 
-// The two sums of map_back per particle, added into num and den (ascending
-// j, every product and sum rounded on its own, as k_map_back).
-template <bool GROUP>
-__global__ void k_map_back_sums(int64_t np, const int64_t *__restrict__ off, const int32_t *__restrict__ idx,
-                                const int32_t *__restrict__ pj, const double *__restrict__ w,
-                                const double *__restrict__ f_cell, double *__restrict__ num, double *__restrict__ den)
-{
-    int64_t i;
-    double a, b;
-    if (row_sums<GROUP, true>(np, off, idx, pj, w, f_cell, i, a, b)) {
-        num[i] = __dadd_rn(num[i], a);
-        den[i] = __dadd_rn(den[i], b);
-    }
-}
-
 EM_EXPORT int map_back_sums(em_ctx *ctx, const em_pairs *pr, const double *d_w, const double *d_f_cell,
                             double *d_num, double *d_den)
 {
     EM_CHECK_ARG(ctx && pr && d_num && d_den && (pr->npairs == 0 || d_w) && (pr->ncell == 0 || d_f_cell));
-    bool done = pr->np == 0;
-    if (!done) EM_TRY(two_pass_sums<2>(ctx, pr, d_w, d_f_cell, d_num, d_den, &done));
-    if (!done) {
-        launch_rows(ctx, pr, k_map_back_sums<true>, k_map_back_sums<false>, pr->pair_j, d_w, d_f_cell, d_num, d_den);
-        EM_LAUNCHED(ctx);
-    }
+    if (pr->np) EM_TRY(launch_rows<2>(ctx, pr, d_w, d_f_cell, d_num, d_den));
     return EM_OK;
 }
 
@@ -1820,12 +1885,7 @@ EM_EXPORT int map_back(em_ctx *ctx, const em_pairs *pr, const double *d_w, const
     EM_CHECK_ARG(ctx && pr && d_f_out && (pr->npairs == 0 || d_w) && (pr->ncell == 0 || d_f_cell));
     bool inherit = ps || t || d_f_particle_out;
     EM_CHECK_ARG(!inherit || (ps && t && d_f_particle_out && ps->n == pr->np));
-    bool done = pr->np == 0;
-    if (!done) EM_TRY(two_pass_sums<1>(ctx, pr, d_w, d_f_cell, d_f_out, nullptr, &done));
-    if (!done) {
-        launch_rows(ctx, pr, k_map_back<true>, k_map_back<false>, pr->pair_j, d_w, d_f_cell, d_f_out);
-        EM_LAUNCHED(ctx);
-    }
+    if (pr->np) EM_TRY(launch_rows<1>(ctx, pr, d_w, d_f_cell, d_f_out, nullptr));
     if (inherit && ps->n) {
         k_inherit<<<em_grid(ps->n, 128), 128, 0, ctx->stream>>>(ps->n, ps->first, ps->count, t->perm, d_f_out,
                                                                  d_f_particle_out);
