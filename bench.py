@@ -508,13 +508,14 @@ ALGO_WORK = {
 }
 # Implementation work of the FP32 pass per pair: the FP32 operations it executes
 # (FMA = 2), float-float bookkeeping included, for the utilisation figure beside
-# the algorithmic one.  Counted by ncu on the 1e5 sphere's 4.34 M pairs with the
-# same arithmetic unpacked (the counters leave packed instructions out); the 1e6
-# cloud's pairs take the same time to 5%.
-IMPL_FLOPS = {"pseudo_1e6": 30432.0, "sphere_1e5": 30432.0}
+# the algorithmic one.  Counted by ncu with the same arithmetic unpacked (the
+# counters leave packed instructions out) on the 1e5 sphere's 4.34 M pairs and on
+# the 4.68 M pseudo-particle pairs of the 2e5 cloud, whose count stands for the
+# 1e6 cloud's too (their pairs are alike: ALGO_WORK).
+IMPL_FLOPS = {"pseudo_1e6": 35096.0, "pseudo_2e5": 35096.0, "sphere_1e5": 30432.0}
 # DRAM traffic of one k_map_fp32 launch per pair (ncu, dram__bytes_read.sum +
 # dram__bytes_write.sum over the pairs of the launch), per workload, from a
-# capture of the current kernel (profiles/k_map_fp32_dram_pseudo_1e6.md)
+# one-pass capture of the current kernel
 TRAFFIC_PER_PAIR = {"pseudo_1e6": 108.53}
 
 

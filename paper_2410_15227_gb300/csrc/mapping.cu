@@ -1290,9 +1290,11 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_map_fp32(int64_t npairs, c
         w[k] = wk;
         // error bound of the FP32 pass: est_k = (ulps) 2^-24 times the sum of
         // the non-negative pieces it summed.  With the default 8 ulps the
-        // largest error/bound ratio seen against FP64 on the 1e5 and 1e6
-        // clouds was 0.81; tiny cells deep inside large kernels (h / V^(1/3)
-        // above ~12, as in the 8e6 cloud) need more
+        // largest error against FP64 on the 1e5 and 1e6 clouds is 0.35 of the
+        // bound where that is above 1e-5 |w|, 0.64 from 3e-6 to 1e-5 |w| (0.51
+        // for tiny cells deep inside large kernels, h / V^(1/3) above 12); below
+        // 1e-6 |w| it reaches 2.2 of it, 1.2e-6 |w|.  With 3 one of the 8e6
+        // cloud's 145.6 M pairs misses the tolerance, with 4 none
         const double est = est_k * magd;
         flag = force || !(est <= fmax((double)tol * fabs(wk), 1e-14));
     }
@@ -1420,8 +1422,8 @@ __device__ __forceinline__ void short_row(int64_t i, int64_t k0, int n, const in
 // next two tiles' weights and values, a third one's cells and a fourth one's pair
 // numbers on their way.  The adding warp is another one from block to block,
 // since a block's warps go to the four schedulers in turn.  It adds whole tiles
-// without asking (with a test at every term 0.11 us a pair of the longest row,
-// so 0.073, the two additions' 128 cycles).
+// without asking (with a test at every term 0.11 us a pair of the longest row, so
+// 0.073, 0.062 of it the two additions' 128 cycles).
 constexpr int SHORT_THREADS = 64, ROW_THREADS = 128, LR_COLS = 12, LR_PER = 4;
 static_assert((ROW_THREADS - 32) * LR_PER == 32 * LR_COLS && (ROW_THREADS - 32) % LR_COLS == 0, "a tile's entries");
 template <int MODE>

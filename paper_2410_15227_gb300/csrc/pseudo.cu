@@ -249,6 +249,10 @@ constexpr int HS_LEAVES = 4;        // 32-point leaves a walk reads together (th
 // of HS_TEAM: each warp of the team takes its share of every walk's leaves, and
 // all add up and decide alike.  (1e6 particles: the longest node 11.5 M cycles
 // against a mean of 0.12 M; tree, walk and h 8.6 ms without teams, 6.4 with.)
+// make_pseudo_particles of these, and with h_tol = 1e-2 (FP64 iterates): 5.7 and
+// 8.8 ms with 24 batches, 4.65 and 7.85 with 48, 4.5 and 7.8 with 96, but a
+// lone warp's sums then have twice the terms (HS_EPS); teams of 4: 4.65 and 8.4,
+// of 16: 4.9 and 7.9.
 constexpr int HS_TEAM = 8;
 constexpr int HS_HEAVY = 48;   // batches of HS_LEAVES leaves: 6,144 entries
 
@@ -795,10 +799,9 @@ __device__ __forceinline__ bool solve_node(const em::ChunkTree &T, const Populat
 
 // One warp per pseudo-particle; the heavy ones are listed for k_h_solve_heavy.
 // 1e6 particles (94,193 nodes, 5,733 of them bisected): 417,533 FP64
-// evaluations of n(h) and 298,116 signs, each with its walk, took 11.2 ms;
-// 112,000 FP64 evaluations, 1.5 walks and 1.8 sums over a list per node took
-// 5.8, most of it the tail of the few nodes whose 2h holds thousands of the
-// population.
+// evaluations of n(h) and 298,116 signs, each with its walk, took 11.2 ms; 1.1
+// FP64 evaluations, 1.5 walks and 1.8 sums over a list per node take 2.2, and
+// 0.9 the few nodes whose 2h holds thousands of the population (k_h_solve_heavy).
 __global__ void __launch_bounds__(32 * HS_WARPS, 6) k_h_solve(
     int64_t npseudo, em::ChunkTree T, Population P, const double *__restrict__ px, const double *__restrict__ py,
     const double *__restrict__ pz, double h_fact, double tol, int max_newton, float margin, double *__restrict__ ph,

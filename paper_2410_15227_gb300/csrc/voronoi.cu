@@ -18,9 +18,9 @@
 // face-vertices: every vertex belongs to three faces) and its counts; after
 // the scan of the counts, a copy pass moves the slots to the cells' offsets.
 //
-// 262,144 sites (16.6 cuts and 86 candidates a cell): 19.9 ms with the derived
+// 262,144 sites (16.6 cuts and 86 candidates a cell): 20 ms with the derived
 // geometry, 23.6 with every candidate tested on its own and its bisector formed
-// on every lane; resident blocks per SM from 10 to 14 make no difference.
+// on every lane (the same code's runs differ by 5%, with its place in memory).
 #include <algorithm>
 #include <cmath>
 
@@ -197,13 +197,12 @@ __device__ void build_one(C &c, const BuildArgs &a, int64_t s, bool first_pass)
 
 // First pass: one warp per cell (sorted index s), the cell in a small
 // shared-memory footprint (MAXV_FIRST vertices) so that more warps fit an SM.
-// First pass, one warp per cell.  Its warps sit all over a long program, so that
-// fetching instructions is its largest stall (8.7 of 16.8 cycles per issue with
-// 156 KB of code): loops are kept rolled but for the three edges or planes of a
-// vertex, and the FP64 side tests, the box test and the clip have one call site
-// each.  262,144 sites with the read-out, mean of three runs that differ by 5%
-// with the code's place: 20.8 ms at 156 KB, 18.7 at 110 KB; 19.4 with 12 blocks
-// per SM asked for instead of 14.
+// Its warps sit all over a long program, so that fetching instructions is its
+// largest stall (8.7 of 16.8 cycles per issue with 156 KB of code, 4.9 with 110):
+// loops are kept rolled but for the three edges or planes of a vertex, and the
+// FP64 side tests, the box test and the clip have one call site each.  The
+// kernel on 65,536 sites: 4.24 ms at 156 KB, 3.74 at 110.  From 10 to 14 resident
+// blocks per SM asked for differ by less than the runs of one of them.
 __global__ void __launch_bounds__(32 * VW, EM_VOR_MINB) k_voronoi_build(BuildArgs a)
 {
     __shared__ WCell<MAXV_FIRST> cells[VW];

@@ -231,7 +231,6 @@ __device__ int wcompact(C &c)
             ++n;
         }
 #pragma unroll 1
-#pragma unroll 1
         for (int t = 0; t < c.nt; ++t) {
             const uint32_t w = c.tri[cur][t];
             c.tri[cur][t] = (uint32_t)map[byte_of(w, 0)] | (uint32_t)map[byte_of(w, 1)] << 8 | (uint32_t)map[byte_of(w, 2)] << 16;
