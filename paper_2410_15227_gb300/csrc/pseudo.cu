@@ -249,12 +249,18 @@ constexpr int HS_LEAVES = 4;        // 32-point leaves a walk reads together (th
 // of HS_TEAM: each warp of the team takes its share of every walk's leaves, and
 // all add up and decide alike.  (1e6 particles: the longest node 11.5 M cycles
 // against a mean of 0.12 M; tree, walk and h 8.6 ms without teams, 6.4 with.)
-// make_pseudo_particles of these, and with h_tol = 1e-2 (FP64 iterates): 5.7 and
-// 8.8 ms with 24 batches, 4.65 and 7.85 with 48, 4.5 and 7.8 with 96, but a
-// lone warp's sums then have twice the terms (HS_EPS); teams of 4: 4.65 and 8.4,
-// of 16: 4.9 and 7.9.
+// The limit: a team redoes what the warp had done of the node, and FP64 sums,
+// bound by the FP64 pipe, gain nothing from it until the other nodes have ended.
+// make_pseudo_particles in us with h_tol 1e-2, 1e-8 and 1e-13, with 48 / 96 / 192
+// batches / without a limit:
+//   1e6 particles, theta 0.065   6750 9446 3377 / 6519 8949 3407 / 6736 9071 3370 / 9822 11987 4170
+//   1e6, theta 0.25              1345 1933  730 / 1157 1515  480 / 1189 1489  487 / 1158  1523  495
+//   3e5, theta 0.2                930 1465  509 /  877 1182  407 /  870 1177  406 /  875  1184  408
+//   1e5, theta 0.1               1324 2098  819 / 1514 2092  821 / 1848 2035  801 / 1831  2071  822
+// Teams of 4 instead of 8: 2% to 7% slower on the first with h_tol 1e-2, of 16: 6%
+// with 1e-13.
 constexpr int HS_TEAM = 8;
-constexpr int HS_HEAVY = 48;   // batches of HS_LEAVES leaves: 6,144 entries
+constexpr int HS_HEAVY = 96;   // batches of HS_LEAVES leaves: 12,288 entries
 
 // A node under solution: its position, the neighbours of its last walk (every
 // population entry within r of it if n >= 0; n = -1: more than the list holds),
@@ -606,7 +612,7 @@ __device__ __forceinline__ Step32 step32(Sum32 u, float hf, float e, float eps)
     r.least = (fabsf(a - 1.f) - e * fabsf(r.c - a) - eps * a) / (fabsf(r.c - 1.f) + e * fabsf(dc) + ce);
     return r;
 }
-// of the sums: a lane's has at most 192 terms in a warp, and keeps what it rounds off in a team
+// of the sums: a lane's adds up at most HS_HEAVY batches in a warp, and keeps what it rounds off in a team
 constexpr float HS_EPS = 2e-6f;
 
 // The root of f near h (an FP32 root, K of Step32 there) in FP64, to its
