@@ -1377,17 +1377,18 @@ __device__ __forceinline__ void short_row(int64_t i, int64_t k0, int n, const in
     };
     double num = 0.0, den = 0.0;
     if (n > 0) {
-        int32_t q0[PB], q1[PB], j[PB];
+        // the first batches' loads of a kind together: a row waits for three in all
+        int32_t qa[PB], qb[PB], ja[PB], jb[PB], q0[PB], q1[PB], j[PB];
         Batch A, B;
-        pairs(0, q0);
-        pairs(PB, q1);
-        cells(q0, j);
-        values(q0, j, A);
-        cells(q1, j);
-        values(q1, j, B);
+        pairs(0, qa);
+        pairs(PB, qb);
         pairs(2 * PB, q0);
-        cells(q0, j);
         pairs(3 * PB, q1);
+        cells(qa, ja);
+        cells(qb, jb);
+        cells(q0, j);
+        values(qa, ja, A);
+        values(qb, jb, B);
         // before the batch at c: q0, j of the one at c + 2 PB, q1 of the next
         auto step = [&](int c, Batch &x) {
 #pragma unroll
@@ -1503,17 +1504,17 @@ __device__ __forceinline__ void long_rows(LongTile<MODE> &sh, int nrow, const in
             x.f[u] = WITH_F && q[u] >= 0 ? __ldg(f + j[u]) : 0.0;
         }
     };
-    int32_t q0[LR_PER], q1[LR_PER], j[LR_PER];
+    int32_t qa[LR_PER], qb[LR_PER], ja[LR_PER], jb[LR_PER], q0[LR_PER], q1[LR_PER], j[LR_PER];
     Part A, B;   // take turns, as in short_row
-    pairs(0, q0);
-    pairs(1, q1);
-    cells(q0, j);
-    values(q0, j, A);
-    cells(q1, j);
-    values(q1, j, B);
+    pairs(0, qa);
+    pairs(1, qb);
     pairs(2, q0);
-    cells(q0, j);
     pairs(3, q1);
+    cells(qa, ja);
+    cells(qb, jb);
+    cells(q0, j);
+    values(qa, ja, A);
+    values(qb, jb, B);
     // before tile c: q0, j of tile c + 2, q1 of the next
     auto step = [&](int c, Part &x) {
         const int s = c & 1;
@@ -1541,10 +1542,10 @@ __device__ __forceinline__ void long_rows(LongTile<MODE> &sh, int nrow, const in
 // ROW_FEW of those beyond ROW_VERY pairs, which then end sooner (24.04 M pairs
 // with rows of up to 3,781: 569 us with 32 of any length, 466 so; 16.4 M with rows
 // of up to 33,417: 2,834 and 2,451).
-// SHORT: the other blocks take the short ones, a row per thread.
+// SHORT: the other blocks take those of up to `longest` pairs, a row per thread.
 template <int MODE, bool LONG, bool SHORT>
 __global__ void __launch_bounds__(LONG ? ROW_THREADS : SHORT_THREADS, LONG ? 5 : 16)
-    k_rows(int64_t np, int nlongb, const int *__restrict__ nlong, const int32_t *__restrict__ rows,
+    k_rows(int64_t np, int nlongb, int longest, const int *__restrict__ nlong, const int32_t *__restrict__ rows,
            const int64_t *__restrict__ off, const int32_t *__restrict__ idx, const int32_t *__restrict__ pj,
            const double *__restrict__ w, const double *__restrict__ f, double *__restrict__ out0,
            double *__restrict__ out1)
@@ -1563,7 +1564,7 @@ __global__ void __launch_bounds__(LONG ? ROW_THREADS : SHORT_THREADS, LONG ? 5 :
         const int64_t i = (int64_t)(blockIdx.x - nlongb) * blockDim.x + threadIdx.x;
         if (i >= np) return;
         const int64_t k0 = off[i], n = off[i + 1] - k0;
-        if (n <= EM_ROW_LONG) short_row<MODE>(i, k0, (int)n, idx, pj, w, f, out0, out1);
+        if (n <= longest) short_row<MODE>(i, k0, (int)n, idx, pj, w, f, out0, out1);
     }
 }
 
@@ -1583,7 +1584,11 @@ __global__ void __launch_bounds__(LONG ? ROW_THREADS : SHORT_THREADS, LONG ? 5 :
 //   4.7 M, up to 2,504                             571  /  284   /  227
 //   24.0 M, up to 3,781                           1,667 /  782   /  466
 //   16.4 M, up to 33,417                         13,596 / 3,145  / 2,451
-constexpr int64_t ROWS_ONE_LAUNCH = 1 << 20;
+// Up to ROWS_ONE_LAUNCH pairs in rows of fewer than ROWS_THREAD on average, every
+// row by a thread: the long rows' blocks, registers and shared memory would be a
+// tenth to a quarter of such a call (500 to 50,000 pairs in rows of 1 to 5: 10.5
+// to 11.8 us, 12.6 to 13.6 with them).
+constexpr int64_t ROWS_ONE_LAUNCH = 1 << 20, ROWS_THREAD = 8;
 template <int MODE>
 static int launch_rows(em_ctx *ctx, const em_pairs *pr, const double *w, const double *f, double *out0, double *out1)
 {
@@ -1591,19 +1596,22 @@ static int launch_rows(em_ctx *ctx, const em_pairs *pr, const double *w, const d
     const int nlongb = pr->npairs > EM_ROW_LONG
                            ? (int)(pr->npairs / (EM_ROW_LONG + 1) / 32 + pr->npairs / ROW_VERY / ROW_FEW) + 2
                            : 0;
-    auto launch = [&](auto kernel, int threads, int nl, int64_t nshort) {
-        kernel<<<(unsigned)(nl + nshort), threads, 0, ctx->stream>>>(pr->np, nl, pr->nlong, pr->long_rows,
+    auto launch = [&](auto kernel, int threads, int nl, int64_t nshort, int longest) {
+        kernel<<<(unsigned)(nl + nshort), threads, 0, ctx->stream>>>(pr->np, nl, longest, pr->nlong, pr->long_rows,
                                                                      pr->part_pair_off, pr->part_pair_idx, pr->pair_j,
                                                                      w, f, out0, out1);
     };
     if (pr->npairs < ROWS_ONE_LAUNCH) {
-        launch(k_rows<MODE, true, true>, ROW_THREADS, nlongb, em_grid(pr->np, ROW_THREADS));
+        if (pr->npairs < ROWS_THREAD * pr->np)
+            launch(k_rows<MODE, false, true>, SHORT_THREADS, 0, em_grid(pr->np, SHORT_THREADS), INT_MAX);
+        else
+            launch(k_rows<MODE, true, true>, ROW_THREADS, nlongb, em_grid(pr->np, ROW_THREADS), EM_ROW_LONG);
         EM_LAUNCHED(ctx);
         return EM_OK;
     }
-    launch(k_rows<MODE, true, false>, ROW_THREADS, nlongb, 0);
+    launch(k_rows<MODE, true, false>, ROW_THREADS, nlongb, 0, 0);
     EM_LAUNCHED(ctx);
-    launch(k_rows<MODE, false, true>, SHORT_THREADS, 0, em_grid(pr->np, SHORT_THREADS));
+    launch(k_rows<MODE, false, true>, SHORT_THREADS, 0, em_grid(pr->np, SHORT_THREADS), EM_ROW_LONG);
     EM_LAUNCHED(ctx);
     return EM_OK;
 }

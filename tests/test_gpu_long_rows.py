@@ -23,6 +23,7 @@ ROWS = {
     "33 long, shuffled": list(np.random.default_rng(1).permutation([130] * 33 + [96] * 200 + [7] * 31)),
     "8 very long": [1500] * 8 + [100] * 31,
     "9 very long": [40] * 40 + [1500] * 9 + [100] * 33,
+    "a thread per row": [1] * 3000 + [0, 97, 2000, 2, 3, 1500],
     "every length": list(np.random.default_rng(2).permutation(np.arange(0, 700))),
     "two launches": EDGE * 20 + list(np.random.default_rng(3).integers(0, 1500, 1200)),
     "two launches, short": [6] * 200000,
